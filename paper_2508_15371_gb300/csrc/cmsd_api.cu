@@ -28,6 +28,7 @@ int cuda_fail(cudaError_t e) {
 std::mutex g_mu;
 std::map<int, int> g_sms;                                   // device -> SM count
 std::map<std::tuple<int, int, int, int, int>, int> g_occ;   // (dev, dtype, mode, variant, smem) -> blocks/SM
+std::map<std::tuple<int, int, int, int>, int> g_seq_res;     // (dev, dtype, CTAs, threads) -> resident clusters
 std::map<std::tuple<int, int, int>, int> g_occ_res;          // (dev, dtype, sampled) -> blocks/SM
 
 int device_sms(int* sms) {
@@ -231,6 +232,73 @@ void fill_sizes(StreamArgs& a, int B, int K, int V) {
   a.soft_norm = (float)(1.0 / (1.0 - 1.0 / (double)V));
 }
 
+// Clusters of seq_kernel that can be resident on the current device (cached).
+int seq_resident(int dtype, int nc, int threads) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const auto key = std::make_tuple(dev, dtype, nc, threads);
+  std::lock_guard<std::mutex> lk(g_mu);
+  auto it = g_seq_res.find(key);
+  if (it == g_seq_res.end()) {
+    const int n = dtype == CMSD_F32 ? seq_clusters_f32(nc, threads) : seq_clusters_bf16(nc, threads);
+    it = g_seq_res.emplace(key, n).first;
+  }
+  return it->second;
+}
+
+// Which kernel takes a call: the one-launch pass with *nc CTAs of *threads
+// threads per sequence (true), or the streaming kernel and its second pass.
+//
+// Both times are estimated, in microseconds, from what was measured on a
+// GB300 over K = 1..16, V = 32000..152064, B = 1..600 (bf16; f32 alike):
+//   streaming kernel   9 + bytes / 6900 MB/s, and with a second launch 7.5
+//     more (14 for the bonus race over every group) and 0.045 (0.09) per
+//     sequence beyond 64;
+//   one launch         5, a draw 4.5, and the time of a sequence's bytes
+//     through its CTAs (a CTA of 256 threads: 27 KB a microsecond under the
+//     PAPER rule, 21 with the target's exponentials or the drafter alone, 30
+//     for the target alone; one of 512 twice that), times the waves when not
+//     every cluster is resident (3.5 more each), and no less than the bytes at
+//     6900 MB/s.
+// Ragged windows are unknown here: half full on average, and the longest
+// decides the one-launch pass, since a sequence keeps to its cluster.
+bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int* nc, int* threads) {
+  if (a.K > kPackedMaxK || (second && sampled && !seq_draw_fits(dtype, a.V))) return false;
+  const double kb = (double)a.K * a.V * (dtype == CMSD_F32 ? 4 : 2) * (mode == kModeFused ? 2 : 1) * 1e-3;
+  const double stream = a.B * kb * (a.k_row ? 0.5 : 1.0) / 6900;
+  double flat = 9 + stream;
+  if (second) {
+    flat += a.bonus ? 14 : 7.5;
+    if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 0.09 : 0.045);
+  }
+  const double rate = mode == kModeVerify ? 30 : (mode == kModeFused && !sampled ? 27 : 21);
+  const double fixed = 5 + (second ? 4.5 : 0);
+  static const int sizes[] = {1, 2, 4, 5, 8, 16};
+  double best = 0.97 * flat;               // (a near tie stays with the streaming kernel)
+  *nc = 0;
+  for (int th = 256; th <= 512; th *= 2) {
+    for (int n : sizes) {
+      // at least two 16-byte vectors per lane and piece, or more CTAs gain nothing
+      if (n > 1 && kb * 1e3 < (double)n * (th / 32) * 1024 * (mode == kModeFused ? 2 : 1)) break;
+      const double part = kb / n / (rate * (th / 256));
+      if (fixed + part >= best) continue;
+      const int res = seq_resident(dtype, n, th);
+      if (res < 1) continue;
+      // (clusters of 4 and more were not all placed at once near the limit)
+      const int fit = n >= 4 ? (res * 9 + 9) / 10 : res;
+      const int waves = (a.B + fit - 1) / fit;
+      const double t = fixed + (th == 512 ? 0.7 : 0.0) + 3.5 * (waves - 1) +
+                       (waves * part > stream ? waves * part : stream);
+      if (t < best) {
+        best = t;
+        *nc = n;
+        *threads = th;
+      }
+    }
+  }
+  return *nc > 0;
+}
+
 int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws_bytes,
            cudaStream_t s) {
   int wmax = 0;
@@ -243,6 +311,16 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   a.Kt = bonus ? a.K + 1 : a.K;
   a.Ko = bonus ? a.K + 1 : a.K;
   const bool second = mode != kModeConf && (sampled || bonus);
+  int nc = 0, threads = 0;
+  if (choose_seq(dtype, mode, sampled, second, a, &nc, &threads)) {
+    prof_record(0, s);
+    const cudaError_t e = dtype == CMSD_F32 ? launch_seq_f32(mode, sampled, second, a, nc, threads, s)
+                                            : launch_seq_bf16(mode, sampled, second, a, nc, threads, s);
+    if (e != cudaSuccess) return cuda_fail(e);
+    prof_record(1, s);
+    prof_record(2, s);
+    return CMSD_OK;
+  }
   const size_t smem = stream_smem_bytes(a.B, a.k_row != nullptr);
   int grid = 0;
   rc = stream_grid(dtype, mode, sampled, second, smem, &grid);
@@ -260,6 +338,7 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
     nclu = a.B < 2 * sms ? a.B : 2 * sms;
   }
   a.nwarps = grid * kStreamWarps;
+  if (!a.k_row) a.split = StreamSplit(a.B * a.K, a.V, dtype == CMSD_F32 ? 4 : 8, a.nwarps, stream_min_len(a.V));
   a.rec_by_seq = bound ? 1 : 0;
   prof_record(0, s);
   cudaError_t e = dtype == CMSD_F32 ? launch_stream_f32(mode, sampled, second, a, grid, smem, s)

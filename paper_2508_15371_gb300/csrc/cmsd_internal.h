@@ -78,6 +78,89 @@ struct Workspace {
   UnitResult* rpart;              // [B + warps]
 };
 
+// Fewest logits per warp slice: small problems are cut finely (latency), large
+// rows into at most about 128 pieces (each piece costs one partial to merge).
+// Measured on one-call latencies: 1024 beat 2048 by 2-3 us at B=1 K=4
+// V=32000, and 512 or 256 gained nothing more.
+__host__ __device__ inline int64_t stream_min_len(int V) {
+  const int64_t a = (int64_t)V / 128 + 64;
+  return a > 1024 ? a : 1024;
+}
+// a / b for 0 <= a, 0 < b, in 32-bit arithmetic when both fit.
+__host__ __device__ inline int64_t div_nn(int64_t a, int64_t b) {
+  if (a <= 0x7FFFFFFF && b <= 0x7FFFFFFF) return (int64_t)((uint32_t)a / (uint32_t)b);
+  return a / b;
+}
+
+// How the present-row stream (R rows of V logits, N = R*V elements) is cut
+// into warp slices.  When there are at least as many warps as rows, each row
+// is cut into wpr pieces of one warp each (no slice crosses a row end, so
+// every warp streams one segment); otherwise the stream is cut into W equal
+// runs of 128-byte lines.  Slices start on multiples of 128 bytes from the
+// row (or stream) start, so that a warp's 512-byte loads cover whole 32-byte
+// sectors when the rows themselves are 128-byte aligned; a 16-byte offset
+// would make every load touch one sector more (the last slice ends at N).
+// Formed on the host for full windows: its 64-bit divisions kept a slice's
+// first loads waiting (0.4 us of a 11.2 us call at B=64 K=1 V=128256).
+constexpr int kLineVecs = 8;   // 16-byte vectors per 128-byte line
+struct StreamSplit {
+  StreamSplit() = default;
+  int64_t N;
+  int W;          // warps with work
+  int V, VEC;
+  int wpr;        // > 0: row-aligned split with wpr warps per row
+  int qv, rv;     // row-aligned: V / wpr, V % wpr
+  int64_t q;      // flat: vectors per warp (the first rem warps one more)
+  int rem;
+  __host__ __device__ StreamSplit(int R, int V_, int vec, int nwarps, int64_t min_len) {
+    V = V_;
+    VEC = vec;
+    N = (int64_t)R * V;
+    int64_t want = N / min_len;
+    if (want < 1) want = 1;
+    const int Wmax = (int)(want < nwarps ? want : nwarps);
+    int p = nwarps / R;                              // pieces per row that fit
+    const int64_t pm = (int64_t)V / min_len;
+    const int pmax = pm > 0 ? (int)pm : 1;
+    if (p > pmax) p = pmax;
+    if (p >= 1 && (int64_t)p * R * 8 >= (int64_t)Wmax * 7) {   // uses at least 7/8 of the warps
+      wpr = p;
+      W = p * R;
+      qv = V / p;
+      rv = V - qv * p;
+      q = 0;
+      rem = 0;
+    } else {
+      wpr = 0;
+      W = Wmax;
+      qv = rv = 0;
+      const int64_t nv = N / (VEC * kLineVecs);
+      q = div_nn(nv, W);
+      rem = (int)(nv - q * W);
+    }
+  }
+  __host__ __device__ int64_t start(int w) const {
+    if (w >= W) return N;
+    if (wpr > 0) {
+      const int row = w / wpr, k = w - row * wpr;
+      const int off = k * qv + (k < rv ? k : rv);
+      return (int64_t)row * V + (off & ~(VEC * kLineVecs - 1));
+    }
+    return ((int64_t)w * q + (w < rem ? w : rem)) * VEC * kLineVecs;
+  }
+  // warps holding the first and the last element of row ar
+  __host__ __device__ int first_warp(int ar) const { return wpr > 0 ? ar * wpr : owner_flat((int64_t)ar * V); }
+  __host__ __device__ int last_warp(int ar) const {
+    return wpr > 0 ? ar * wpr + wpr - 1 : owner_flat((int64_t)ar * V + V - 1);
+  }
+  __host__ __device__ int owner_flat(int64_t e) const {
+    const int64_t ev = e / (VEC * kLineVecs);
+    const int64_t big = (q + 1) * rem;
+    const int w = ev < big ? (int)div_nn(ev, q + 1) : rem + (int)div_nn(ev - big, q);
+    return w < W ? w : W - 1;
+  }
+};
+
 struct StreamArgs {
   const void* draft;
   const void* target;
@@ -109,6 +192,7 @@ struct StreamArgs {
   unsigned char* accept;
   Workspace ws;
   int nwarps;             // warps launched
+  StreamSplit split;      // full windows: the cut of the B*K rows
   int rec_by_seq;         // 1: second-pass records at each sequence's own slot rec[b], every sequence
                           // writing one (the bounded residual draw); 0: a compacted queue (rec_count)
 };
@@ -119,6 +203,16 @@ cudaError_t launch_stream_f32(int mode, bool sampled, bool second, const StreamA
                               size_t smem, cudaStream_t s);
 cudaError_t launch_stream_bf16(int mode, bool sampled, bool second, const StreamArgs& a, int grid,
                                size_t smem, cudaStream_t s);
+// The pass in one launch, a cluster of nc CTAs of `threads` (256 or 512)
+// threads per sequence (cmsd_seq_impl.cuh).
+cudaError_t launch_seq_f32(int mode, bool sampled, bool second, const StreamArgs& a, int nc, int threads,
+                            cudaStream_t s);
+cudaError_t launch_seq_bf16(int mode, bool sampled, bool second, const StreamArgs& a, int nc, int threads,
+                            cudaStream_t s);
+// Clusters of nc such CTAs that can be resident on the current device (0: none).
+int seq_clusters_f32(int nc, int threads);
+int seq_clusters_bf16(int nc, int threads);
+bool seq_draw_fits(int dtype, int V);
 cudaError_t launch_resample_f32(bool sampled, const StreamArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_resample_bf16(bool sampled, const StreamArgs& a, int grid, cudaStream_t s);
 // The residual draw by group bounds (sampled rule, no bonus row): clusters

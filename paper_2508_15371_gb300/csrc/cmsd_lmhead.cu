@@ -36,38 +36,6 @@ namespace {
 constexpr int kMergeRowsPerCta = 8;                 // one warp per row
 
 // ---- shared-memory barriers and 2D TMA loads -----------------------------------
-__device__ __forceinline__ unsigned long long lh_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-constexpr unsigned long long kLhWaitLimitNs = 1000000000ull;   // the launch takes well under a millisecond
-__device__ __forceinline__ void mbar_init(uint32_t bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-// arrive once and expect tx bytes of asynchronous copies in this phase
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t tx) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(tx) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// true once the phase with this parity has completed, false after kLhWaitLimitNs
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = lh_ns();
-  for (;;) {
-    for (int k = 0; k < 32; ++k)
-      if (mbar_try_wait(bar, parity)) return true;
-    if (lh_ns() - t0 > kLhWaitLimitNs) return false;
-  }
-}
 // box of the 2D tensor map at (x, y) (x: innermost, in elements) into shared
 // memory at dst, completing `bar` by transaction count
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -406,9 +374,7 @@ __global__ void __launch_bounds__(32 * kMergeRowsPerCta) lmhead_merge_kernel(con
       if (k0 + 32 * j < h.nct) fold_d(m, DRed{x0[j].x, x0[j].y, x0[j].z, x0[j].w, __float_as_int(x1[j].x)});
   }
   const DRed dr = reduce_d(m);
-  bool acc;
-  unsigned long long cfx;
-  row_results<float, kModeConf, false>(a, r, 0, 0, dr, tred_empty(), 0.f, 0.f, lane, acc, cfx);
+  row_results<kModeConf, false>(a, r, 0, 0, dr, tred_empty(), 0.f, 0.f, 0.f, 0.f, lane);
 }
 
 }  // namespace

@@ -172,11 +172,12 @@ __device__ __forceinline__ void t_reref(TLane& t, float mx) {
   t.negrL = dup2(-nrL);
 }
 
-// --- drafter: one element at a time (segment heads/tails) --------------------
+// --- drafter: one element at a time (segment heads/tails, in any order with
+// the lane's vectors) ----------------------------------------------------------
 __device__ __forceinline__ void d_scalar(DLane& d, float z, int v) {
   d.f2 = fmaxf(d.f2, fminf(d.f1, z));
   d.f1 = fmaxf(d.f1, z);
-  if (z > d.m) { d.pos = v; d.posw = 1; }
+  if (z > d.m || (z == d.m && v < d.pos)) { d.pos = v; d.posw = 1; }
   d.m = fmaxf(d.m, z);
   const float me = d_mexp(d);
   if (me > d.ref + kRefSlack) d_reref(d, me);
@@ -237,7 +238,7 @@ __device__ __forceinline__ void d_vexp(const DLane& d, float4 q, u64& ss, u64& t
 // --- target -----------------------------------------------------------------------
 template <bool SAMPLED>
 __device__ __forceinline__ void t_scalar(TLane& t, float z, int v, float c, int beta) {
-  if (z > t.M) { t.pos = v; t.posw = 1; }
+  if (z > t.M || (z == t.M && v < t.pos)) { t.pos = v; t.posw = 1; }
   t.M = fmaxf(t.M, z);
   if (t.cnt < beta && z > c) ++t.cnt;
   if (SAMPLED) {
@@ -338,31 +339,25 @@ __device__ __forceinline__ int first_in_vec(uint4 q, float m, bool clamp) {
 // warp reductions (results identical in every lane)
 // ---------------------------------------------------------------------------
 
+// Maxima and minima are one redux.sync (floats: the sm_100 family's f32
+// form), sums a butterfly: its lanes add the same pairs in the same tree, so
+// every lane gets the same bits.
 __device__ __forceinline__ float warp_max(float x) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) x = fmaxf(x, __shfl_xor_sync(kFull, x, o));
-  return x;
+  float y;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+  return y;
 }
 __device__ __forceinline__ float warp_min(float x) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) x = fminf(x, __shfl_xor_sync(kFull, x, o));
-  return x;
+  float y;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+  return y;
 }
-__device__ __forceinline__ int warp_min_i(int x) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) x = min(x, __shfl_xor_sync(kFull, x, o));
-  return x;
-}
-__device__ __forceinline__ int warp_sum_i(int x) {
+__device__ __forceinline__ int warp_min_i(int x) { return __reduce_min_sync(kFull, x); }
+__device__ __forceinline__ int warp_sum_i(int x) { return __reduce_add_sync(kFull, x); }
+__device__ __forceinline__ float warp_sum_f(float x) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
   return x;
-}
-// Sum with a fixed tree, broadcast from lane 0 (same bits in every lane).
-__device__ __forceinline__ float warp_sum_f(float x) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-  return __shfl_sync(kFull, x, 0);
 }
 
 struct DRed { float m, s, t2, top2; int idx; };
@@ -431,20 +426,6 @@ __device__ __forceinline__ void fold_t(TRed& a, const TRed& b) {
 // work split
 // ---------------------------------------------------------------------------
 
-// Fewest logits per warp slice: small problems are cut finely (latency), large
-// rows into at most about 128 pieces (each piece costs one partial to merge).
-// Measured on one-call latencies: 1024 beat 2048 by 2-3 us at B=1 K=4
-// V=32000, and 512 or 256 gained nothing more.
-__device__ __forceinline__ int64_t stream_min_len(int V) {
-  const int64_t a = (int64_t)V / 128 + 64;
-  return a > 1024 ? a : 1024;
-}
-// a / b for 0 <= a, 0 < b, in 32-bit arithmetic when both fit.
-__device__ __forceinline__ int64_t div_nn(int64_t a, int64_t b) {
-  if (a <= 0x7FFFFFFF && b <= 0x7FFFFFFF) return (int64_t)((uint32_t)a / (uint32_t)b);
-  return a / b;
-}
-
 // N units over W warps, contiguous and in order: the first rem warps get q+1.
 struct EvenSplit {
   int64_t q;
@@ -457,72 +438,6 @@ struct EvenSplit {
   __device__ int owner(int64_t u) const {
     const int64_t big = (q + 1) * rem;
     return u < big ? (int)div_nn(u, q + 1) : rem + (int)div_nn(u - big, q);
-  }
-};
-
-// How the present-row stream (R rows of V logits, N = R*V elements) is cut
-// into warp slices.  When there are at least as many warps as rows, each row
-// is cut into wpr pieces of one warp each (no slice crosses a row end, so
-// every warp streams one segment); otherwise the stream is cut into W equal
-// runs of 128-byte lines.  Slices start on multiples of 128 bytes from the
-// row (or stream) start, so that a warp's 512-byte loads cover whole 32-byte
-// sectors when the rows themselves are 128-byte aligned; a 16-byte offset
-// would make every load touch one sector more (the last slice ends at N).
-constexpr int kLineVecs = 8;   // 16-byte vectors per 128-byte line
-struct StreamSplit {
-  int64_t N;
-  int W;          // warps with work
-  int V, VEC;
-  int wpr;        // > 0: row-aligned split with wpr warps per row
-  int qv, rv;     // row-aligned: V / wpr, V % wpr
-  int64_t q;      // flat: vectors per warp (the first rem warps one more)
-  int rem;
-  __device__ StreamSplit(int R, int V_, int vec, int nwarps, int64_t min_len) {
-    V = V_;
-    VEC = vec;
-    N = (int64_t)R * V;
-    int64_t want = N / min_len;
-    if (want < 1) want = 1;
-    const int Wmax = (int)(want < nwarps ? want : nwarps);
-    int p = nwarps / R;                              // pieces per row that fit
-    const int64_t pm = (int64_t)V / min_len;
-    const int pmax = pm > 0 ? (int)pm : 1;
-    if (p > pmax) p = pmax;
-    if (p >= 1 && (int64_t)p * R * 8 >= (int64_t)Wmax * 7) {   // uses at least 7/8 of the warps
-      wpr = p;
-      W = p * R;
-      qv = V / p;
-      rv = V - qv * p;
-      q = 0;
-      rem = 0;
-    } else {
-      wpr = 0;
-      W = Wmax;
-      qv = rv = 0;
-      const int64_t nv = N / (VEC * kLineVecs);
-      q = div_nn(nv, W);
-      rem = (int)(nv - q * W);
-    }
-  }
-  __device__ int64_t start(int w) const {
-    if (w >= W) return N;
-    if (wpr > 0) {
-      const int row = w / wpr, k = w - row * wpr;
-      const int off = k * qv + (k < rv ? k : rv);
-      return (int64_t)row * V + (off & ~(VEC * kLineVecs - 1));
-    }
-    return ((int64_t)w * q + (w < rem ? w : rem)) * VEC * kLineVecs;
-  }
-  // warps holding the first and the last element of row ar
-  __device__ int first_warp(int ar) const { return wpr > 0 ? ar * wpr : owner_flat((int64_t)ar * V); }
-  __device__ int last_warp(int ar) const {
-    return wpr > 0 ? ar * wpr + wpr - 1 : owner_flat((int64_t)ar * V + V - 1);
-  }
-  __device__ int owner_flat(int64_t e) const {
-    const int64_t ev = e / (VEC * kLineVecs);
-    const int64_t big = (q + 1) * rem;
-    const int w = ev < big ? (int)div_nn(ev, q + 1) : rem + (int)div_nn(ev - big, q);
-    return w < W ? w : W - 1;
   }
 };
 
@@ -557,23 +472,35 @@ struct Seg {
   int v0, v1, va, vb;
 };
 
+// The part [v0, min(v0 + len_max, V)) of the row at `row` as a segment.
+template <typename T>
+__device__ __forceinline__ Seg seg_geom(const T* row, int v0, int V, int64_t len_max) {
+  constexpr int VEC = Elem<T>::kVec;
+  Seg s;
+  s.ar = s.b = s.i = s.r = 0;
+  s.v0 = v0;
+  const int len = (int)min((int64_t)(V - v0), len_max);
+  s.v1 = v0 + len;
+  const int mis = (int)(((uintptr_t)(row + v0) & 15) / sizeof(T));
+  const int head = mis ? min(VEC - mis, len) : 0;
+  s.va = v0 + head;
+  s.vb = s.va + ((s.v1 - s.va) / VEC) * VEC;
+  return s;
+}
+
 template <typename T>
 __device__ __forceinline__ Seg make_seg(const StreamArgs& a, const int* pref, int64_t e, int64_t e_end,
                                         const void* base, bool base_is_target) {
-  constexpr int VEC = Elem<T>::kVec;
-  Seg s;
-  s.ar = (int)(e / a.V);
-  s.v0 = (int)(e - (int64_t)s.ar * a.V);
-  const int len = (int)min((int64_t)(a.V - s.v0), e_end - e);
-  s.v1 = s.v0 + len;
-  map_row(a, pref, s.ar, s.b, s.i);
-  s.r = s.b * a.K + s.i;
-  const size_t row = base_is_target ? (size_t)s.b * a.Kt + s.i : (size_t)s.r;
-  const uintptr_t addr = (uintptr_t)((const T*)base + row * (size_t)a.V + s.v0);
-  const int mis = (int)((addr & 15) / sizeof(T));
-  const int head = mis ? min(VEC - mis, len) : 0;
-  s.va = s.v0 + head;
-  s.vb = s.va + ((s.v1 - s.va) / VEC) * VEC;
+  const int ar = (int)div_nn(e, a.V);
+  int b, i;
+  map_row(a, pref, ar, b, i);
+  const int r = b * a.K + i;
+  const size_t row = base_is_target ? (size_t)b * a.Kt + i : (size_t)r;
+  Seg s = seg_geom<T>((const T*)base + row * (size_t)a.V, (int)(e - (int64_t)ar * a.V), a.V, e_end - e);
+  s.ar = ar;
+  s.b = b;
+  s.i = i;
+  s.r = r;
   return s;
 }
 
@@ -753,23 +680,30 @@ __device__ __forceinline__ void dot3_exact(float l0, float c0, float l1, float c
 
 constexpr float kFixedScale = 68719476736.0f;   // 2^36
 
+// A row's decision and what its sequence and the residual draw need of it.
+struct RowOut {
+  bool acc;
+  unsigned long long cfx;   // C in fixed point
+  float2 ds, ts;            // sampled rule: drafter and target (max * log2e, sum)
+};
+
 // Called by the whole warp (statistics identical in every lane): the row's
 // exponentials and reciprocals are spread one per lane, so each costs one
-// instruction sequence instead of a chain on one lane.  Lane 0 writes.
-template <typename T, int MODE, bool SAMPLED>
-__device__ __forceinline__ void row_results(const StreamArgs& a, int r, int b, int i, const DRed& d, const TRed& t,
-                                         float c_tgt, float zd, int lane, bool& acc_out,
-                                         unsigned long long& cfx_out) {
+// instruction sequence instead of a chain on one lane.  Lane 0 writes the
+// outputs.  lse_in, conf_in: the caller's signals (verify mode).
+template <int MODE, bool SAMPLED>
+__device__ __forceinline__ RowOut row_results(const StreamArgs& a, int r, int b, int i, const DRed& d, const TRed& t,
+                                              float c_tgt, float zd, float lse_in, float conf_in, int lane) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
-  const Workspace& W = a.ws;
+  RowOut o;
+  o.ds = o.ts = make_float2(0.f, 1.f);
   const float MLd0 = HAS_D ? mlog2e(d.m) : 0.f;
   const float MLt = HAS_T ? mlog2e(t.m) : 0.f;
   const float res_m = HAS_D ? fmaf(d.m, kLog2e, -MLd0) : 0.f;   // exact rounding residuals of m log2e
   const float res_t = HAS_T ? fmaf(t.m, kLog2e, -MLt) : 0.f;
   const bool has2 = HAS_D && d.top2 > neg_clamp();
   const float margin = has2 ? d.m - d.top2 : pos_inf();
-  const float lse_in = (MODE == kModeVerify && SAMPLED) ? __ldg(a.lse_in + r) : 0.f;
   // one exponential per lane
   float x = 0.f;
   if (lane == 0) x = has2 ? d.top2 - d.m : -pos_inf();        // e^(z(2) - m)
@@ -819,7 +753,7 @@ __device__ __forceinline__ void row_results(const StreamArgs& a, int r, int b, i
       if (a.lse) a.lse[r] = d.m + kLn2 * (l2s - res_m);
     }
   } else {
-    C = __ldg(a.conf_in + r);
+    C = conf_in;
     cfx = __float2ull_rn(fminf(1.0f, fmaxf(0.0f, C)) * kFixedScale);
   }
   bool acc = false;
@@ -837,24 +771,18 @@ __device__ __forceinline__ void row_results(const StreamArgs& a, int r, int b, i
       const U4 w = philox4x32_10(U4{0u, (uint32_t)b, (uint32_t)i, iter_word(a.iteration, kPurposeAccept)},
                                  seed_lo(a.seed), seed_hi(a.seed));
       acc = rank_ok && (word_to_unit(w.x) * q < expf(tau) * p);
-      if (lane == 0) {
-        float MLd = MLd0, Sd = d.s;
-        if (MODE == kModeVerify) {            // q_v = 2^(z log2e - MLd) / Sd with MLd = lse log2e
-          MLd = lse_in * kLog2e;
-          Sd = exp2f(fmaf(lse_in, kLog2e, -MLd));
-        }
-        W.row_dstat[r] = make_float2(MLd, Sd);
-        W.row_tstat[r] = make_float2(MLt, t.s);
+      float MLd = MLd0, Sd = d.s;
+      if (MODE == kModeVerify) {              // q_v = 2^(z log2e - MLd) / Sd with MLd = lse log2e
+        MLd = lse_in * kLog2e;
+        Sd = exp2f(fmaf(lse_in, kLog2e, -MLd));
       }
-    }
-    if (lane == 0) {
-      W.row_acc[r] = acc ? 1 : 0;
-      W.row_targmax[r] = t.idx;
+      o.ds = make_float2(MLd, Sd);
+      o.ts = make_float2(MLt, t.s);
     }
   }
-  if (lane == 0) W.row_conf[r] = cfx;
-  acc_out = acc;
-  cfx_out = cfx;
+  o.acc = acc;
+  o.cfx = cfx;
+  return o;
 }
 
 // ---------------------------------------------------------------------------
@@ -869,15 +797,12 @@ struct SegState {
   float zd;         // drafter logit at the drafted token (SAMPLED rule)
 };
 
-// End of a segment (row ar, position r = b*K + i, len logits): warp-reduce,
-// publish the partial, and merge the row / run the sequence epilogue if this
-// warp completes them.
-template <typename T, int MODE, bool SAMPLED, bool PH2>
-__device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int b, int i, int len,
-                           const StreamSplit& sp, int w, int lane, const T* dp, const T* tp) {
+// The warp's statistics of the segment its lanes have reduced, in every lane.
+template <typename T, int MODE, bool SAMPLED>
+__device__ __forceinline__ void seg_reduce(const SegState& ss, bool want_didx, bool want_tidx, const T* dp, const T* tp,
+                                           DRed& dr, TRed& tr) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
-  const Workspace& W = a.ws;
   // The exact index of a lane's maximum inside its first 16-byte vector needs
   // that vector again.  Under the sampled rule only the lanes holding the
   // segment maximum request it (one sector each, usually one lane; this saved
@@ -885,14 +810,10 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
   // PAPER rule every lane requests its vector before the warp reductions, so
   // the loads overlap the shuffles: there the kernel's tail is this latency,
   // and the early requests measured 3 us faster than the late ones.
+  // Without a wanted index a lane's vector start stands in (distinct per lane
+  // and ordered like the index, so the merges still tell the maximum's lane
+  // from a duplicate of its value) and nothing is re-read.
   const float me = HAS_D ? d_mexp(ss.d) : 0.f;
-  // Under the sampled rule the exact indices feed only the drafter's argmax
-  // output and resample_kernel's empty-residual fallback (the bounded draw
-  // finds that argmax itself): without them a lane's vector start stands in
-  // (distinct per lane and ordered like the index, so the merges still tell
-  // the maximum's lane from a duplicate of its value) and nothing is re-read.
-  const bool want_didx = !SAMPLED || a.argmax != nullptr;
-  const bool want_tidx = !SAMPLED || !a.rec_by_seq;
   uint4 dq = make_uint4(0, 0, 0, 0), tq = make_uint4(0, 0, 0, 0);
   if (!SAMPLED) {
     if (HAS_D && ss.d.posw > 1) dq = __ldcg(reinterpret_cast<const uint4*>(dp + ss.d.pos));
@@ -905,8 +826,8 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
     if (want_didx && dhit && ss.d.posw > 1) dq = __ldcg(reinterpret_cast<const uint4*>(dp + ss.d.pos));
     if (want_tidx && thit && ss.t.posw > 1) tq = __ldcg(reinterpret_cast<const uint4*>(tp + ss.t.pos));
   }
-  DRed dr = dred_empty();
-  TRed tr = tred_empty();
+  dr = dred_empty();
+  tr = tred_empty();
   if (HAS_D) {
     const DLane& d = ss.d;
     float top1 = d.f1, top2 = d.f2;
@@ -928,6 +849,23 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
     if (thit) idx = (want_tidx && t.posw > 1) ? t.pos + first_in_vec<T>(tq, t.M, false) : t.pos;
     tr = reduce_t(TRed{t.M, SAMPLED ? t_final(t) : 0.f, idx, t.cnt});
   }
+}
+
+// End of a segment (row ar, position r = b*K + i, len logits): warp-reduce,
+// publish the partial, and merge the row / run the sequence epilogue if this
+// warp completes them.
+template <typename T, int MODE, bool SAMPLED, bool PH2>
+__device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int b, int i, int len,
+                           const StreamSplit& sp, int w, int lane, const T* dp, const T* tp) {
+  constexpr bool HAS_D = MODE != kModeVerify;
+  constexpr bool HAS_T = MODE != kModeConf;
+  const Workspace& W = a.ws;
+  // Under the sampled rule the exact indices feed only the drafter's argmax
+  // output and resample_kernel's empty-residual fallback (the bounded draw
+  // finds that argmax itself).
+  DRed dr;
+  TRed tr;
+  seg_reduce<T, MODE, SAMPLED>(ss, !SAMPLED || a.argmax != nullptr, !SAMPLED || !a.rec_by_seq, dp, tp, dr, tr);
   // lane 0 stores the partial and counts it with a release; the warp that
   // completes the row sees every other slice's partial through the acquire
   // of its own count (extended to the other lanes by __syncwarp)
@@ -961,30 +899,34 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
   }
   if (HAS_D) dr = reduce_d(dm);
   if (HAS_T) tr = reduce_t(tm);
-  if (packed) {
-    unsigned long long word = 0ull;
-    bool acc;
-    unsigned long long cfx;
-    row_results<T, MODE, SAMPLED>(a, r, b, i, dr, tr, ss.c, ss.zd, lane, acc, cfx);
-    if (lane == 0) {
-      W.row_done[r] = 0;
-      const unsigned long long mine = 1ull | ((unsigned long long)(acc ? 1u : 0u) << (6 + i)) | (cfx << 22);
-      word = atom_add_acq_rel_u64(W.seq_word + b, mine) + mine;
+  const float lse_in = (MODE == kModeVerify && SAMPLED) ? __ldg(a.lse_in + r) : 0.f;
+  const float conf_in = MODE == kModeVerify ? __ldg(a.conf_in + r) : 0.f;
+  const RowOut o = row_results<MODE, SAMPLED>(a, r, b, i, dr, tr, ss.c, ss.zd, lse_in, conf_in, lane);
+  unsigned long long word = 0ull;
+  int sold = 0;
+  if (lane == 0) {
+    if (HAS_T && SAMPLED) {
+      W.row_dstat[r] = o.ds;
+      W.row_tstat[r] = o.ts;
     }
+    if (HAS_T) W.row_targmax[r] = tr.idx;
+    W.row_done[r] = 0;
+    if (packed) {
+      const unsigned long long mine = 1ull | ((unsigned long long)(o.acc ? 1u : 0u) << (6 + i)) | (o.cfx << 22);
+      word = atom_add_acq_rel_u64(W.seq_word + b, mine) + mine;
+    } else {
+      if (HAS_T) W.row_acc[r] = o.acc ? 1 : 0;
+      W.row_conf[r] = o.cfx;
+      sold = atom_add_acq_rel(W.seq_done + b, 1);
+    }
+  }
+  if (packed) {
     word = __shfl_sync(kFull, word, 0);
     if ((int)(word & 63ull) == kb) {
       __syncwarp();
       seq_epilogue_packed<MODE, SAMPLED, PH2>(a, b, kb, word, tok, lane);
     }
   } else {
-    int sold = 0;
-    bool acc;
-    unsigned long long cfx;
-    row_results<T, MODE, SAMPLED>(a, r, b, i, dr, tr, ss.c, ss.zd, lane, acc, cfx);
-    if (lane == 0) {
-      W.row_done[r] = 0;
-      sold = atom_add_acq_rel(W.seq_done + b, 1);
-    }
     sold = __shfl_sync(kFull, sold, 0);
     if (sold + 1 == kb) {
       __syncwarp();
@@ -1000,21 +942,20 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
 #ifndef CMSD_UNROLL
 #define CMSD_UNROLL 2
 #endif
-template <typename T>
+template <typename T, int U>
 struct Pipe {
-  uint4 d[CMSD_UNROLL], t[CMSD_UNROLL];   // the stage in flight
+  uint4 d[U], t[U];                       // the stage in flight
   const uint4* gd;
   const uint4* gt;
   int nt, nst;                            // this lane's vectors; warp-uniform stages
 };
 
 // issue the loads of stage 0
-template <typename T, int MODE>
-__device__ __forceinline__ void pipe_start(Pipe<T>& p, const T* dp, const T* tp, int va, int vb, int lane) {
+template <typename T, int MODE, int U>
+__device__ __forceinline__ void pipe_start(Pipe<T, U>& p, const T* dp, const T* tp, int va, int vb, int lane) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
   constexpr int VEC = Elem<T>::kVec;
-  constexpr int U = CMSD_UNROLL;
   const int nvec = (vb - va) / VEC;
   p.nt = nvec > lane ? (nvec - lane + 31) / 32 : 0;
   p.nst = (nvec + 32 * U - 1) / (32 * U);
@@ -1029,12 +970,12 @@ __device__ __forceinline__ void pipe_start(Pipe<T>& p, const T* dp, const T* tp,
   }
 }
 
-template <typename T, int MODE, bool SAMPLED>
-__device__ __forceinline__ void pipe_run(Pipe<T>& p, SegState& ss, int va, int beta, int lane) {
+template <typename T, int MODE, bool SAMPLED, int U>
+__device__ __forceinline__ void pipe_run(Pipe<T, U>& p, SegState& ss, int va, int beta, int lane) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
   constexpr int VEC = Elem<T>::kVec;
-  constexpr int U = CMSD_UNROLL;
+#pragma unroll 1
   for (int s = 0; s < p.nst; ++s) {
     uint4 nd[U], nx[U];
     const int t1 = (s + 1) * U;
@@ -1101,7 +1042,7 @@ __device__ void walk_slice(const StreamArgs& a, const int* s_pref, int64_t e_beg
     e0 += len;
     const T* dp = (const T*)a.draft + (size_t)sg.r * (size_t)a.V;
     const T* tp = HAS_T ? (const T*)a.target + ((size_t)sg.b * a.Kt + sg.i) * (size_t)a.V : nullptr;
-    Pipe<T> pp;
+    Pipe<T, CMSD_UNROLL> pp;
     pipe_start<T, MODE>(pp, dp, tp, sg.va, sg.vb, lane);
     float c = 0.f, zd = 0.f;
     if (HAS_T) {
@@ -1198,13 +1139,34 @@ __device__ __forceinline__ float resid_vec(uint4 qt, uint4 qd, const RowStat& s)
 }
 
 // 16 bytes of logits at entry v of one row: one vector load when the vector is
-// aligned and inside the row, else element loads with entries past the row
-// end read as -inf (p = q = 0, so r = 0).
+// aligned and inside the row; off 16-byte boundaries the two aligned vectors
+// that hold it, shifted together, while both lie inside the row (the lower one
+// starts at most 15 bytes before entry v, and no row starts before its
+// tensor's 16-byte aligned base); at the row's end element loads, with entries
+// past it read as -inf (p = q = 0, so r = 0).
 template <typename T>
 __device__ __forceinline__ uint4 load_logits(const T* p, int v, int V, bool vec_ok) {
   constexpr int VEC = Elem<T>::kVec;
   if (vec_ok && v + VEC <= V) return __ldcg(reinterpret_cast<const uint4*>(p + v));
   uint32_t w[4];
+  if (!vec_ok && v + 2 * VEC <= V) {
+    const uintptr_t at = (uintptr_t)(p + v);
+    const uint4* q = reinterpret_cast<const uint4*>(at & ~(uintptr_t)15);
+    const uint4 x = __ldcg(q), y = __ldcg(q + 1);
+    const unsigned sh = (unsigned)(at & 15);
+    uint32_t u[6] = {x.x, x.y, x.z, x.w, y.x, y.y};      // words from the first whole word pair on
+    uint32_t u6 = y.z, u7 = y.w;
+    if (sh & 8) {
+      u[0] = u[2]; u[1] = u[3]; u[2] = u[4]; u[3] = u[5]; u[4] = u6; u[5] = u7;
+    }
+    if (sh & 4) {
+      u[0] = u[1]; u[1] = u[2]; u[2] = u[3]; u[3] = u[4]; u[4] = u[5];
+    }
+    const unsigned bits = (sh & 3) * 8;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = __funnelshift_r(u[k], u[k + 1], bits);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+  }
   if (sizeof(T) == 2) {
     const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
 #pragma unroll
@@ -1775,15 +1737,29 @@ __device__ __forceinline__ unsigned poll_record(const unsigned* p, unsigned* err
   }
 }
 
+// The CTA's largest (value, lowest index) as one 64-bit key in every thread:
+// the value's bits in increasing order (-0 taken as +0, so that equal values
+// tie), then the complemented index.  *s_am holds 0 on entry (reset behind a
+// barrier).
+__device__ __forceinline__ unsigned long long argmax_key_cta(float bm, int bi, unsigned long long* s_am) {
+  uint32_t ub = __float_as_uint(bm + 0.0f);
+  ub = (ub & 0x80000000u) ? ~ub : (ub | 0x80000000u);
+  const uint32_t um = __reduce_max_sync(kFull, ub);
+  const uint32_t ui = __reduce_max_sync(kFull, ub == um ? ~(uint32_t)bi : 0u);
+  if ((threadIdx.x & 31) == 0) atomicMax(s_am, ((unsigned long long)um << 32) | ui);
+  __syncthreads();
+  return *s_am;
+}
+
 // The verifier row's argmax (the lowest index of its largest logit), by the
-// whole CTA from global memory: the token of a row whose residual is empty.
-// *s_am holds 0 on entry (reset behind a barrier).
-template <typename T>
+// whole CTA of NT threads from global memory: the token of a row whose
+// residual is empty.
+template <typename T, int NT>
 __device__ int row_argmax_cta(const T* tp, int V, bool vec_ok, unsigned long long* s_am) {
   constexpr int VEC = Elem<T>::kVec;
   float bm = -pos_inf();
   int bi = kIntMax;
-  for (int v = (int)threadIdx.x * VEC; v < V; v += kCluThreads * VEC) {
+  for (int v = (int)threadIdx.x * VEC; v < V; v += NT * VEC) {
     const uint4 q = load_logits<T>(tp, v, V, vec_ok);
 #pragma unroll
     for (int k = 0; k < VEC; ++k) {
@@ -1794,15 +1770,7 @@ __device__ int row_argmax_cta(const T* tp, int V, bool vec_ok, unsigned long lon
       }
     }
   }
-  // (value, index) as one 64-bit key: the value's bits in increasing order
-  // (-0 taken as +0, so that equal values tie), then the complemented index
-  uint32_t ub = __float_as_uint(bm + 0.0f);
-  ub = (ub & 0x80000000u) ? ~ub : (ub | 0x80000000u);
-  const uint32_t um = __reduce_max_sync(kFull, ub);
-  const uint32_t ui = __reduce_max_sync(kFull, ub == um ? ~(uint32_t)bi : 0u);
-  if ((threadIdx.x & 31) == 0) atomicMax(s_am, ((unsigned long long)um << 32) | ui);
-  __syncthreads();
-  return (int)~(uint32_t)(*s_am);
+  return (int)~(uint32_t)argmax_key_cta(bm, bi, s_am);
 }
 
 template <typename T>
@@ -2009,7 +1977,7 @@ __global__ void __launch_bounds__(kCluThreads, CMSD_CLU_MIN_BLOCKS) resample_bou
       }
       __syncthreads();
       int tok = s_fb;
-      if (tok < 0) tok = row_argmax_cta<T>(tp, a.V, vec_ok, &s_am);   // empty residual: the argmax
+      if (tok < 0) tok = row_argmax_cta<T, kCluThreads>(tp, a.V, vec_ok, &s_am);   // empty residual: the argmax
       if (threadIdx.x == 0) {
         a.out_tokens[(size_t)b * a.Ko + pos] = tok;
         *rec_word(W, rr) = 0u;             // every CTA of the cluster has read it (the barrier above)
@@ -2092,7 +2060,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
   }
 
   if (nrows > 0) {
-    const StreamSplit sp(nrows, a.V, VEC, a.nwarps, stream_min_len(a.V));
+    StreamSplit sp;
+    if (ragged) sp = StreamSplit(nrows, a.V, VEC, a.nwarps, stream_min_len(a.V));
+    else sp = a.split;
     if (w < sp.W) {
       const int64_t e_begin = sp.start(w);
       const int64_t e_end = sp.start(w + 1);

@@ -1,0 +1,125 @@
+"""The one-launch pass (a cluster per sequence) against the streaming kernel.
+
+Windows of at most 16 positions of small and medium problems are taken by one
+kernel with a thread-block cluster per sequence; wider windows by the
+streaming kernel and its second pass.  The uniforms depend on (sequence,
+position, iteration) only, so the same rows in a wider window (K = 17, its
+last position never present) must give the same decisions, bit for bit, and
+signals equal up to the rounding of 32-bit sums added in another order.
+Both are compared with the oracle elsewhere (test_gpu_parity).
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+# Each logarithm, sum and quotient of a signal is good to a few units of 2^-24
+# of values up to ln V < 12: 16 such units.  C adds three terms of at most 1.
+SIGNAL_TOL = 16 * 12 * 2.0 ** -24
+
+
+@pytest.fixture(scope="module")
+def cmsd():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2508_15371_gb300 import cmsd as c
+    c.lib()
+    return c
+
+
+def _inputs(B, K, V, dtype, bonus, masked, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    Kt = K + 1 if bonus else K
+    z = 1.5 * torch.randn((B, Kt, V), generator=g, device="cuda")
+    at = torch.randint(0, V, (B, Kt, 1), generator=g, device="cuda")
+    z.scatter_add_(2, at, 8.0 * torch.rand((B, Kt, 1), generator=g, device="cuda"))
+    t = z + torch.randn((B, Kt, V), generator=g, device="cuda")
+    if masked:
+        off = torch.rand((V,), generator=g, device="cuda") < 0.4
+        off[:2] = False
+        z[:, :, off] = -float("inf")
+        t[:, :, off] = -float("inf")
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    e = torch.rand((B, K, V), generator=g, device="cuda").clamp_(1e-9, 1 - 1e-7)
+    z = z.to(dt)
+    tok = (z[:, :K].float() - torch.log(-torch.log(e))).argmax(dim=2).to(torch.int32)
+    return z[:, :K].contiguous(), t.to(dt), tok
+
+
+def _widen(x, extra):
+    """The same rows with `extra` more (of zeros) at the end of each window."""
+    pad = torch.zeros((x.shape[0], extra) + tuple(x.shape[2:]), dtype=x.dtype, device=x.device)
+    return torch.cat([x, pad], dim=1).contiguous()
+
+
+def _same(narrow, wide, k_row, bonus):
+    K = narrow["out_tokens"].shape[1] - (1 if bonus else 0)
+    for b, kb in enumerate(k_row.tolist()):
+        assert int(narrow["n_accept"][b]) == int(wide["n_accept"][b])
+        assert torch.equal(narrow["out_tokens"][b], wide["out_tokens"][b, :K + (1 if bonus else 0)]), (b, kb)
+        if "accept" in narrow:
+            assert torch.equal(narrow["accept"][b], wide["accept"][b, :K])
+        if "k_next" in narrow:
+            assert int(narrow["k_next"][b]) == int(wide["k_next"][b])
+        for n in ("H", "margin", "conf", "lse"):
+            if n in narrow and kb:
+                d = (narrow[n][b, :kb] - wide[n][b, :kb]).abs().max().item()
+                assert d <= SIGNAL_TOL, (n, b, d)
+        if "argmax" in narrow and kb:
+            assert torch.equal(narrow["argmax"][b, :kb], wide["argmax"][b, :kb])
+
+
+# Sizes: no whole vector, one group, lines and pieces that end inside a row,
+# the cluster sizes of the rule (1 to 16 CTAs of 256 or 512 threads).
+SHAPES = [(1, 1, 2), (3, 2, 33), (2, 16, 1000), (1, 4, 32000), (5, 7, 4099), (8, 8, 32128), (40, 3, 8193),
+          (70, 5, 6400), (150, 2, 4096), (700, 1, 2048), (2, 8, 128256)]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("rule", ["paper", "sampled"])
+@pytest.mark.parametrize("B,K,V", SHAPES)
+def test_one_launch_equals_streaming(cmsd, B, K, V, rule, dtype):
+    es = 4 if dtype == "f32" else 2
+    for bonus in ([False, True] if (V * es) % 16 == 0 else [False]):
+        d, t, tok = _inputs(B, K, V, dtype, bonus, masked=V >= 1000 and B % 2 == 0, seed=V + B)
+        rng = np.random.default_rng(V)
+        k_row = torch.from_numpy(rng.integers(0, K + 1, B).astype(np.int32)).cuda()
+        k_row[0] = K
+        W = 17 - K
+        p = cmsd.params(K, rule, bonus=bonus, tau_base=-0.5)
+        pw = cmsd.params(K, rule, bonus=bonus, tau_base=-0.5)     # the same draft-length bounds
+        d2, tok2 = _widen(d, W), _widen(tok[:, :, None], W)[:, :, 0].contiguous()
+        t2 = _widen(t, W)
+        full = torch.full((B,), K, dtype=torch.int32, device="cuda")
+        for kr in (k_row, None):
+            a = cmsd.confidence_verify(d, t, tok, k_row=kr, p=p, seed=9, iteration=3)
+            b = cmsd.confidence_verify(d2, t2, tok2, k_row=full if kr is None else kr, p=pw, seed=9, iteration=3)
+            _same(a, b, full if kr is None else kr, bonus)
+        kr = k_row
+        sig = cmsd.confidence(d, k_row=kr, p=p)
+        sig2 = cmsd.confidence(d2, k_row=kr, p=pw)
+        for i, kb in enumerate(kr.tolist()):
+            assert int(sig["k_next"][i]) == int(sig2["k_next"][i])
+            assert torch.equal(sig["argmax"][i, :kb], sig2["argmax"][i, :kb])
+        conf = sig["conf"].nan_to_num(0.5).clamp(0, 1)
+        lse = sig["lse"].nan_to_num(0.0)
+        a = cmsd.verify(d, t, tok, conf, draft_lse=lse, k_row=kr, p=p, seed=9, iteration=4)
+        b = cmsd.verify(d2, t2, tok2, _widen(conf[:, :, None], W)[:, :, 0].contiguous(),
+                        draft_lse=_widen(lse[:, :, None], W)[:, :, 0].contiguous(), k_row=kr, p=pw, seed=9, iteration=4)
+        _same(a, b, kr, bonus)
+
+
+def test_device_errors_are_reported(cmsd):
+    """Out-of-range tokens and windows are clamped and set their bits."""
+    d, t, tok = _inputs(3, 4, 4096, "bf16", False, False, 1)
+    p = cmsd.params(4, "sampled")
+    ws = cmsd.workspace(3, 4, 4096)
+    cmsd.workspace_errors(ws)
+    cmsd.confidence_verify(d, t, tok, p=p, ws=ws)
+    assert cmsd.workspace_errors(ws) == 0
+    tok[1, 2] = 4096
+    cmsd.confidence_verify(d, t, tok, p=p, ws=ws)
+    assert cmsd.workspace_errors(ws) == 1
+    tok[1, 2] = 0
+    cmsd.confidence_verify(d, t, tok, p=p, ws=ws, k_row=torch.tensor([4, -1, 5], dtype=torch.int32, device="cuda"))
+    assert cmsd.workspace_errors(ws) == 2
