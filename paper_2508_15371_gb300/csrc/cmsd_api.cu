@@ -28,6 +28,7 @@ int cuda_fail(cudaError_t e) {
 std::mutex g_mu;
 std::map<int, int> g_sms;                                   // device -> SM count
 std::map<std::tuple<int, int, int, int, int>, int> g_occ;   // (dev, dtype, mode, variant, smem) -> blocks/SM
+std::map<std::tuple<int, int, int, int>, int> g_draw_res;    // (dev, dtype, V, CTAs) -> resident clusters
 std::map<std::tuple<int, int, int, int>, int> g_seq_res;     // (dev, dtype, CTAs, threads) -> resident clusters
 std::map<std::tuple<int, int, int>, int> g_occ_res;          // (dev, dtype, sampled) -> blocks/SM
 
@@ -299,6 +300,53 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
   return *nc > 0;
 }
 
+// Clusters of draw_kernel (nc > 0) or of the staged residual draw (nc == 0)
+// that can be resident on the current device for rows of V entries (cached).
+int draw_resident(int dtype, int V, int nc) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const auto key = std::make_tuple(dev, dtype, V, nc);
+  std::lock_guard<std::mutex> lk(g_mu);
+  auto it = g_draw_res.find(key);
+  if (it == g_draw_res.end()) {
+    if (g_draw_res.size() >= 4096) g_draw_res.clear();
+    int n;
+    if (nc == 0) n = dtype == CMSD_F32 ? resample_bound_clusters_f32(V) : resample_bound_clusters_bf16(V);
+    else n = dtype == CMSD_F32 ? draw_clusters_f32(V, nc) : draw_clusters_bf16(V, nc);
+    it = g_draw_res.emplace(key, n).first;
+  }
+  return it->second;
+}
+
+// Which kernel makes the second pass of a streamed call, or false where a
+// row's share does not fit (resample_kernel draws): the staged residual draw
+// while every sequence's cluster can be resident and there is no bonus row;
+// else draw_kernel with four CTAs per sequence up to 152 sequences (B=128 K=8
+// V=128256 with the bonus row: 94.9 us a call against 98.8 with two), two
+// beyond (B=256 K=16 V=152064: 380 us against 383).
+struct DrawPlan {
+  int clusters, nc;                        // nc == 0: the staged residual draw
+};
+bool draw_plan(int dtype, bool sampled, bool bonus, int B, int V, DrawPlan* d) {
+  d->nc = 4;
+  if (sampled && !bonus && B <= draw_resident(dtype, V, 0)) d->nc = 0;
+  else if (B > 152) d->nc = 2;
+  int res = draw_resident(dtype, V, d->nc);
+  if (res < 1 && d->nc == 2) {
+    d->nc = 4;                             // (half a row's groups did not fit)
+    res = draw_resident(dtype, V, 4);
+  }
+  d->clusters = B < 2 * res ? B : 2 * res;
+  return res > 0;
+}
+
+cudaError_t launch_draw(int dtype, bool sampled, const StreamArgs& a, const DrawPlan& d, cudaStream_t s) {
+  if (d.nc == 0)
+    return dtype == CMSD_F32 ? launch_resample_bound_f32(a, d.clusters, s) : launch_resample_bound_bf16(a, d.clusters, s);
+  return dtype == CMSD_F32 ? launch_draw_f32(sampled, a, d.clusters, d.nc, s)
+                           : launch_draw_bf16(sampled, a, d.clusters, d.nc, s);
+}
+
 int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws_bytes,
            cudaStream_t s) {
   int wmax = 0;
@@ -325,17 +373,12 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   int grid = 0;
   rc = stream_grid(dtype, mode, sampled, second, smem, &grid);
   if (rc) return rc;
-  int g2 = 0, nclu = 0;
-  // the sampled rule's residual draw without the bonus row: by group bounds,
-  // one cluster per queued row (up to two per SM pair's worth; more rows loop)
-  const bool bound = second && sampled && !bonus && resample_bound_fits(dtype, a.V);
-  if (second) {
+  int g2 = 0;
+  DrawPlan dp;
+  const bool bound = second && draw_plan(dtype, sampled, bonus, a.B, a.V, &dp);
+  if (second && !bound) {
     rc = resample_grid(dtype, sampled, &g2);
     if (rc) return rc;
-    int sms = 0;
-    rc = device_sms(&sms);
-    if (rc) return rc;
-    nclu = a.B < 2 * sms ? a.B : 2 * sms;
   }
   a.nwarps = grid * kStreamWarps;
   if (!a.k_row) a.split = StreamSplit(a.B * a.K, a.V, dtype == CMSD_F32 ? 4 : 8, a.nwarps, stream_min_len(a.V));
@@ -349,7 +392,7 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
     StreamArgs b = a;
     b.nwarps = g2 * kResWarps;
     if (bound)
-      e = dtype == CMSD_F32 ? launch_resample_bound_f32(b, nclu, s) : launch_resample_bound_bf16(b, nclu, s);
+      e = launch_draw(dtype, sampled, b, dp, s);
     else
       e = dtype == CMSD_F32 ? launch_resample_f32(sampled, b, g2, s) : launch_resample_bf16(sampled, b, g2, s);
     if (e != cudaSuccess) {
@@ -533,15 +576,13 @@ int cmsd_test_record_wait_timeout(const void* draft_logits, const void* target_l
   if (B == 0 || K == 0) return CMSD_OK;
   if (!draft_logits || !target_logits || !out_tokens) return CMSD_EINVAL;
   if (!aligned16(draft_logits) || !aligned16(target_logits)) return CMSD_EALIGN;
-  if (!resample_bound_fits(dtype, V)) return CMSD_EDTYPE;
+  DrawPlan dp;
+  if (!draw_plan(dtype, true, false, B, V, &dp)) return CMSD_EDTYPE;
   int wmax = 0;
   rc = wmax_warps(&wmax);
   if (rc) return rc;
   const Layout L = make_layout(B, K, wmax);
   if (!ws || ws_bytes < L.total) return CMSD_ENOWS;
-  int sms = 0;
-  rc = device_sms(&sms);
-  if (rc) return rc;
   StreamArgs a = blank_args();
   fill_sizes(a, B, K, V);
   a.draft = draft_logits;
@@ -554,8 +595,7 @@ int cmsd_test_record_wait_timeout(const void* draft_logits, const void* target_l
   // no record is released: every sequence's wait runs out
   cudaError_t e = cudaMemsetAsync(a.ws.rec, 0, (size_t)B * sizeof(int4), s);
   if (e != cudaSuccess) return cuda_fail(e);
-  const int nclu = B < 2 * sms ? B : 2 * sms;
-  e = dtype == CMSD_F32 ? launch_resample_bound_f32(a, nclu, s) : launch_resample_bound_bf16(a, nclu, s);
+  e = launch_draw(dtype, true, a, dp, s);
   return e == cudaSuccess ? CMSD_OK : cuda_fail(e);
 }
 

@@ -194,7 +194,7 @@ struct StreamArgs {
   int nwarps;             // warps launched
   StreamSplit split;      // full windows: the cut of the B*K rows
   int rec_by_seq;         // 1: second-pass records at each sequence's own slot rec[b], every sequence
-                          // writing one (the bounded residual draw); 0: a compacted queue (rec_count)
+                          // writing one (the draw by group bounds); 0: a compacted queue (rec_count)
 };
 
 // Kernel launchers (one translation unit per dtype).  `second`: this call
@@ -215,13 +215,20 @@ int seq_clusters_bf16(int nc, int threads);
 bool seq_draw_fits(int dtype, int V);
 cudaError_t launch_resample_f32(bool sampled, const StreamArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_resample_bf16(bool sampled, const StreamArgs& a, int grid, cudaStream_t s);
-// The residual draw by group bounds (sampled rule, no bonus row): clusters
-// of CTAs, one queued row per cluster at a time; resample_bound_fits says
-// whether a row's share fits its shared memory and such a cluster can be
-// resident on the current device (else resample_kernel draws the residual).
+// The draw by group bounds (residual and bonus tokens): clusters of nc CTAs,
+// one sequence per cluster at a time; draw_clusters says how many such
+// clusters can be resident on the current device for rows of V entries (0:
+// resample_kernel takes the call).
+cudaError_t launch_draw_f32(bool sampled, const StreamArgs& a, int clusters, int nc, cudaStream_t s);
+cudaError_t launch_draw_bf16(bool sampled, const StreamArgs& a, int clusters, int nc, cudaStream_t s);
+int draw_clusters_f32(int V, int nc);
+int draw_clusters_bf16(int V, int nc);
+// The residual draw with its share staged in shared memory (clusters of a
+// fixed size); how many clusters can be resident (0: the share does not fit).
 cudaError_t launch_resample_bound_f32(const StreamArgs& a, int clusters, cudaStream_t s);
 cudaError_t launch_resample_bound_bf16(const StreamArgs& a, int clusters, cudaStream_t s);
-bool resample_bound_fits(int dtype, int V);
+int resample_bound_clusters_f32(int V);
+int resample_bound_clusters_bf16(int V);
 cudaError_t occupancy_stream(int dtype, int mode, bool sampled, bool second, size_t smem,
                              int* blocks_per_sm);
 cudaError_t occupancy_resample(int dtype, bool sampled, int* blocks_per_sm);

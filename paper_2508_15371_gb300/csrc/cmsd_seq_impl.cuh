@@ -19,12 +19,13 @@
 //            sequence's outputs;
 //   draw     under the sampled rule, or for the bonus row, the cluster draws
 //            the token itself: the race by group bounds (cluster_draw).
+//            Its rows were streamed moments ago and come from L2.
 #pragma once
 #include "cmsd_stream_impl.cuh"
 
 namespace cmsd {
 
-constexpr int kSeqMaxCtas = 16;          // CTAs per cluster (16: a non-portable size)
+constexpr int kSeqMaxCtas = kDrawMaxCtas;   // CTAs per cluster (16: a non-portable size)
 constexpr int kSeqMaxK = kPackedMaxK;    // positions per window
 #ifndef CMSD_SEQ_UNROLL
 #define CMSD_SEQ_UNROLL 4
@@ -32,262 +33,6 @@ constexpr int kSeqMaxK = kPackedMaxK;    // positions per window
 #ifndef CMSD_SEQ_UNROLL1
 #define CMSD_SEQ_UNROLL1 8
 #endif
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() {
-  cluster_arrive();
-  cluster_wait();
-}
-
-// ---------------------------------------------------------------------------
-// the draw by group bounds, by the cluster that holds the sequence
-// ---------------------------------------------------------------------------
-//
-// The race of resample_bound_kernel (bound, probe, race, level 2; the same
-// keys, filter and tie rule), with the group maxima taken from global memory:
-// the row was streamed moments ago and comes from L2, so it is not staged.
-// The bonus race is the same with r = p, p relative to the row's maximum
-// (the normaliser does not change the order of the keys).
-
-constexpr int kDrawCands = 1024;         // candidate list; past it the share is raced whole
-
-template <typename T, int NT>
-struct DrawShared {
-  static constexpr int kLpg = kGroup / Elem<T>::kVec;     // lanes per group
-  static constexpr int kSets = NT / kLpg;                 // lane sets per CTA
-  unsigned long long best[2];            // key_min_cta of the probes, of the race
-  unsigned long long am;                 // rank 0: row_argmax_cta's reduction
-  unsigned long long arg[kSeqMaxCtas];   // rank 0: each CTA's (value, ~index) of the bonus argmax
-  uint4 qt[NT], qd[NT];                  // vectors of each lane set's best group
-  int probe[kSets];                      // the group each lane set probed
-  int list[kDrawCands];
-  float ref[kSeqMaxCtas];                // each CTA's largest logit (bonus race)
-  float k1[kSeqMaxCtas];                 // each CTA's least probe key
-  float rk[kSeqMaxCtas];                 // rank 0: each CTA's (key, group, token)
-  int rg[kSeqMaxCtas], rt[kSeqMaxCtas];
-  float wmax[NT / 32];
-  int n, hold, fb;
-};
-
-// Groups per CTA of an nc-CTA cluster: a multiple of four, so that a share
-// starts on a block of four group uniforms.
-__host__ __device__ inline int draw_share(int ng, int nc) { return ((ng + nc - 1) / nc + 3) & ~3; }
-// dynamic shared memory of the draw: the share's uniforms and bounds
-__host__ __device__ inline size_t draw_smem_bytes(int V, int nc) {
-  return (size_t)draw_share((V + kGroup - 1) / kGroup, nc) * 2 * sizeof(float);
-}
-
-template <typename T, int NT>
-__device__ void cluster_draw(const StreamArgs& a, cg::cluster_group& cl, int nc, int cr, int b, int pos, bool bonus,
-                             const T* tp, const T* dp, RowStat st, float* s_u, DrawShared<T, NT>& sh) {
-  constexpr int VEC = Elem<T>::kVec;
-  constexpr int LPG = DrawShared<T, NT>::kLpg;
-  constexpr int SETS = DrawShared<T, NT>::kSets;
-  constexpr int UL = 4;                  // vectors in flight per thread of the maxima pass
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int sub = lane % LPG, set = tid / LPG;
-  const int ng = (a.V + kGroup - 1) / kGroup;
-  const int ngs = draw_share(ng, nc);
-  const int gs = cr * ngs;                                   // the share: groups [gs, gs + nloc)
-  const int nloc = max(0, min(ng, gs + ngs) - gs);
-  float* s_rb = s_u + ngs;
-  const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
-  const uint32_t cw_grp = iter_word(a.iteration, kPurposeGroup);
-  const uint32_t cw_ent = iter_word(a.iteration, kPurposeResidual);
-  const bool vec_ok = ((((uintptr_t)tp) | ((uintptr_t)dp)) & 15) == 0;
-  if (tid == 0) {
-    sh.best[0] = sh.best[1] = ~0ull;
-    sh.am = 0ull;
-    sh.n = 0;
-    sh.hold = 0;
-  }
-  // largest logit of each group of the share (-inf past the row end)
-  const int nv = nloc * LPG, v0 = gs * kGroup;
-  for (int j0 = 0; j0 < nv; j0 += NT * UL) {
-    uint4 q[UL];
-#pragma unroll
-    for (int k = 0; k < UL; ++k) {
-      const int j = j0 + k * NT + tid;
-      q[k] = j < nv ? load_logits<T>(tp, v0 + j * VEC, a.V, vec_ok) : neg_inf_vec<T>();
-    }
-#pragma unroll
-    for (int k = 0; k < UL; ++k) {
-      const int j = j0 + k * NT + tid;
-      float m = vec_max(q[k], (const T*)nullptr);
-#pragma unroll
-      for (int o = 1; o < LPG; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
-      if (sub == 0 && j < nv) s_rb[j / LPG] = m;
-    }
-  }
-  for (int q = tid; q < (nloc + 3) / 4; q += NT) {
-    const U4 wd = philox4x32_10(U4{(uint32_t)(gs / 4 + q), (uint32_t)b, (uint32_t)pos, cw_grp}, k0, k1);
-    s_u[4 * q + 0] = word_to_unit(wd.x);
-    s_u[4 * q + 1] = word_to_unit(wd.y);
-    s_u[4 * q + 2] = word_to_unit(wd.z);
-    s_u[4 * q + 3] = word_to_unit(wd.w);
-  }
-  __syncthreads();
-  if (bonus) {                           // p relative to the row's largest logit
-    float m = -pos_inf();
-    for (int gl = tid; gl < nloc; gl += NT) m = fmaxf(m, s_rb[gl]);
-    m = warp_max(m);
-    if (lane == 0) sh.wmax[warp] = m;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NT / 32; ++k) m = fmaxf(m, sh.wmax[k]);
-    if (tid < nc) *cl.map_shared_rank(&sh.ref[cr], tid) = m;
-    cluster_sync();
-    for (int c = 0; c < nc; ++c) m = fmaxf(m, sh.ref[c]);
-    st = RowStat{mlog2e(m), 1.0f, 0.f, 0.f};
-  }
-  // bound: each thread keeps its lowest U_g / Rb_g (compared as U_a Rb_b <
-  // U_b Rb_a), then each lane set the lowest of its LPG threads'
-  float bu = 0.f, brb = 1.f;
-  int lg = -1;
-  for (int gl = tid; gl < nloc; gl += NT) {
-    const float rb = group_bound(s_rb[gl], st);
-    s_rb[gl] = rb;
-    const float u = s_u[gl];
-    if (lg < 0 || u * brb < bu * rb) {
-      bu = u;
-      brb = rb;
-      lg = gl;
-    }
-  }
-#pragma unroll
-  for (int o = 1; o < LPG; o <<= 1) {
-    const float u2 = __shfl_xor_sync(kFull, bu, o), rb2 = __shfl_xor_sync(kFull, brb, o);
-    const int g2 = __shfl_xor_sync(kFull, lg, o);
-    if (g2 >= 0 && (lg < 0 || u2 * brb < bu * rb2 || (u2 * brb == bu * rb2 && g2 < lg))) {
-      bu = u2;
-      brb = rb2;
-      lg = g2;
-    }
-  }
-  // probe: the lane set's lowest-bound group, exactly
-  float sk = pos_inf();                  // the lane set's best (key, group), its vectors in qt, qd
-  int sg = kIntMax;
-  {
-    uint4 qt = neg_inf_vec<T>(), qd = bonus ? make_uint4(0, 0, 0, 0) : neg_inf_vec<T>();
-    if (lg >= 0) {
-      qt = load_logits<T>(tp, (gs + lg) * kGroup + sub * VEC, a.V, vec_ok);
-      if (!bonus) qd = load_logits<T>(dp, (gs + lg) * kGroup + sub * VEC, a.V, vec_ok);
-    }
-    sk = group_key<T>(qt, qd, st, lg >= 0 ? s_u[lg] : 0.f, lg >= 0);
-    sg = sk != pos_inf() ? gs + lg : kIntMax;
-    sh.qt[tid] = qt;
-    sh.qd[tid] = qd;
-    if (sub == 0) sh.probe[set] = lg;
-  }
-  float K1 = sk;
-  int g1 = sg;
-  key_min_cta(K1, g1, &sh.best[0]);
-  // K1: the least probe key of the cluster, an upper bound on the winner's key
-  if (tid < nc) *cl.map_shared_rank(&sh.k1[cr], tid) = K1;
-  cluster_sync();
-  for (int c = 0; c < nc; ++c) K1 = fminf(K1, sh.k1[c]);
-  // race: the groups of the share that the bound leaves at or below K1 and
-  // that no lane set has probed
-  for (int gl = tid; gl < nloc; gl += NT) {
-    if (!(s_u[gl] * kRaceFilter > K1 * s_rb[gl]) && sh.probe[(gl % NT) / LPG] != gl) {
-      const int i = atomicAdd(&sh.n, 1);
-      if (i < kDrawCands) sh.list[i] = gl;
-    }
-  }
-  __syncthreads();
-  const int ncand = sh.n;
-  const bool whole = ncand > kDrawCands;
-  const int items = whole ? nloc : ncand;
-  for (int i0 = 0; i0 < items; i0 += SETS) {                 // block-uniform trip count
-    const int i = i0 + set;
-    const int gl = i < items ? (whole ? i : sh.list[i]) : -1;
-    uint4 qt = neg_inf_vec<T>(), qd = bonus ? make_uint4(0, 0, 0, 0) : neg_inf_vec<T>();
-    if (gl >= 0) {
-      qt = load_logits<T>(tp, (gs + gl) * kGroup + sub * VEC, a.V, vec_ok);
-      if (!bonus) qd = load_logits<T>(dp, (gs + gl) * kGroup + sub * VEC, a.V, vec_ok);
-    }
-    const float key = group_key<T>(qt, qd, st, gl >= 0 ? s_u[gl] : 0.f, gl >= 0);
-    if (key != pos_inf() && (key < sk || (key == sk && gs + gl < sg))) {   // the whole lane set agrees
-      sk = key;
-      sg = gs + gl;
-      sh.qt[tid] = qt;
-      sh.qd[tid] = qd;
-    }
-  }
-  // the CTA's least (key, group), the lane set holding it, and its level-2
-  // winner, pushed to rank 0 of the cluster
-  float ck = sk;
-  int cgrp = sg;
-  key_min_cta(ck, cgrp, &sh.best[1]);
-  if (sub == 0 && cgrp != kIntMax && sk == ck && sg == cgrp) sh.hold = set;   // holders share one group
-  __syncthreads();
-  if (warp == 0) {
-    int tok = -1;
-    if (cgrp != kIntMax) {
-      const int h = sh.hold;
-      tok = race_group_entries<T>(sh.qt[h * LPG + sub], sh.qd[h * LPG + sub], cgrp, 0, lane, st, (uint32_t)b,
-                                  (uint32_t)pos, cw_ent, k0, k1);
-    }
-    if (lane == 0) {
-      *cl.map_shared_rank(&sh.rk[cr], 0) = ck;
-      *cl.map_shared_rank(&sh.rg[cr], 0) = cgrp;
-      *cl.map_shared_rank(&sh.rt[cr], 0) = tok;
-    }
-  }
-  cluster_sync();                             // every CTA's result is in rank 0
-  if (cr == 0) {
-    if (warp == 0) {
-      float k = lane < nc ? sh.rk[lane] : pos_inf();
-      const int g = lane < nc ? sh.rg[lane] : kIntMax;
-      const uint32_t kb = __reduce_min_sync(kFull, __float_as_uint(k));      // keys are >= 0 or +inf
-      const uint32_t gb = __reduce_min_sync(kFull, __float_as_uint(k) == kb ? (uint32_t)g : 0xFFFFFFFFu);
-      const unsigned who = __ballot_sync(kFull, __float_as_uint(k) == kb && (uint32_t)g == gb);
-      const int c = __ffs(who) - 1;
-      if (lane == 0) sh.fb = (gb == (uint32_t)kIntMax || sh.rt[c] < 0) ? -1 : sh.rt[c];
-    }
-    __syncthreads();
-    int tok = sh.fb;
-    if (tok < 0) tok = row_argmax_cta<T, NT>(tp, a.V, vec_ok, &sh.am);   // empty residual: the argmax
-    if (tid == 0) a.out_tokens[(size_t)b * a.Ko + pos] = tok;
-  }
-}
-
-// The extra verifier row's argmax (PAPER rule, bonus row; lowest index), each
-// CTA a share of the row.
-template <typename T, int NT>
-__device__ void cluster_argmax(const StreamArgs& a, cg::cluster_group& cl, int nc, int cr, int b, int pos, const T* tp,
-                               DrawShared<T, NT>& sh) {
-  constexpr int VEC = Elem<T>::kVec;
-  const int tid = threadIdx.x;
-  const bool vec_ok = (((uintptr_t)tp) & 15) == 0;
-  const int nvec = (a.V + VEC - 1) / VEC;
-  const int per = (nvec + nc - 1) / nc;
-  const int j1 = min(nvec, (cr + 1) * per);
-  if (tid == 0) sh.am = 0ull;
-  float bm = -pos_inf();
-  int bi = kIntMax;
-  for (int j = cr * per + tid; j < j1; j += NT) {
-    const uint4 q = load_logits<T>(tp, j * VEC, a.V, vec_ok);
-#pragma unroll
-    for (int k = 0; k < VEC; ++k) {
-      const float z = logit_at<T>(q, k);
-      if (j * VEC + k < a.V && (z > bm || (z == bm && j * VEC + k < bi))) {
-        bm = z;
-        bi = j * VEC + k;
-      }
-    }
-  }
-  __syncthreads();
-  const unsigned long long key = argmax_key_cta(bm, bi, &sh.am);
-  if (tid == 0) *cl.map_shared_rank(&sh.arg[cr], 0) = key;
-  cluster_sync();
-  if (cr == 0 && tid == 0) {
-    unsigned long long m = 0ull;
-    for (int c = 0; c < nc; ++c) m = max(m, sh.arg[c]);
-    a.out_tokens[(size_t)b * a.Ko + pos] = (int)~(uint32_t)m;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // the kernel
 // ---------------------------------------------------------------------------
@@ -461,14 +206,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
       return;
     }
     const bool bonus = kind == kSeqBonus;
-    RowStat st{0.f, 1.f, 0.f, 0.f};
-    const T* dp = tp;
-    if (!bonus) {
-      const float4 q = s_row[n].stat;
-      st = RowStat{q.z, 1.0f / q.w, q.x, -1.0f / q.y};
-      dp = (const T*)a.draft + ((size_t)b * a.K + n) * (size_t)a.V;
-    }
-    cluster_draw<T, NT>(a, cl, nc, cr, b, n, bonus, tp, dp, st, s_u, sh);
+    const float4 q = bonus ? make_float4(0.f, 1.f, 0.f, 1.f) : s_row[n].stat;
+    const T* dp = bonus ? tp : (const T*)a.draft + ((size_t)b * a.K + n) * (size_t)a.V;
+    cluster_draw<T, NT, 4>(a, cl, nc, cr, b, n, bonus, tp, dp, make_float2(q.z, q.w), make_float2(q.x, q.y), s_u, sh);
   }
 }
 

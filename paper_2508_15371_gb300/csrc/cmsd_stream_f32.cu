@@ -11,14 +11,17 @@ cudaError_t launch_resample_f32(bool sampled, const StreamArgs& a, int grid, cud
   return launch_resample_t<float>(sampled, a, grid, s);
 }
 
+cudaError_t launch_draw_f32(bool sampled, const StreamArgs& a, int clusters, int nc, cudaStream_t s) {
+  return launch_draw_t<float>(sampled, a, clusters, nc, s);
+}
+
+int draw_clusters_f32(int V, int nc) { return draw_clusters_t<float>(V, nc); }
+
 cudaError_t launch_resample_bound_f32(const StreamArgs& a, int clusters, cudaStream_t s) {
   return launch_resample_bound_t<float>(a, clusters, s);
 }
 
-bool resample_bound_fits_bf16(int V);
-bool resample_bound_fits(int dtype, int V) {
-  return dtype == 0 ? resample_bound_fits_t<float>(V) : resample_bound_fits_bf16(V);
-}
+int resample_bound_clusters_f32(int V) { return resample_bound_clusters_t<float>(V); }
 
 cudaError_t occupancy_resample(int dtype, bool sampled, int* nb) {
   return dtype == 0 ? occupancy_resample_t<float>(sampled, nb) : occupancy_resample_bf16(sampled, nb);

@@ -53,9 +53,6 @@
 // arithmetic so that e^(z-m) * (z-m) is 0, not NaN.
 #pragma once
 #include <cooperative_groups.h>
-#include <map>
-#include <mutex>
-#include <utility>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -1575,7 +1572,7 @@ __global__ void __launch_bounds__(kResThreads, CMSD_RES_MIN_BLOCKS) resample_ker
 }
 
 // ---------------------------------------------------------------------------
-// residual draw by group bounds (sampled rule, no bonus row)
+// the draw by group bounds
 // ---------------------------------------------------------------------------
 //
 // The same two-level race, with the same keys, reading far less.  Since
@@ -1584,12 +1581,11 @@ __global__ void __launch_bounds__(kResThreads, CMSD_RES_MIN_BLOCKS) resample_ker
 //   R_g <= Rb_g = kGroup p(m_g) (1 + 2^-16) + 2^-100
 // (the factor covers the rounding of the 32-term sum and of ex2, the floor
 // entries whose p underflows), and its key E_g / R_g >= U_g / Rb_g because
-// E = -log(1 - U) >= U.  A cluster of kCluCtas CTAs takes one sequence's
-// rejected row (its record at the sequence's own slot), a share of its groups
-// each:
-//   stage   the share of the target row is copied to shared memory (cp.async)
-//           while the share's uniforms are drawn;
-//   bound   m_g and Rb_g of every group of the share, from shared memory;
+// E = -log(1 - U) >= U.  A cluster of CTAs takes one sequence's row, a share
+// of its groups each:
+//   maxima  m_g of every group of the share, while the share's uniforms are
+//           drawn;
+//   bound   Rb_g of every group;
 //   probe   each lane set races its lowest-bound group exactly (the drafter
 //           vectors are the only logits read from memory besides the
 //           target row); K1, the least of these keys over the cluster, is
@@ -1603,38 +1599,12 @@ __global__ void __launch_bounds__(kResThreads, CMSD_RES_MIN_BLOCKS) resample_ker
 // relative, far above the rounding of E, of the sum and of the quotient), so
 // it can neither win nor tie: the token is the one the race over every group
 // draws.  The drafter row and the exponentials are touched for a few groups
-// per row instead of all of them.
-#ifndef CMSD_CLU_CTAS
-#define CMSD_CLU_CTAS 4
-#endif
-#ifndef CMSD_CLU_THREADS
-#define CMSD_CLU_THREADS 512
-#endif
-#ifndef CMSD_CLU_MIN_BLOCKS
-#define CMSD_CLU_MIN_BLOCKS 2
-#endif
-constexpr int kCluCtas = CMSD_CLU_CTAS;                  // CTAs per row (one cluster)
-constexpr int kCluThreads = CMSD_CLU_THREADS;
-constexpr int kCluWarps = kCluThreads / 32;
-constexpr int kCluCands = 1024;                          // candidate list; past it the share is raced whole
-constexpr size_t kCluSmemMax = 200 * 1024;               // larger shares take the race over every group
+// per row instead of all of them.  The bonus race is the same with r = p, p
+// relative to the row's maximum (the normaliser does not change the order of
+// the keys).
 constexpr float kGroupBoundScale = 32.0f + 1.0f / 2048.0f;   // kGroup (1 + 2^-16)
 constexpr float kGroupBoundFloor = 0x1p-100f;
 static_assert(kGroup == 32, "the bound's factor is kGroup (1 + 2^-16)");
-
-// Groups per CTA: a multiple of four, so that a share starts on a block of
-// four group uniforms.
-__host__ __device__ inline int clu_share(int ng) {
-  const int s = (ng + kCluCtas - 1) / kCluCtas;
-  return (s + 3) & ~3;
-}
-// Dynamic shared memory of one CTA: the staged target share, the share's
-// uniforms and bounds, the candidate list.
-template <typename T>
-__host__ __device__ inline size_t clu_smem_bytes(int V) {
-  const size_t ngs = (size_t)clu_share((V + kGroup - 1) / kGroup);
-  return ngs * kGroup * sizeof(T) + ngs * 2 * sizeof(float) + (size_t)kCluCands * sizeof(int);
-}
 
 __device__ __forceinline__ float expo_u(float u) { return -log1pf(-u); }   // expo() of the same word
 
@@ -1645,35 +1615,6 @@ __device__ __forceinline__ float vec_max(uint4 q, const uint16_t*) {
 }
 __device__ __forceinline__ float vec_max(uint4 q, const float*) {
   return fmaxf(fmaxf(__uint_as_float(q.x), __uint_as_float(q.y)), fmaxf(__uint_as_float(q.z), __uint_as_float(q.w)));
-}
-
-// The staged share keeps group g's vectors in 16-byte slots g LPG .. g LPG +
-// LPG - 1, vector k in slot g LPG + ((k + rot(g)) mod LPG), rot(g) = g LPG / 8:
-// a thread that reads a whole group (one vector per load) and its neighbours
-// reading theirs then touch eight different 16-byte bank slots per quarter
-// warp.
-template <int LPG>
-__device__ __forceinline__ int clu_slot(int g, int k) {
-  return g * LPG + ((k + ((g * LPG) >> 3)) & (LPG - 1));
-}
-
-// The largest logit of staged group g.
-__device__ __forceinline__ float group_max(const unsigned char* stage, int g, const uint16_t*) {
-  const uint4* q = reinterpret_cast<const uint4*>(stage);
-  const uint4 a = q[clu_slot<4>(g, 0)], b = q[clu_slot<4>(g, 1)], c = q[clu_slot<4>(g, 2)], d = q[clu_slot<4>(g, 3)];
-  const uint32_t x = bmax2(bmax2(a.x, b.x), bmax2(c.x, d.x));
-  const uint32_t y = bmax2(bmax2(a.y, b.y), bmax2(c.y, d.y));
-  const uint32_t z = bmax2(bmax2(a.z, b.z), bmax2(c.z, d.z));
-  const uint32_t w = bmax2(bmax2(a.w, b.w), bmax2(c.w, d.w));
-  const uint32_t m = bmax2(bmax2(x, y), bmax2(z, w));
-  return fmaxf(bf_lo(m), bf_hi(m));
-}
-__device__ __forceinline__ float group_max(const unsigned char* stage, int g, const float*) {
-  const uint4* q = reinterpret_cast<const uint4*>(stage);
-  float m = -pos_inf();
-#pragma unroll
-  for (int k = 0; k < 8; ++k) m = fmaxf(m, vec_max(q[clu_slot<8>(g, k)], (const float*)nullptr));
-  return m;
 }
 
 // Rb_g from the group's largest target logit.
@@ -1773,8 +1714,381 @@ __device__ int row_argmax_cta(const T* tp, int V, bool vec_ok, unsigned long lon
   return (int)~(uint32_t)argmax_key_cta(bm, bi, s_am);
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
+}
+
+constexpr int kDrawMaxCtas = 16;         // CTAs per cluster
+constexpr int kDrawCands = 1024;         // candidate list; past it the share is raced whole
+
+template <typename T, int NT>
+struct DrawShared {
+  static constexpr int kLpg = kGroup / Elem<T>::kVec;     // lanes per group
+  static constexpr int kSets = NT / kLpg;                 // lane sets per CTA
+  unsigned long long best[2];            // key_min_cta of the probes, of the race
+  unsigned long long am;                 // rank 0: row_argmax_cta's reduction
+  unsigned long long arg[kDrawMaxCtas];   // rank 0: each CTA's (value, ~index) of the bonus argmax
+  uint4 qt[NT], qd[NT];                  // vectors of each lane set's best group
+  int probe[kSets];                      // the group each lane set probed
+  int list[kDrawCands];
+  float ref[kDrawMaxCtas];                // each CTA's largest logit (bonus race)
+  float k1[kDrawMaxCtas];                 // each CTA's least probe key
+  float rk[kDrawMaxCtas];                 // rank 0: each CTA's (key, group, token)
+  int rg[kDrawMaxCtas], rt[kDrawMaxCtas];
+  float wmax[NT / 32];
+  int n, hold, fb;
+};
+
+// Groups per CTA of an nc-CTA cluster: a multiple of four, so that a share
+// starts on a block of four group uniforms.
+__host__ __device__ inline int draw_share(int ng, int nc) { return ((ng + nc - 1) / nc + 3) & ~3; }
+// dynamic shared memory of the draw: the share's uniforms and bounds
+__host__ __device__ inline size_t draw_smem_bytes(int V, int nc) {
+  return (size_t)draw_share((V + kGroup - 1) / kGroup, nc) * 2 * sizeof(float);
+}
+
+// UL: vectors in flight per thread of the maxima pass.  ts, ds: the row's
+// target and drafter (max * log2e, sum).
+template <typename T, int NT, int UL>
+__device__ void cluster_draw(const StreamArgs& a, cg::cluster_group& cl, int nc, int cr, int b, int pos, bool bonus,
+                             const T* tp, const T* dp, float2 ts, float2 ds, float* s_u, DrawShared<T, NT>& sh) {
+  constexpr int VEC = Elem<T>::kVec;
+  constexpr int LPG = DrawShared<T, NT>::kLpg;
+  constexpr int SETS = DrawShared<T, NT>::kSets;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sub = lane % LPG, set = tid / LPG;
+  const int ng = (a.V + kGroup - 1) / kGroup;
+  const int ngs = draw_share(ng, nc);
+  const int gs = cr * ngs;                                   // the share: groups [gs, gs + nloc)
+  const int nloc = max(0, min(ng, gs + ngs) - gs);
+  float* s_rb = s_u + ngs;
+  const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
+  const uint32_t cw_grp = iter_word(a.iteration, kPurposeGroup);
+  const uint32_t cw_ent = iter_word(a.iteration, kPurposeResidual);
+  const bool vec_ok = ((((uintptr_t)tp) | ((uintptr_t)dp)) & 15) == 0;
+  if (tid == 0) {
+    sh.best[0] = sh.best[1] = ~0ull;
+    sh.am = 0ull;
+    sh.n = 0;
+    sh.hold = 0;
+  }
+  // largest logit of each group of the share (-inf past the row end); the
+  // uniforms are drawn while the first vectors are on their way
+  const int nv = nloc * LPG, v0 = gs * kGroup;
+  uint4 q[UL];
+  auto request = [&](int j0) {
+#pragma unroll
+    for (int k = 0; k < UL; ++k) {
+      const int j = j0 + k * NT + tid;
+      q[k] = j < nv ? load_logits<T>(tp, v0 + j * VEC, a.V, vec_ok) : neg_inf_vec<T>();
+    }
+  };
+  request(0);
+  for (int i = tid; i < (nloc + 3) / 4; i += NT) {
+    const U4 wd = philox4x32_10(U4{(uint32_t)(gs / 4 + i), (uint32_t)b, (uint32_t)pos, cw_grp}, k0, k1);
+    *reinterpret_cast<float4*>(s_u + 4 * i) =
+        make_float4(word_to_unit(wd.x), word_to_unit(wd.y), word_to_unit(wd.z), word_to_unit(wd.w));
+  }
+  for (int j0 = 0; j0 < nv; j0 += NT * UL) {
+#pragma unroll
+    for (int k = 0; k < UL; ++k) {
+      const int j = j0 + k * NT + tid;
+      float m = vec_max(q[k], (const T*)nullptr);
+#pragma unroll
+      for (int o = 1; o < LPG; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+      if (sub == 0 && j < nv) s_rb[j / LPG] = m;
+    }
+    if (j0 + NT * UL < nv) request(j0 + NT * UL);
+  }
+  RowStat st{ts.x, 1.0f / ts.y, ds.x, -1.0f / ds.y};
+  __syncthreads();
+  if (bonus) {                           // p relative to the row's largest logit
+    float m = -pos_inf();
+    for (int gl = tid; gl < nloc; gl += NT) m = fmaxf(m, s_rb[gl]);
+    m = warp_max(m);
+    if (lane == 0) sh.wmax[warp] = m;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NT / 32; ++k) m = fmaxf(m, sh.wmax[k]);
+    if (tid < nc) *cl.map_shared_rank(&sh.ref[cr], tid) = m;
+    cluster_sync();
+    for (int c = 0; c < nc; ++c) m = fmaxf(m, sh.ref[c]);
+    st = RowStat{mlog2e(m), 1.0f, 0.f, 0.f};
+  }
+  // bound: each thread keeps its lowest U_g / Rb_g (compared as U_a Rb_b <
+  // U_b Rb_a), then each lane set the lowest of its LPG threads'
+  float bu = 0.f, brb = 1.f;
+  int lg = -1;
+  for (int gl = tid; gl < nloc; gl += NT) {
+    const float rb = group_bound(s_rb[gl], st);
+    s_rb[gl] = rb;
+    const float u = s_u[gl];
+    if (lg < 0 || u * brb < bu * rb) {
+      bu = u;
+      brb = rb;
+      lg = gl;
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < LPG; o <<= 1) {
+    const float u2 = __shfl_xor_sync(kFull, bu, o), rb2 = __shfl_xor_sync(kFull, brb, o);
+    const int g2 = __shfl_xor_sync(kFull, lg, o);
+    if (g2 >= 0 && (lg < 0 || u2 * brb < bu * rb2 || (u2 * brb == bu * rb2 && g2 < lg))) {
+      bu = u2;
+      brb = rb2;
+      lg = g2;
+    }
+  }
+  // probe: the lane set's lowest-bound group, exactly
+  float sk = pos_inf();                  // the lane set's best (key, group), its vectors in qt, qd
+  int sg = kIntMax;
+  {
+    uint4 qt = neg_inf_vec<T>(), qd = bonus ? make_uint4(0, 0, 0, 0) : neg_inf_vec<T>();
+    if (lg >= 0) {
+      qt = load_logits<T>(tp, (gs + lg) * kGroup + sub * VEC, a.V, vec_ok);
+      if (!bonus) qd = load_logits<T>(dp, (gs + lg) * kGroup + sub * VEC, a.V, vec_ok);
+    }
+    sk = group_key<T>(qt, qd, st, lg >= 0 ? s_u[lg] : 0.f, lg >= 0);
+    sg = sk != pos_inf() ? gs + lg : kIntMax;
+    sh.qt[tid] = qt;
+    sh.qd[tid] = qd;
+    if (sub == 0) sh.probe[set] = lg;
+  }
+  float K1 = sk;
+  int g1 = sg;
+  key_min_cta(K1, g1, &sh.best[0]);
+  // K1: the least probe key of the cluster, an upper bound on the winner's key
+  if (tid < nc) *cl.map_shared_rank(&sh.k1[cr], tid) = K1;
+  cluster_sync();
+  for (int c = 0; c < nc; ++c) K1 = fminf(K1, sh.k1[c]);
+  // race: the groups of the share that the bound leaves at or below K1 and
+  // that no lane set has probed
+  for (int gl = tid; gl < nloc; gl += NT) {
+    if (!(s_u[gl] * kRaceFilter > K1 * s_rb[gl]) && sh.probe[(gl % NT) / LPG] != gl) {
+      const int i = atomicAdd(&sh.n, 1);
+      if (i < kDrawCands) sh.list[i] = gl;
+    }
+  }
+  __syncthreads();
+  const int ncand = sh.n;
+  const bool whole = ncand > kDrawCands;
+  const int items = whole ? nloc : ncand;
+  for (int i0 = 0; i0 < items; i0 += SETS) {                 // block-uniform trip count
+    const int i = i0 + set;
+    const int gl = i < items ? (whole ? i : sh.list[i]) : -1;
+    uint4 qt = neg_inf_vec<T>(), qd = bonus ? make_uint4(0, 0, 0, 0) : neg_inf_vec<T>();
+    if (gl >= 0) {
+      qt = load_logits<T>(tp, (gs + gl) * kGroup + sub * VEC, a.V, vec_ok);
+      if (!bonus) qd = load_logits<T>(dp, (gs + gl) * kGroup + sub * VEC, a.V, vec_ok);
+    }
+    const float key = group_key<T>(qt, qd, st, gl >= 0 ? s_u[gl] : 0.f, gl >= 0);
+    if (key != pos_inf() && (key < sk || (key == sk && gs + gl < sg))) {   // the whole lane set agrees
+      sk = key;
+      sg = gs + gl;
+      sh.qt[tid] = qt;
+      sh.qd[tid] = qd;
+    }
+  }
+  // the CTA's least (key, group), the lane set holding it, and its level-2
+  // winner, pushed to rank 0 of the cluster
+  float ck = sk;
+  int cgrp = sg;
+  key_min_cta(ck, cgrp, &sh.best[1]);
+  if (sub == 0 && cgrp != kIntMax && sk == ck && sg == cgrp) sh.hold = set;   // holders share one group
+  __syncthreads();
+  if (warp == 0) {
+    int tok = -1;
+    if (cgrp != kIntMax) {
+      const int h = sh.hold;
+      tok = race_group_entries<T>(sh.qt[h * LPG + sub], sh.qd[h * LPG + sub], cgrp, 0, lane, st, (uint32_t)b,
+                                  (uint32_t)pos, cw_ent, k0, k1);
+    }
+    if (lane == 0) {
+      *cl.map_shared_rank(&sh.rk[cr], 0) = ck;
+      *cl.map_shared_rank(&sh.rg[cr], 0) = cgrp;
+      *cl.map_shared_rank(&sh.rt[cr], 0) = tok;
+    }
+  }
+  cluster_sync();                             // every CTA's result is in rank 0
+  if (cr == 0) {
+    if (warp == 0) {
+      float k = lane < nc ? sh.rk[lane] : pos_inf();
+      const int g = lane < nc ? sh.rg[lane] : kIntMax;
+      const uint32_t kb = __reduce_min_sync(kFull, __float_as_uint(k));      // keys are >= 0 or +inf
+      const uint32_t gb = __reduce_min_sync(kFull, __float_as_uint(k) == kb ? (uint32_t)g : 0xFFFFFFFFu);
+      const unsigned who = __ballot_sync(kFull, __float_as_uint(k) == kb && (uint32_t)g == gb);
+      const int c = __ffs(who) - 1;
+      if (lane == 0) sh.fb = (gb == (uint32_t)kIntMax || sh.rt[c] < 0) ? -1 : sh.rt[c];
+    }
+    __syncthreads();
+    int tok = sh.fb;
+    if (tok < 0) tok = row_argmax_cta<T, NT>(tp, a.V, vec_ok, &sh.am);   // empty residual: the argmax
+    if (tid == 0) a.out_tokens[(size_t)b * a.Ko + pos] = tok;
+  }
+}
+
+// The extra verifier row's argmax (PAPER rule, bonus row; lowest index), each
+// CTA a share of the row.
+template <typename T, int NT>
+__device__ void cluster_argmax(const StreamArgs& a, cg::cluster_group& cl, int nc, int cr, int b, int pos, const T* tp,
+                               DrawShared<T, NT>& sh) {
+  constexpr int VEC = Elem<T>::kVec;
+  const int tid = threadIdx.x;
+  const bool vec_ok = (((uintptr_t)tp) & 15) == 0;
+  const int nvec = (a.V + VEC - 1) / VEC;
+  const int per = (nvec + nc - 1) / nc;
+  const int j1 = min(nvec, (cr + 1) * per);
+  if (tid == 0) sh.am = 0ull;
+  float bm = -pos_inf();
+  int bi = kIntMax;
+  for (int j = cr * per + tid; j < j1; j += NT) {
+    const uint4 q = load_logits<T>(tp, j * VEC, a.V, vec_ok);
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) {
+      const float z = logit_at<T>(q, k);
+      if (j * VEC + k < a.V && (z > bm || (z == bm && j * VEC + k < bi))) {
+        bm = z;
+        bi = j * VEC + k;
+      }
+    }
+  }
+  __syncthreads();
+  const unsigned long long key = argmax_key_cta(bm, bi, &sh.am);
+  if (tid == 0) *cl.map_shared_rank(&sh.arg[cr], 0) = key;
+  cluster_sync();
+  if (cr == 0 && tid == 0) {
+    unsigned long long m = 0ull;
+    for (int c = 0; c < nc; ++c) m = max(m, sh.arg[c]);
+    a.out_tokens[(size_t)b * a.Ko + pos] = (int)~(uint32_t)m;
+  }
+}
+
+constexpr int kDrawThreads = 256;
+constexpr int kDrawUl = 4;
+constexpr size_t kDrawSmemMax = 200 * 1024;
+
+// The draw as a kernel of its own, for calls whose rows the streaming kernel
+// streams: a cluster of nc CTAs per sequence at a time.
+//
+// No griddepcontrol.wait at the top: a sequence's draw starts as soon as its
+// epilogue has released the record word (every read below follows that
+// acquire), while the streaming kernel may still be finishing other
+// sequences.  Its CTAs have all started (they trigger this launch at their
+// top), so it completes whatever this kernel does.
+//
+// Every sequence passes the same number of cluster barriers, whatever its
+// record says, so CTAs that disagree (one poll timed out) still meet at every
+// barrier: two (three when the call has a bonus row, whose race takes one
+// more).  A peer's slot written before one barrier is read only between it
+// and the next.
+template <typename T, bool SAMPLED>
+__global__ void __launch_bounds__(kDrawThreads, 4) draw_kernel(const StreamArgs a, int nc) {
+  constexpr int NT = kDrawThreads;
+  extern __shared__ __align__(16) unsigned char draw_smem[];
+  __shared__ unsigned s_word;            // the sequence's record word
+  DrawShared<T, NT>& sh = *reinterpret_cast<DrawShared<T, NT>*>(draw_smem);
+  float* s_u = reinterpret_cast<float*>(draw_smem + sizeof(DrawShared<T, NT>));
+  cg::cluster_group cl = cg::this_cluster();
+  const int cr = (int)cl.block_rank();
+  const int ncl = (int)(gridDim.x / (unsigned)nc);
+  const Workspace& W = a.ws;
+  cluster_arrive();
+  bool first = true;
+  for (int b = (int)(blockIdx.x / (unsigned)nc); b < a.B; b += ncl) {
+    if (threadIdx.x == 0) s_word = poll_record(rec_word(W, b), W.err);
+    __syncthreads();
+    if (first) cluster_wait();           // a peer's shared memory is written only once it has started
+    first = false;
+    const unsigned word = s_word;
+    const int kind = (int)((word >> 1) & 3u), pos = (int)(word >> 3);
+    const int r = b * a.K + pos;
+    const T* tp = (const T*)a.target + ((size_t)b * a.Kt + pos) * (size_t)a.V;
+    if (kind == kSeqNone) {
+      cluster_sync();
+    } else if (!SAMPLED) {
+      cluster_argmax<T, NT>(a, cl, nc, cr, b, pos, tp, sh);
+    } else {
+      const bool bonus = kind == kSeqBonus;
+      float2 ts = make_float2(0.f, 1.f), ds = ts;
+      if (!bonus) {
+        ts = __ldcg(W.row_tstat + r);
+        ds = __ldcg(W.row_dstat + r);
+      }
+      const T* dp = bonus ? tp : (const T*)a.draft + (size_t)r * (size_t)a.V;
+      cluster_draw<T, NT, kDrawUl>(a, cl, nc, cr, b, pos, bonus, tp, dp, ts, ds, s_u, sh);
+    }
+    // the barriers that the branch above did not take
+    if (kind == kSeqNone || !SAMPLED) cluster_sync();
+    if (SAMPLED && a.bonus && kind != kSeqBonus) cluster_sync();
+    if (cr == 0 && threadIdx.x == 0) *rec_word(W, b) = 0u;   // every CTA of the cluster has read it
+  }
+  // this grid completes only after the streaming grid (whatever comes next on
+  // the stream then sees both)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
+// the residual draw with its share staged (few sequences, no bonus row)
+// ---------------------------------------------------------------------------
+//
+// The same draw by a cluster of kCluCtas CTAs of 512 threads, the share of the
+// target row copied to shared memory (cp.async, all of it in flight at once)
+// while the share's uniforms are drawn: the shorter chain, where every
+// sequence's cluster can be resident (B=64 K=8 V=128256: 54.6 us a step
+// against 56.3 with draw_kernel).
+constexpr int kCluCtas = 4;                  // CTAs per row (one cluster)
+constexpr int kCluThreads = 512;
+constexpr int kCluWarps = kCluThreads / 32;
+constexpr int kCluCands = 1024;                          // candidate list; past it the share is raced whole
+constexpr size_t kCluSmemMax = 200 * 1024;               // larger shares take the race over every group
+// Groups per CTA: a multiple of four, so that a share starts on a block of
+// four group uniforms.
+__host__ __device__ inline int clu_share(int ng) {
+  const int s = (ng + kCluCtas - 1) / kCluCtas;
+  return (s + 3) & ~3;
+}
+// Dynamic shared memory of one CTA: the staged target share, the share's
+// uniforms and bounds, the candidate list.
 template <typename T>
-__global__ void __launch_bounds__(kCluThreads, CMSD_CLU_MIN_BLOCKS) resample_bound_kernel(const StreamArgs a) {
+__host__ __device__ inline size_t clu_smem_bytes(int V) {
+  const size_t ngs = (size_t)clu_share((V + kGroup - 1) / kGroup);
+  return ngs * kGroup * sizeof(T) + ngs * 2 * sizeof(float) + (size_t)kCluCands * sizeof(int);
+}
+
+// The staged share keeps group g's vectors in 16-byte slots g LPG .. g LPG +
+// LPG - 1, vector k in slot g LPG + ((k + rot(g)) mod LPG), rot(g) = g LPG / 8:
+// a thread that reads a whole group (one vector per load) and its neighbours
+// reading theirs then touch eight different 16-byte bank slots per quarter
+// warp.
+template <int LPG>
+__device__ __forceinline__ int clu_slot(int g, int k) {
+  return g * LPG + ((k + ((g * LPG) >> 3)) & (LPG - 1));
+}
+
+// The largest logit of staged group g.
+__device__ __forceinline__ float group_max(const unsigned char* stage, int g, const uint16_t*) {
+  const uint4* q = reinterpret_cast<const uint4*>(stage);
+  const uint4 a = q[clu_slot<4>(g, 0)], b = q[clu_slot<4>(g, 1)], c = q[clu_slot<4>(g, 2)], d = q[clu_slot<4>(g, 3)];
+  const uint32_t x = bmax2(bmax2(a.x, b.x), bmax2(c.x, d.x));
+  const uint32_t y = bmax2(bmax2(a.y, b.y), bmax2(c.y, d.y));
+  const uint32_t z = bmax2(bmax2(a.z, b.z), bmax2(c.z, d.z));
+  const uint32_t w = bmax2(bmax2(a.w, b.w), bmax2(c.w, d.w));
+  const uint32_t m = bmax2(bmax2(x, y), bmax2(z, w));
+  return fmaxf(bf_lo(m), bf_hi(m));
+}
+__device__ __forceinline__ float group_max(const unsigned char* stage, int g, const float*) {
+  const uint4* q = reinterpret_cast<const uint4*>(stage);
+  float m = -pos_inf();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) m = fmaxf(m, vec_max(q[clu_slot<8>(g, k)], (const float*)nullptr));
+  return m;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCluThreads, 2) resample_bound_kernel(const StreamArgs a) {
   constexpr int VEC = Elem<T>::kVec;
   constexpr int LPG = kGroup / VEC;      // lanes per group
   constexpr int GPI = 32 / LPG;          // lane sets per warp
@@ -2138,6 +2452,72 @@ cudaError_t launch_resample_one(const StreamArgs& a, int grid, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, resample_kernel<T, SAMPLED>, a);
 }
 
+// The draw kernel: `clusters` clusters of nc CTAs, launched the same way (the
+// row loop covers any number of sequences).
+template <typename T>
+size_t draw_kernel_smem(int V, int nc) {
+  return sizeof(DrawShared<T, kDrawThreads>) + draw_smem_bytes(V, nc);
+}
+template <typename T, bool SAMPLED>
+cudaError_t draw_attrs() {
+  static unsigned long long done = 0ull;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (__atomic_load_n(&done, __ATOMIC_ACQUIRE) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(draw_kernel<T, SAMPLED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDrawSmemMax);
+  if (e == cudaSuccess) __atomic_fetch_or(&done, bit, __ATOMIC_ACQ_REL);
+  return e;
+}
+inline void draw_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int clusters, int nc, size_t smem) {
+  cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * nc));
+  cfg.blockDim = dim3(kDrawThreads);
+  cfg.dynamicSmemBytes = smem;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)nc;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+}
+template <typename T, bool SAMPLED>
+cudaError_t launch_draw_one(const StreamArgs& a, int clusters, int nc, cudaStream_t s) {
+  const cudaError_t e = draw_attrs<T, SAMPLED>();
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  draw_config(cfg, attr, clusters, nc, draw_kernel_smem<T>(a.V, nc));
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, draw_kernel<T, SAMPLED>, a, nc);
+}
+template <typename T>
+cudaError_t launch_draw_t(bool sampled, const StreamArgs& a, int clusters, int nc, cudaStream_t s) {
+  return sampled ? launch_draw_one<T, true>(a, clusters, nc, s) : launch_draw_one<T, false>(a, clusters, nc, s);
+}
+
+// Clusters of nc CTAs of the draw kernel that can be resident on the current
+// device for rows of V entries (0: none, or the share does not fit; the race
+// over every group then draws).
+template <typename T>
+int draw_clusters_t(int V, int nc) {
+  const size_t smem = draw_kernel_smem<T>(V, nc);
+  if (smem > kDrawSmemMax || draw_attrs<T, true>() != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  draw_config(cfg, attr, 1, nc, smem);
+  cfg.numAttrs = 1;                      // the cluster size
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, draw_kernel<T, true>, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();            // a refused query leaves no error behind for the caller
+    return 0;
+  }
+  return n;
+}
+
 // The residual draw by group bounds: `clusters` clusters of kCluCtas CTAs,
 // launched the same way (the row loop covers any number of queued rows).
 template <typename T>
@@ -2169,42 +2549,34 @@ cudaError_t launch_resample_bound_t(const StreamArgs& a, int clusters, cudaStrea
   return cudaLaunchKernelEx(&cfg, resample_bound_kernel<T>, a);
 }
 
-// Whether the residual draw by group bounds takes rows of V entries on the
-// current device: the share fits kCluSmemMax, and a cluster of kCluCtas CTAs
-// with that much shared memory can be resident (answer cached per device and
-// size).  Otherwise resample_kernel draws the residual.
+// Clusters of the staged residual draw that can be resident on the current
+// device for rows of V entries (0: the share does not fit, or none).
 template <typename T>
-bool resample_bound_fits_t(int V) {
+int resample_bound_clusters_t(int V) {
   const size_t smem = clu_smem_bytes<T>(V);
-  if (smem > kCluSmemMax) return false;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  static std::mutex mu;
-  static std::map<std::pair<int, size_t>, bool> cache;
-  std::lock_guard<std::mutex> lk(mu);
-  const auto key = std::make_pair(dev, smem);
-  const auto it = cache.find(key);
-  if (it != cache.end()) return it->second;
-  bool ok = false;
+  if (smem > kCluSmemMax) return 0;
   if (cudaFuncSetAttribute(resample_bound_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kCluSmemMax) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kCluCtas);
-    cfg.blockDim = dim3(kCluThreads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kCluCtas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    ok = cudaOccupancyMaxActiveClusters(&n, resample_bound_kernel<T>, &cfg) == cudaSuccess && n > 0;
+                           (int)kCluSmemMax) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
   }
-  if (!ok) (void)cudaGetLastError();   // a refused query leaves no error behind for the caller
-  cache.emplace(key, ok);
-  return ok;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCluCtas);
+  cfg.blockDim = dim3(kCluThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kCluCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, resample_bound_kernel<T>, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();   // a refused query leaves no error behind for the caller
+    return 0;
+  }
+  return n;
 }
 
 template <typename T>
