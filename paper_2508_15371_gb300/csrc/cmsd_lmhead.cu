@@ -77,7 +77,6 @@ __device__ __forceinline__ void fold32(DLane& st, const float* z_src, int v0, in
     st.pos = up ? v0 + k : st.pos;
     st.m = up ? z[k] : st.m;
   }
-  st.posw = 1;
   // one reference check, then the exponentials, summed among themselves
   const float me = d_mexp(st);
   if (me > st.ref + kRefSlack) d_reref(st, me);

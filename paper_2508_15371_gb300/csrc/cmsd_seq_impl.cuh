@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     pipe_run<T, MODE, SAMPLED>(pp, ss, sg.va, beta, lane);
     DRed dr;
     TRed tr;
-    seg_reduce<T, MODE, SAMPLED>(ss, !SAMPLED || a.argmax != nullptr, !SAMPLED, dp, tp, dr, tr);
+    seg_reduce<T, MODE, SAMPLED>(ss, sg, !SAMPLED || a.argmax != nullptr, dp, tp, dr, tr);
     if (first) cluster_wait();         // every CTA of the cluster has started
     first = false;
     if (lane == 0) {

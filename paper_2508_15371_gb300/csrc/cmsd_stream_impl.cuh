@@ -101,7 +101,7 @@ struct DLane {               // drafter
   float t, ct;               // sum of e*x, and its compensation
   float f1, f2;              // top-2 of elements taken one at a time (all f32 data)
   uint32_t T1, T2;           // top-2 of bf16 vector elements, per half-word lane
-  int pos, posw;             // first unit (start, width) that reached m
+  int pos;                   // start of the first vector (or the element) that reached m
 };
 
 struct TLane {               // target
@@ -110,7 +110,7 @@ struct TLane {               // target
   u64 negrL;
   float s, cs;               // sum of e^(z - ref), and its compensation
   float thr;                 // PAPER rule: elements above thr may be counted
-  int pos, posw;
+  int pos;                   // as the drafter's (PAPER rule)
   int cnt;
 };
 
@@ -122,7 +122,6 @@ __device__ __forceinline__ void dlane_init(DLane& d) {
   d.f1 = d.f2 = kNegInit;
   d.T1 = d.T2 = kNegInf2;
   d.pos = kIntMax;
-  d.posw = 0;
 }
 __device__ __forceinline__ void tlane_init(TLane& t, float c, int beta) {
   t.M = kNegInit;
@@ -130,7 +129,6 @@ __device__ __forceinline__ void tlane_init(TLane& t, float c, int beta) {
   t.negrL = dup2(-mlog2e(kNegInit));
   t.s = t.cs = 0.f;
   t.pos = kIntMax;
-  t.posw = 0;
   t.cnt = 0;
   t.thr = pos_inf();
   if (beta > 0) t.thr = c;   // c is a pending load: read it only when needed
@@ -174,7 +172,7 @@ __device__ __forceinline__ void t_reref(TLane& t, float mx) {
 __device__ __forceinline__ void d_scalar(DLane& d, float z, int v) {
   d.f2 = fmaxf(d.f2, fminf(d.f1, z));
   d.f1 = fmaxf(d.f1, z);
-  if (z > d.m || (z == d.m && v < d.pos)) { d.pos = v; d.posw = 1; }
+  if (z > d.m || (z == d.m && v < d.pos)) d.pos = v;
   d.m = fmaxf(d.m, z);
   const float me = d_mexp(d);
   if (me > d.ref + kRefSlack) d_reref(d, me);
@@ -195,7 +193,6 @@ __device__ __forceinline__ void d_vmax(DLane& d, uint4 q, int v) {
   const float mx = fmaxf(bf_lo(d.T1), bf_hi(d.T1));
   const bool up = mx > d.m;
   d.pos = up ? v : d.pos;
-  d.posw = up ? 8 : d.posw;
   d.m = fmaxf(d.m, mx);
 }
 __device__ __forceinline__ void d_vmax(DLane& d, float4 q, int v) {
@@ -207,7 +204,6 @@ __device__ __forceinline__ void d_vmax(DLane& d, float4 q, int v) {
   }
   const bool up = d.f1 > d.m;
   d.pos = up ? v : d.pos;
-  d.posw = up ? 4 : d.posw;
   d.m = fmaxf(d.m, d.f1);
 }
 
@@ -235,7 +231,7 @@ __device__ __forceinline__ void d_vexp(const DLane& d, float4 q, u64& ss, u64& t
 // --- target -----------------------------------------------------------------------
 template <bool SAMPLED>
 __device__ __forceinline__ void t_scalar(TLane& t, float z, int v, float c, int beta) {
-  if (z > t.M || (z == t.M && v < t.pos)) { t.pos = v; t.posw = 1; }
+  if (!SAMPLED && (z > t.M || (z == t.M && v < t.pos))) t.pos = v;
   t.M = fmaxf(t.M, z);
   if (t.cnt < beta && z > c) ++t.cnt;
   if (SAMPLED) {
@@ -244,13 +240,12 @@ __device__ __forceinline__ void t_scalar(TLane& t, float z, int v, float c, int 
   }
 }
 
+template <bool SAMPLED>
 __device__ __forceinline__ void t_vmax(TLane& t, uint4 q, int v, float c, int beta) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
   const uint32_t a = bmax2(bmax2(w[0], w[1]), bmax2(w[2], w[3]));
   const float vmax = fmaxf(bf_lo(a), bf_hi(a));
-  const bool up = vmax > t.M;
-  t.pos = up ? v : t.pos;
-  t.posw = up ? 8 : t.posw;
+  if (!SAMPLED) t.pos = vmax > t.M ? v : t.pos;
   t.M = fmaxf(t.M, vmax);
   if (vmax > t.thr) {          // PAPER rule, rank gate: count logits above the draft's
 #pragma unroll
@@ -258,12 +253,11 @@ __device__ __forceinline__ void t_vmax(TLane& t, uint4 q, int v, float c, int be
     if (t.cnt >= beta) t.thr = pos_inf();
   }
 }
+template <bool SAMPLED>
 __device__ __forceinline__ void t_vmax(TLane& t, float4 q, int v, float c, int beta) {
   const float z[4] = {q.x, q.y, q.z, q.w};
   const float vmax = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));
-  const bool up = vmax > t.M;
-  t.pos = up ? v : t.pos;
-  t.posw = up ? 4 : t.posw;
+  if (!SAMPLED) t.pos = vmax > t.M ? v : t.pos;
   t.M = fmaxf(t.M, vmax);
   if (vmax > t.thr) {
     t.cnt += (z[0] > c) + (z[1] > c) + (z[2] > c) + (z[3] > c);
@@ -796,7 +790,7 @@ struct SegState {
 
 // The warp's statistics of the segment its lanes have reduced, in every lane.
 template <typename T, int MODE, bool SAMPLED>
-__device__ __forceinline__ void seg_reduce(const SegState& ss, bool want_didx, bool want_tidx, const T* dp, const T* tp,
+__device__ __forceinline__ void seg_reduce(const SegState& ss, const Seg& sg, bool want_didx, const T* dp, const T* tp,
                                            DRed& dr, TRed& tr) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
@@ -804,25 +798,25 @@ __device__ __forceinline__ void seg_reduce(const SegState& ss, bool want_didx, b
   // that vector again.  Under the sampled rule only the lanes holding the
   // segment maximum request it (one sector each, usually one lane; this saved
   // 19 MB of the 263 MB per launch at B=64 K=8 V=128256 and 2 us).  Under the
-  // PAPER rule every lane requests its vector before the warp reductions, so
+  // PAPER rule (the only one that needs the target's index) every lane
+  // requests its vector before the warp reductions, so
   // the loads overlap the shuffles: there the kernel's tail is this latency,
   // and the early requests measured 3 us faster than the late ones.
   // Without a wanted index a lane's vector start stands in (distinct per lane
   // and ordered like the index, so the merges still tell the maximum's lane
   // from a duplicate of its value) and nothing is re-read.
   const float me = HAS_D ? d_mexp(ss.d) : 0.f;
+  const bool dvec = HAS_D && ss.d.pos >= sg.va && ss.d.pos < sg.vb;   // (a vector's start, not an element)
+  const bool tvec = HAS_T && !SAMPLED && ss.t.pos >= sg.va && ss.t.pos < sg.vb;
   uint4 dq = make_uint4(0, 0, 0, 0), tq = make_uint4(0, 0, 0, 0);
   if (!SAMPLED) {
-    if (HAS_D && ss.d.posw > 1) dq = __ldcg(reinterpret_cast<const uint4*>(dp + ss.d.pos));
-    if (HAS_T && ss.t.posw > 1) tq = __ldcg(reinterpret_cast<const uint4*>(tp + ss.t.pos));
+    if (dvec) dq = __ldcg(reinterpret_cast<const uint4*>(dp + ss.d.pos));
+    if (tvec) tq = __ldcg(reinterpret_cast<const uint4*>(tp + ss.t.pos));
   }
   const float Md = HAS_D ? warp_max(me) : 0.f;
   const float Mt = HAS_T ? warp_max(ss.t.M) : 0.f;
-  const bool dhit = HAS_D && me == Md && ss.d.posw, thit = HAS_T && ss.t.M == Mt && ss.t.posw;
-  if (SAMPLED) {
-    if (want_didx && dhit && ss.d.posw > 1) dq = __ldcg(reinterpret_cast<const uint4*>(dp + ss.d.pos));
-    if (want_tidx && thit && ss.t.posw > 1) tq = __ldcg(reinterpret_cast<const uint4*>(tp + ss.t.pos));
-  }
+  const bool dhit = HAS_D && me == Md && ss.d.pos != kIntMax, thit = HAS_T && ss.t.M == Mt && ss.t.pos != kIntMax;
+  if (SAMPLED && want_didx && dhit && dvec) dq = __ldcg(reinterpret_cast<const uint4*>(dp + ss.d.pos));
   dr = dred_empty();
   tr = tred_empty();
   if (HAS_D) {
@@ -837,13 +831,13 @@ __device__ __forceinline__ void seg_reduce(const SegState& ss, bool want_didx, b
     float s, t2;
     d_final(d, s, t2);
     int idx = kIntMax;
-    if (dhit) idx = (want_didx && d.posw > 1) ? d.pos + first_in_vec<T>(dq, me, true) : d.pos;
+    if (dhit) idx = (want_didx && dvec) ? d.pos + first_in_vec<T>(dq, me, true) : d.pos;
     dr = reduce_d(DRed{me, s, t2, top2, idx});
   }
   if (HAS_T) {
     const TLane& t = ss.t;
     int idx = kIntMax;
-    if (thit) idx = (want_tidx && t.posw > 1) ? t.pos + first_in_vec<T>(tq, t.M, false) : t.pos;
+    if (!SAMPLED && thit) idx = tvec ? t.pos + first_in_vec<T>(tq, t.M, false) : t.pos;
     tr = reduce_t(TRed{t.M, SAMPLED ? t_final(t) : 0.f, idx, t.cnt});
   }
 }
@@ -852,17 +846,17 @@ __device__ __forceinline__ void seg_reduce(const SegState& ss, bool want_didx, b
 // publish the partial, and merge the row / run the sequence epilogue if this
 // warp completes them.
 template <typename T, int MODE, bool SAMPLED, bool PH2>
-__device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int b, int i, int len,
-                           const StreamSplit& sp, int w, int lane, const T* dp, const T* tp) {
+__device__ void seg_finish(const StreamArgs& a, SegState& ss, const Seg& sg, int len, const StreamSplit& sp, int w,
+                           int lane, const T* dp, const T* tp) {
+  const int ar = sg.ar, r = sg.r, b = sg.b, i = sg.i;
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
   const Workspace& W = a.ws;
-  // Under the sampled rule the exact indices feed only the drafter's argmax
-  // output and resample_kernel's empty-residual fallback (the bounded draw
-  // finds that argmax itself).
+  // Under the sampled rule the exact index feeds only the drafter's argmax
+  // output (an empty residual's draw finds the target's itself).
   DRed dr;
   TRed tr;
-  seg_reduce<T, MODE, SAMPLED>(ss, !SAMPLED || a.argmax != nullptr, !SAMPLED || !a.rec_by_seq, dp, tp, dr, tr);
+  seg_reduce<T, MODE, SAMPLED>(ss, sg, !SAMPLED || a.argmax != nullptr, dp, tp, dr, tr);
   // lane 0 stores the partial and counts it with a release; the warp that
   // completes the row sees every other slice's partial through the acquire
   // of its own count (extended to the other lanes by __syncwarp)
@@ -906,7 +900,6 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
       W.row_dstat[r] = o.ds;
       W.row_tstat[r] = o.ts;
     }
-    if (HAS_T) W.row_targmax[r] = tr.idx;
     W.row_done[r] = 0;
     if (packed) {
       const unsigned long long mine = 1ull | ((unsigned long long)(o.acc ? 1u : 0u) << (6 + i)) | (o.cfx << 22);
@@ -935,88 +928,128 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, int ar, int r, int
 // ---- one segment body, pipelined ----------------------------------------------
 // The lane's vectors of the aligned body [va, vb) are j = lane + 32 t,
 // t = 0, 1, ...; stage s holds t in [s*U, s*U + U) and is loaded (streaming,
-// no L1 allocation) while stage s-1 is reduced.
+// no L1 allocation) while stage s-1 is reduced.  Only the last stage can be
+// partial: its missing vectors read as -inf, which adds nothing.
 #ifndef CMSD_UNROLL
-#define CMSD_UNROLL 2
+#define CMSD_UNROLL 4
 #endif
+template <typename T>
+__device__ __forceinline__ uint4 neg_inf_vec() {
+  return sizeof(T) == 2 ? make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2)
+                        : make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u);
+}
 template <typename T, int U>
 struct Pipe {
-  uint4 d[U], t[U];                       // the stage in flight
-  const uint4* gd;
+  uint4 d[U], t[U];                       // the stage to reduce next
+  const uint4* gd;                        // the lane's vectors from that stage on
   const uint4* gt;
-  int nt, nst;                            // this lane's vectors; warp-uniform stages
+  int rem;                                // vectors of the body from that stage on (warp-uniform; may end below 0)
 };
 
-// issue the loads of stage 0
+// the U vectors at g; each lane's `left` says how many there are
+template <int U>
+__device__ __forceinline__ void load_full(const uint4* g, uint4 (&x)[U]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) x[u] = ld_stream(g + 32 * u);
+}
+template <typename T, int U>
+__device__ __forceinline__ void load_part(const uint4* g, int left, uint4 (&x)[U]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    x[u] = neg_inf_vec<T>();
+    if (32 * u < left) x[u] = ld_stream(g + 32 * u);
+  }
+}
+
+// the pipeline of a segment, its stage 0 requested
 template <typename T, int MODE, int U>
 __device__ __forceinline__ void pipe_start(Pipe<T, U>& p, const T* dp, const T* tp, int va, int vb, int lane) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
-  constexpr int VEC = Elem<T>::kVec;
-  const int nvec = (vb - va) / VEC;
-  p.nt = nvec > lane ? (nvec - lane + 31) / 32 : 0;
-  p.nst = (nvec + 32 * U - 1) / (32 * U);
+  const int nvec = (vb - va) / Elem<T>::kVec;
+  p.rem = nvec;
   p.gd = HAS_D ? reinterpret_cast<const uint4*>(dp + va) + lane : nullptr;
   p.gt = HAS_T ? reinterpret_cast<const uint4*>(tp + va) + lane : nullptr;
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    if (u < p.nt) {
-      if (HAS_D) p.d[u] = ld_stream(p.gd + 32 * u);
-      if (HAS_T) p.t[u] = ld_stream(p.gt + 32 * u);
-    }
-  }
+  if (HAS_D) load_part<T>(p.gd, nvec - lane, p.d);
+  if (HAS_T) load_part<T>(p.gt, nvec - lane, p.t);
 }
 
+// Reduce a lane's vectors of one stage, vector u at row entry v0 + 32 u VEC.
+template <typename T, int MODE, bool SAMPLED, int U>
+__device__ __forceinline__ void stage_reduce(SegState& ss, const uint4 (&d)[U], const uint4 (&t)[U], int v0, int beta) {
+  constexpr bool HAS_D = MODE != kModeVerify;
+  constexpr bool HAS_T = MODE != kModeConf;
+  constexpr int VEC = Elem<T>::kVec;
+  // maximum phase: running maxima, top-2, rank count
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int v = v0 + 32 * u * VEC;
+    if (HAS_D) d_vmax(ss.d, as_vec<T>(d[u]), v);
+    if (HAS_T) t_vmax<SAMPLED>(ss.t, as_vec<T>(t[u]), v, ss.c, beta);
+  }
+  // one reference check per stage, then the stage's exponentials
+  if (HAS_D) {
+    const float me = d_mexp(ss.d);
+    if (me > ss.d.ref + kRefSlack) d_reref(ss.d, me);
+  }
+  if (HAS_T && SAMPLED && ss.t.M > ss.t.ref + kRefSlack) t_reref(ss.t, ss.t.M);
+  u64 ds = 0ull, dt = 0ull, ts = 0ull;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (HAS_D) d_vexp(ss.d, as_vec<T>(d[u]), ds, dt);
+    if (HAS_T && SAMPLED) t_vexp(ss.t, as_vec<T>(t[u]), ts);
+  }
+  if (HAS_D) {
+    kahan(ss.d.s, ss.d.cs, lo32f(ds) + hi32f(ds));
+    kahan(ss.d.t, ss.d.ct, lo32f(dt) + hi32f(dt));
+  }
+  if (HAS_T && SAMPLED) kahan(ss.t.s, ss.t.cs, lo32f(ts) + hi32f(ts));
+}
+
+// Whole stages two at a time, each in registers of its own (a copy of the
+// loaded stage into the one to reduce would wait for its loads) and without a
+// condition on any load; the last few one at a time.  Against one guarded loop
+// with a copy, B=64 K=8 V=128256 bf16, sampled: 28.3 M warp instructions
+// instead of 38.3 M, and the slices end 37 us into the launch instead of 40.
+// Refilling each vector as soon as it had been used was slower (8.7 against
+// 7.7 us at B=8 K=8 V=32128).
 template <typename T, int MODE, bool SAMPLED, int U>
 __device__ __forceinline__ void pipe_run(Pipe<T, U>& p, SegState& ss, int va, int beta, int lane) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
   constexpr int VEC = Elem<T>::kVec;
+  constexpr int SV = 32 * U;               // vectors per stage
+  uint4 d[U], t[U];
+  int v = va + lane * VEC;
 #pragma unroll 1
-  for (int s = 0; s < p.nst; ++s) {
-    uint4 nd[U], nx[U];
-    const int t1 = (s + 1) * U;
+  while (p.rem >= 3 * SV) {
+    if (HAS_D) load_full(p.gd + SV, d);
+    if (HAS_T) load_full(p.gt + SV, t);
+    stage_reduce<T, MODE, SAMPLED, U>(ss, p.d, p.t, v, beta);
+    if (HAS_D) load_full(p.gd + 2 * SV, p.d);
+    if (HAS_T) load_full(p.gt + 2 * SV, p.t);
+    stage_reduce<T, MODE, SAMPLED, U>(ss, d, t, v + SV * VEC, beta);
+    v += 2 * SV * VEC;
+    if (HAS_D) p.gd += 2 * SV;
+    if (HAS_T) p.gt += 2 * SV;
+    p.rem -= 2 * SV;
+  }
+#pragma unroll 1
+  while (p.rem > 0) {
+    p.rem -= SV;
+    if (HAS_D) p.gd += SV;
+    if (HAS_T) p.gt += SV;
+    if (p.rem > 0) {
+      if (HAS_D) load_part<T>(p.gd, p.rem - lane, d);
+      if (HAS_T) load_part<T>(p.gt, p.rem - lane, t);
+    }
+    stage_reduce<T, MODE, SAMPLED, U>(ss, p.d, p.t, v, beta);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (t1 + u < p.nt) {
-        if (HAS_D) nd[u] = ld_stream(p.gd + 32 * (t1 + u));
-        if (HAS_T) nx[u] = ld_stream(p.gt + 32 * (t1 + u));
-      }
+      if (HAS_D) p.d[u] = d[u];
+      if (HAS_T) p.t[u] = t[u];
     }
-    const int t0 = s * U;
-    // maximum phase: running maxima, top-2, rank count
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (t0 + u < p.nt) {
-        const int v = va + (lane + 32 * (t0 + u)) * VEC;
-        if (HAS_D) d_vmax(ss.d, as_vec<T>(p.d[u]), v);
-        if (HAS_T) t_vmax(ss.t, as_vec<T>(p.t[u]), v, ss.c, beta);
-      }
-    }
-    // one reference check per stage, then the stage's exponentials
-    if (HAS_D) {
-      const float me = d_mexp(ss.d);
-      if (me > ss.d.ref + kRefSlack) d_reref(ss.d, me);
-    }
-    if (HAS_T && SAMPLED && ss.t.M > ss.t.ref + kRefSlack) t_reref(ss.t, ss.t.M);
-    u64 ds = 0ull, dt = 0ull, ts = 0ull;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (t0 + u < p.nt) {
-        if (HAS_D) d_vexp(ss.d, as_vec<T>(p.d[u]), ds, dt);
-        if (HAS_T && SAMPLED) t_vexp(ss.t, as_vec<T>(p.t[u]), ts);
-      }
-    }
-    if (HAS_D) {
-      kahan(ss.d.s, ss.d.cs, lo32f(ds) + hi32f(ds));
-      kahan(ss.d.t, ss.d.ct, lo32f(dt) + hi32f(dt));
-    }
-    if (HAS_T && SAMPLED) kahan(ss.t.s, ss.t.cs, lo32f(ts) + hi32f(ts));
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (HAS_D) p.d[u] = nd[u];
-      if (HAS_T) p.t[u] = nx[u];
-    }
+    v += SV * VEC;
   }
 }
 
@@ -1068,7 +1101,7 @@ __device__ void walk_slice(const StreamArgs& a, const int* s_pref, int64_t e_beg
       if (HAS_D) d_scalar(ss.d, Elem<T>::load(dp + v), v);
       if (HAS_T) t_scalar<SAMPLED>(ss.t, Elem<T>::load(tp + v), v, ss.c, beta);
     }
-    seg_finish<T, MODE, SAMPLED, PH2>(a, ss, sg.ar, sg.r, sg.b, sg.i, len, sp, w, lane, dp, tp);
+    seg_finish<T, MODE, SAMPLED, PH2>(a, ss, sg, len, sp, w, lane, dp, tp);
   }
 }
 
@@ -1178,12 +1211,6 @@ __device__ __forceinline__ uint4 load_logits(const T* p, int v, int V, bool vec_
     for (int k = 0; k < 4; ++k) w[k] = (v + k < V) ? __ldg(q + v + k) : 0xFF800000u;
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-template <typename T>
-__device__ __forceinline__ uint4 neg_inf_vec() {
-  return sizeof(T) == 2 ? make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2)
-                        : make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u);
 }
 
 // Level 2 on group gm, whose logits sit in lanes own .. own+LPG-1 (vector
@@ -1319,6 +1346,28 @@ __device__ __forceinline__ uint4 staged_vec(const unsigned char* stage, const T*
   const int j = (g - gc) * LPG + sub;
   if (j < nfull) return *reinterpret_cast<const uint4*>(stage + 16 * j);
   return load_logits<T>(row, g * kGroup + sub * VEC, V, false);
+}
+
+// The verifier row's argmax (the lowest index of its largest logit), by one
+// warp from global memory: the token of a row whose residual is empty.
+template <typename T>
+__device__ int row_argmax_warp(const T* tp, int V, bool vec_ok, int lane) {
+  constexpr int VEC = Elem<T>::kVec;
+  float bm = -pos_inf();
+  int bi = kIntMax;
+  for (int v = lane * VEC; v < V; v += 32 * VEC) {
+    const uint4 q = load_logits<T>(tp, v, V, vec_ok);
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) {
+      const float z = logit_at<T>(q, k);
+      if (v + k < V && z > bm) {
+        bm = z;
+        bi = v + k;
+      }
+    }
+  }
+  const float m = warp_max(bm);
+  return warp_min_i(bm == m ? bi : kIntMax);
 }
 
 template <typename T, bool SAMPLED>
@@ -1548,10 +1597,10 @@ __global__ void __launch_bounds__(kResThreads, CMSD_RES_MIN_BLOCKS) resample_ker
           const float km = warp_min(key);
           const int gm = warp_min_i(key == km ? gw_ : kIntMax);
           const int tm = warp_min_i((key == km && gw_ == gm && tw >= 0) ? tw : kIntMax);
+          int out = tm;
+          if (gm == kIntMax || tm == kIntMax) out = row_argmax_warp<T>(tp, a.V, vec_ok, lane);   // empty residual
           if (lane == 0) {
             W.res_done[rr] = 0;
-            int out = tm;
-            if (gm == kIntMax || tm == kIntMax) out = __ldcg(W.row_targmax + r);   // empty residual: argmax
             a.out_tokens[(size_t)b * a.Ko + pos] = out;
           }
         }
