@@ -137,13 +137,21 @@ def params(K, rule="paper", preset="full", **kw):
     return p
 
 
+_torch_mod = None
+_raw_stream = None      # (device index) -> cudaStream_t of the current stream, without a Stream object
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_mod, _raw_stream
+    if _torch_mod is None:
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch_mod = torch
+    return _torch_mod
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dtype_code(t):
@@ -163,16 +171,19 @@ def _check_target(draft, target, p):
 
 
 def _stream():
-    torch = _torch()
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    torch = _torch_mod or _torch()
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _need_cuda(*ts):
     for t in ts:
-        if t is not None and not t.is_cuda:
-            raise CmsdError("all tensors must be CUDA tensors (the library has no CPU path)")
-        if t is not None and not t.is_contiguous():
-            raise CmsdError("tensors must be contiguous")
+        if t is not None:
+            if not t.is_cuda:
+                raise CmsdError("all tensors must be CUDA tensors (the library has no CPU path)")
+            if not t.is_contiguous():
+                raise CmsdError("tensors must be contiguous")
 
 
 _ws_cache = {}
@@ -204,12 +215,11 @@ def workspace_errors(ws):
 
 
 def _out(out, name, shape, dtype, device, want=True):
-    torch = _torch()
     if out is not None and name in out:
         return out[name]
     if not want:
         return None
-    return torch.empty(shape, dtype=dtype, device=device)
+    return _torch().empty(shape, dtype=dtype, device=device)
 
 
 def confidence(draft, k_row=None, p=None, out=None, ws=None):

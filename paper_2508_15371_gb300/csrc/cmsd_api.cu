@@ -5,6 +5,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -29,7 +30,6 @@ std::mutex g_mu;
 std::map<int, int> g_sms;                                   // device -> SM count
 std::map<std::tuple<int, int, int, int, int>, int> g_occ;   // (dev, dtype, mode, variant, smem) -> blocks/SM
 std::map<std::tuple<int, int, int, int>, int> g_draw_res;    // (dev, dtype, V, CTAs) -> resident clusters
-std::map<std::tuple<int, int, int, int>, int> g_seq_res;     // (dev, dtype, CTAs, threads) -> resident clusters
 std::map<std::tuple<int, int, int>, int> g_occ_res;          // (dev, dtype, sampled) -> blocks/SM
 
 int device_sms(int* sms) {
@@ -233,18 +233,21 @@ void fill_sizes(StreamArgs& a, int B, int K, int V) {
   a.soft_norm = (float)(1.0 / (1.0 - 1.0 / (double)V));
 }
 
-// Clusters of seq_kernel that can be resident on the current device (cached).
-int seq_resident(int dtype, int nc, int threads) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  const auto key = std::make_tuple(dev, dtype, nc, threads);
-  std::lock_guard<std::mutex> lk(g_mu);
-  auto it = g_seq_res.find(key);
-  if (it == g_seq_res.end()) {
-    const int n = dtype == CMSD_F32 ? seq_clusters_f32(nc, threads) : seq_clusters_bf16(nc, threads);
-    it = g_seq_res.emplace(key, n).first;
+// CTAs per cluster that choose_seq weighs.
+constexpr int kSeqSizes[] = {1, 2, 4, 5, 8, 16};
+constexpr int kSeqNumSizes = 6;
+
+// Clusters of seq_kernel that can be resident on device dev, which is current
+// (cached; n: index into kSeqSizes).
+int seq_resident(int dev, int dtype, int n, int threads) {
+  static std::atomic<int> known[64][2][2][kSeqNumSizes];   // 0: not asked yet, else the answer + 1
+  std::atomic<int>& k = known[dev & 63][dtype][threads == 512][n];
+  int v = dev < 64 ? k.load(std::memory_order_relaxed) : 0;
+  if (v == 0) {
+    v = 1 + (dtype == CMSD_F32 ? seq_clusters_f32(kSeqSizes[n], threads) : seq_clusters_bf16(kSeqSizes[n], threads));
+    if (dev < 64) k.store(v, std::memory_order_relaxed);
   }
-  return it->second;
+  return v - 1;
 }
 
 // Which kernel takes a call: the one-launch pass with *nc CTAs of *threads
@@ -274,16 +277,18 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
   }
   const double rate = mode == kModeVerify ? 30 : (mode == kModeFused && !sampled ? 27 : 21);
   const double fixed = 5 + (second ? 4.5 : 0);
-  static const int sizes[] = {1, 2, 4, 5, 8, 16};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
   double best = 0.97 * flat;               // (a near tie stays with the streaming kernel)
   *nc = 0;
   for (int th = 256; th <= 512; th *= 2) {
-    for (int n : sizes) {
+    for (int k = 0; k < kSeqNumSizes; ++k) {
+      const int n = kSeqSizes[k];
       // at least two 16-byte vectors per lane and piece, or more CTAs gain nothing
       if (n > 1 && kb * 1e3 < (double)n * (th / 32) * 1024 * (mode == kModeFused ? 2 : 1)) break;
       const double part = kb / n / (rate * (th / 256));
       if (fixed + part >= best) continue;
-      const int res = seq_resident(dtype, n, th);
+      const int res = seq_resident(dev, dtype, k, th);
       if (res < 1) continue;
       // (clusters of 4 and more were not all placed at once near the limit)
       const int fit = n >= 4 ? (res * 9 + 9) / 10 : res;
