@@ -6,8 +6,8 @@
 // weight, and reads from each logit row the entropy, logit margin and softmax
 // margin of Sec. III.B(1).  Here the product runs on the 5th-generation
 // tensor cores (tcgen05.mma, bf16 in, fp32 accumulators in tensor memory) and
-// each finished tile of 128 vocabulary entries x 64 hidden rows is folded, in
-// the GEMM's epilogue, into per-row running statistics: running maximum and
+// each finished tile of 128 vocabulary entries is folded, in the GEMM's
+// epilogue, into per-row running statistics: running maximum and
 // its first index, second largest logit, and compensated sums of e^(z - ref)
 // and e^(z - ref)(z - ref) log2 e against a lazily moved exponent reference
 // (the same arithmetic as the logits pass).  The logits never reach HBM
@@ -17,15 +17,22 @@
 //
 // Layout: hidden [R][d] and weight [V][d] row-major bf16 (the usual
 // [out][in] layout of a linear layer's weight), d a multiple of 64.  Each CTA
-// owns a contiguous run of the vocabulary for one block of 64 hidden rows and
+// owns a contiguous run of the vocabulary for one block of hidden rows and
 // streams its weight rows once through a ring of shared-memory stages filled
 // by 2D tensor-memory-access (TMA) loads: per stage one box of 64 hidden
-// dimensions x 128 weight rows (the MMA's A) and one of 64 x 64 hidden rows
-// (its B), both with the 128-byte swizzle that the MMA's shared-memory
-// descriptors name; rows past R or V arrive as zeros.  The hidden block is
-// re-read from L2 for every tile.
+// dimensions x 128 weight rows and the same dimensions of the hidden rows, both
+// with the 128-byte swizzle that the MMA's shared-memory descriptors name; rows
+// past R or V arrive as zeros.  The hidden block is re-read from L2 for every
+// tile.
+//
+// Bounds, on a GB300: up to 128 hidden rows DRAM (R=64 d=2048 V=128256: 525.6 MB
+// in 89 us, 5.9 TB/s); at 256 rows the MMAs, whose operands take the shared
+// memory's bandwidth (109 us, 1.23 PFLOP/s; 131 us when the epilogue transposed
+// every tile); small calls the launch, the fill of the ring and the merge
+// kernel (R=16 d=1024 V=32000: 19.2 us for 65.6 MB).
 #include <cuda.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "cmsd_stream_impl.cuh"
@@ -45,6 +52,17 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// the same box into every CTA of the cluster named in `mask`: at the same
+// shared offset, completing the barrier at the same offset
+__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar,
+                                               uint16_t mask) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
+      "[%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
+      : "memory");
+}
+
 // The vocabulary run of CTA `cta` of a row block: nct near-equal runs of
 // 8 entries ([v0, v1), v1 <= V).
 __device__ __forceinline__ void cta_run(int V, int nct, int cta, int& v0, int& v1) {
@@ -57,25 +75,42 @@ __device__ __forceinline__ void cta_run(int V, int nct, int cta, int& v0, int& v
 
 // Fold 32 consecutive logits (vocabulary entries v0 .. v0+31, those at or
 // past vend masked) into a thread's running drafter statistics.
-__device__ __forceinline__ void fold32(DLane& st, const float* z_src, int v0, int vend) {
-  float z[32];
+__device__ __forceinline__ void fold32(DLane& st, float (&z)[32], int v0, int vend) {
+  if (v0 + 32 > vend) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float4 q = *reinterpret_cast<const float4*>(z_src + 4 * k);
-    z[4 * k] = q.x; z[4 * k + 1] = q.y; z[4 * k + 2] = q.z; z[4 * k + 3] = q.w;
+    for (int k = 0; k < 32; ++k)
+      if (v0 + k >= vend) z[k] = -pos_inf();
+  }
+  // top-2 of the 32 in four independent chains, then with the lane's so far
+  float a1[4], a2[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    a1[c] = z[8 * c];
+    a2[c] = kNegInit;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+      a2[c] = fmaxf(a2[c], fminf(a1[c], z[8 * c + k]));
+      a1[c] = fmaxf(a1[c], z[8 * c + k]);
+    }
   }
 #pragma unroll
-  for (int k = 0; k < 32; ++k)
-    if (v0 + k >= vend) z[k] = -pos_inf();
-  // maxima: top-2 and the first index of the running maximum (entries come
-  // in increasing index order, so a strict increase keeps the lowest index)
+  for (int o = 2; o; o >>= 1) {
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    st.f2 = fmaxf(st.f2, fminf(st.f1, z[k]));
-    st.f1 = fmaxf(st.f1, z[k]);
-    const bool up = z[k] > st.m;
-    st.pos = up ? v0 + k : st.pos;
-    st.m = up ? z[k] : st.m;
+    for (int c = 0; c < o; ++c) {
+      a2[c] = fmaxf(fmaxf(a2[c], a2[c + o]), fminf(a1[c], a1[c + o]));
+      a1[c] = fmaxf(a1[c], a1[c + o]);
+    }
+  }
+  st.f2 = fmaxf(fmaxf(st.f2, a2[0]), fminf(st.f1, a1[0]));
+  st.f1 = fmaxf(st.f1, a1[0]);
+  // entries come in increasing index order, so a strict increase keeps the
+  // lowest index; the first entry equal to the new maximum is its index
+  if (a1[0] > st.m) {
+    int k0 = 0;
+#pragma unroll
+    for (int k = 31; k >= 0; --k) k0 = z[k] == a1[0] ? k : k0;
+    st.pos = v0 + k0;
+    st.m = a1[0];
   }
   // one reference check, then the exponentials, summed among themselves
   const float me = d_mexp(st);
@@ -95,47 +130,53 @@ __device__ __forceinline__ void fold32(DLane& st, const float* z_src, int v0, in
 }
 
 // ===========================================================================
-// tcgen05 variant: the product on the 5th-generation tensor cores
+// the product on the 5th-generation tensor cores, the statistics in its epilogue
 // ===========================================================================
 //
-// One CTA of 192 threads per SM:
-//   warp 0      lane 0 issues the TMA loads of each stage (weight box 64 x 128
-//               rows = the MMA's A, hidden box 64 x 64 rows = its B);
-//   warp 1      allocates TMEM (two 64-column fp32 accumulators), and lane 0
-//               issues tcgen05.mma (M = 128 vocabulary entries, N = 64 hidden
-//               rows, K = 16 per instruction) and the commits;
-//   warps 2..5  the epilogue: warp w reads TMEM lanes 32 (w mod 4) .. (one
-//               vocabulary entry per thread, 64 logits: one per hidden row),
-//               transposes the tile through shared memory and folds it into
-//               the per-row statistics (each thread: one hidden row, one half
-//               of the 128 entries).
+// The MMA's M is the hidden rows and its N the vocabulary, so a TMEM lane is a
+// hidden row and its columns are consecutive logits of that row: an epilogue
+// thread reads and folds its own row, without a transpose.  (With the
+// vocabulary as M every chunk went through shared memory behind two barriers,
+// folded by four warps: at 256 rows a tile took 17 us to fold against 11 us of
+// MMAs.)  A tile is 128 vocabulary entries.  Blocks of H = 64, 128 or 256
+// hidden rows: 64 rows fill the 128 lanes twice over, 256 rows take two MMAs
+// and accumulators of 128 lanes.
+//
+// One CTA of 320 threads per SM:
+//   warp 0      lane 0 issues the TMA loads of each stage (weight box of 64 x
+//               128 rows = the MMA's B, hidden boxes = its A);
+//   warp 1      allocates TMEM (two sets of accumulators of 128 columns), and
+//               lane 0 issues tcgen05.mma (K = 16 per instruction) and the
+//               commits;
+//   warps 2..9  the epilogue: warp w reads TMEM lanes 32 (w mod 4) ..; the two
+//               warps of a lane quarter, and the two copies of 64 rows, take
+//               an equal part of the tile's columns each.
 // Barriers: full[s] / empty[s] per stage (TMA -> MMA -> TMA), tfull[b] /
-// tempty[b] per accumulator (MMA -> epilogue -> MMA).  Every wait is bounded;
-// TMEM is released after the last commit and the last load have completed.
-constexpr int kTcM = 128;                           // vocabulary entries per tile (MMA M)
-constexpr int kTcAStage = kTcM * 128;               // 16 KB: 128 rows x 64 bf16
-constexpr int kTcThreads = 192;
-constexpr int kTcCPitch = kTcM + 4;                 // floats per row of the transposed 64-row chunk
+// tempty[b] per accumulator set (MMA -> epilogue -> MMA).  Every wait is
+// bounded; TMEM is released after the last commit and the last load have
+// completed.
+constexpr int kTcN = 128;                           // vocabulary entries per tile (MMA N)
+constexpr int kTcWStage = kTcN * 128;               // 16 KB: 128 weight rows x 64 bf16
+constexpr int kTcEpiThreads = 256;
+constexpr int kTcThreads = 64 + kTcEpiThreads;
 
-// Shapes for a block of N hidden rows (the MMA's N: 64, 128 or 256).  The
-// accumulators take 2N TMEM columns; the epilogue walks them in chunks of 64
-// columns (hidden rows); the stage count fills the shared memory.
-template <int N>
+template <int H>
 struct TcShape {
-  static_assert(N == 64 || N == 128 || N == 256, "block rows");
-  static constexpr int kStages = N == 256 ? 4 : (N == 128 ? 5 : 6);
-  static constexpr int kBStage = N * 128;
-  static constexpr int kCols = 2 * N;
-  static constexpr int kChunks = N / 64;
-  static constexpr size_t kStageBytes = (size_t)kStages * (kTcAStage + kBStage);
-  static constexpr size_t kCBytes = (size_t)64 * kTcCPitch * 4;
-  static constexpr size_t kSmem = 1024 + kStageBytes + kCBytes + 8 * (2 * kStages + 4) + 16;
-  // instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, both
-  // K-major, N >> 3 at bit 17, M >> 4 at bit 24
-  static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-                                     ((uint32_t)(kTcM >> 4) << 24);
+  static_assert(H == 64 || H == 128 || H == 256, "block rows");
+  static constexpr int kAcc = H == 256 ? 2 : 1;     // accumulators of 128 lanes
+  static constexpr int kSplit = 256 / H;            // threads per hidden row
+  static constexpr int kCols = kTcN / kSplit;       // columns each of them folds
+  static constexpr int kStages = H == 256 ? 4 : 6;
+  static constexpr int kHStage = kAcc * 128 * 128;  // bytes of hidden rows per stage
+  static constexpr int kTmem = 2 * kAcc * kTcN;     // TMEM columns
+  static constexpr size_t kStageBytes = (size_t)kStages * (kTcWStage + kHStage);
+  static constexpr size_t kRedBytes = (size_t)kTcEpiThreads * 20;   // DRed per thread, 5 arrays
+  static constexpr size_t kSmem = 1024 + kStageBytes + kRedBytes + 8 * (2 * kStages + 4) + 16;
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
+// instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, both
+// K-major, N >> 3 at bit 17, M >> 4 at bit 24
+constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
 // Shared-memory matrix descriptor of a K-major tile with 128-byte rows and the
 // 128-byte swizzle: start address, leading offset (unused for this layout),
@@ -157,40 +198,53 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+// the same, arriving on the barrier at that offset of every CTA in `mask`
+__device__ __forceinline__ void tc_commit_mc(uint32_t bar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"(mask)
+      : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// 32 lanes x 64 columns of fp32 from TMEM: thread i gets lane (taddr lane + i), columns c .. c + 63
-__device__ __forceinline__ void tc_ld64(uint32_t taddr, float (&v)[64]) {
-  uint32_t r[64];
+// 32 lanes x 32 columns of fp32 from TMEM: thread i gets lane (taddr lane + i), columns c .. c + 31
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,"
-      "%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];"
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
-        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
-        "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int k = 0; k < 64; ++k) v[k] = __uint_as_float(r[k]);
+  for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]);
 }
-// named barrier among the 128 epilogue threads (barrier 0 is __syncthreads)
-__device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// named barrier among the epilogue threads (barrier 0 is __syncthreads)
+__device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-template <int N>
-__global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadArgs h,
+// CS CTAs of a cluster share the hidden rows' loads: each reads 1/CS of a
+// stage's box from L2 and multicasts it to all of them, so they walk the same
+// number of tiles in step.  hrows: rows loaded of a block (lanes beyond them
+// hold whatever was there: a lane's result depends on its own row alone).
+// tmap_w0, tmap_w1: the weight in boxes of the rows of a run's last tile (runs
+// of q and q + 1 groups of eight entries), so that no row is read twice (a
+// whole box there made the kernel read 1.06 x the weight at V=128256).
+template <int H, int CS>
+__global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadArgs h, const int hrows, const int tail0,
+                                                                 const int tail1,
                                                                  const __grid_constant__ CUtensorMap tmap_h,
-                                                                 const __grid_constant__ CUtensorMap tmap_w) {
-  using S = TcShape<N>;
+                                                                 const __grid_constant__ CUtensorMap tmap_w,
+                                                                 const __grid_constant__ CUtensorMap tmap_w0,
+                                                                 const __grid_constant__ CUtensorMap tmap_w1) {
+  using S = TcShape<H>;
+  constexpr uint16_t kAll = (uint16_t)((1 << CS) - 1);
   constexpr int kStages = S::kStages;
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -198,39 +252,56 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   int v0, v1;
   cta_run(h.V, h.nct, cta, v0, v1);
-  const int ntiles = v1 > v0 ? (v1 - v0 + kTcM - 1) / kTcM : 0;
+  const int own = v1 > v0 ? (v1 - v0 + kTcN - 1) / kTcN : 0;   // tiles of this CTA's run
+  const int cr = CS > 1 ? cta % CS : 0;            // rank in the cluster (nct is a multiple of CS)
+  int ntiles = own;                                // the cluster's: the longest run's
+  if (CS > 1) {
+#pragma unroll
+    for (int c = 0; c < CS; ++c) {
+      int a0, a1;
+      cta_run(h.V, h.nct, cta - cr + c, a0, a1);
+      const int n = a1 > a0 ? (a1 - a0 + kTcN - 1) / kTcN : 0;
+      ntiles = n > ntiles ? n : ntiles;
+    }
+  }
+  // the last tile's rows: runs of q + 1 groups come first
+  const int n8 = (h.V + 7) / 8;
+  const bool longer = cta < n8 - (n8 / h.nct) * h.nct;
+  const CUtensorMap* map_last = longer ? &tmap_w1 : &tmap_w0;
+  const int tail = longer ? tail1 : tail0;
   const int nkc = h.d / 64;
   const int G = ntiles * nkc;
-  const int row0 = rb * N;
+  const int row0 = rb * H;
 
   const uint32_t raw = smem_u32(tc_smem_raw);
   const uint32_t pad = ((raw + 1023u) & ~1023u) - raw;
   unsigned char* sm = tc_smem_raw + pad;
-  const uint32_t sA = raw + pad, sB = sA + kStages * kTcAStage;
-  float* sC = reinterpret_cast<float*>(sm + S::kStageBytes);
-  const uint32_t bars = smem_u32(sm + S::kStageBytes + S::kCBytes);
+  const uint32_t sW = raw + pad, sH = sW + kStages * kTcWStage;
+  float* s_red = reinterpret_cast<float*>(sm + S::kStageBytes);
+  const uint32_t bars = smem_u32(sm + S::kStageBytes + S::kRedBytes);
   const uint32_t full = bars, empty = bars + 8 * kStages;
   const uint32_t tfull = bars + 16 * kStages, tempty = tfull + 16;
-  uint32_t* s_taddr = reinterpret_cast<uint32_t*>(sm + S::kStageBytes + S::kCBytes + 8 * (2 * kStages + 4));
+  uint32_t* s_taddr = reinterpret_cast<uint32_t*>(sm + S::kStageBytes + S::kRedBytes + 8 * (2 * kStages + 4));
   if (tid == 0) {
     for (int k = 0; k < kStages; ++k) {
       mbar_init(full + 8 * k, 1);
-      mbar_init(empty + 8 * k, 1);
+      mbar_init(empty + 8 * k, CS);                // every CTA's MMAs have read what it multicast
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull + 8 * b, 1);
-      mbar_init(tempty + 8 * b, 128);
+      mbar_init(tempty + 8 * b, kTcEpiThreads);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_taddr)),
-                 "r"(S::kCols)
+                 "r"(S::kTmem)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  if (CS > 1) cluster_sync();                      // the peers' barriers exist before the first multicast
   tc_fence_after();
   const uint32_t tbase = *s_taddr;
   bool ok = true;
@@ -242,9 +313,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
         const int slot = g % kStages;
         if (g >= kStages && ok) ok = mbar_wait(empty + 8 * slot, (uint32_t)((g / kStages - 1) & 1));
         const int t = g / nkc, kc = g - t * nkc;
-        mbar_arrive_tx(full + 8 * slot, kTcAStage + S::kBStage);
-        tma_load_2d(sA + slot * kTcAStage, &tmap_w, kc * 64, v0 + t * kTcM, full + 8 * slot);
-        tma_load_2d(sB + slot * S::kBStage, &tmap_h, kc * 64, row0, full + 8 * slot);
+        const uint32_t wbytes = t < own - 1 ? kTcWStage : (t == own - 1 ? tail * 128 : 0);
+        mbar_arrive_tx(full + 8 * slot, wbytes + (H == 64 ? 2 : 1) * hrows * 128);
+        if (t < own)
+          tma_load_2d(sW + slot * kTcWStage, t < own - 1 ? &tmap_w : map_last, kc * 64, v0 + t * kTcN, full + 8 * slot);
+        // the hidden rows (64 of them: twice), this CTA's part of the box
+        const uint32_t hdst = sH + slot * S::kHStage + cr * (hrows / CS) * 128;
+#pragma unroll
+        for (int c = 0; c < (H == 64 ? 2 : 1); ++c) {
+          if (CS == 1)
+            tma_load_2d(hdst + c * 64 * 128, &tmap_h, kc * 64, row0, full + 8 * slot);
+          else
+            tma_load_2d_mc(hdst + c * 64 * 128, &tmap_h, kc * 64, row0 + cr * (hrows / CS), full + 8 * slot, kAll);
+        }
       }
     }
   } else if (warp == 1) {
@@ -254,78 +335,92 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
         const int b = t & 1;
         if (t >= 2 && ok) ok = mbar_wait(tempty + 8 * b, (uint32_t)((t / 2 - 1) & 1));
         tc_fence_after();
-        const uint32_t d = tbase + (uint32_t)(b * N);
+        const uint32_t d = tbase + (uint32_t)(b * S::kAcc * kTcN);
         for (int kc = 0; kc < nkc; ++kc) {
           const int g = t * nkc + kc, slot = g % kStages;
           if (ok) ok = mbar_wait(full + 8 * slot, (uint32_t)((g / kStages) & 1));
           tc_fence_after();
-          const uint64_t ad = umma_desc_sw128(sA + slot * kTcAStage);
-          const uint64_t bd = umma_desc_sw128(sB + slot * S::kBStage);
+          const uint64_t wd = umma_desc_sw128(sW + slot * kTcWStage);
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)          // K = 16 per instruction: 32 bytes along the row
-            tc_mma(d, ad + (uint64_t)(2 * ks), bd + (uint64_t)(2 * ks), S::kIdesc, (kc | ks) != 0);
-          tc_commit(empty + 8 * slot);             // the stage may be refilled once these MMAs are done
+          for (int c = 0; c < S::kAcc; ++c) {
+            const uint64_t hd = umma_desc_sw128(sH + slot * S::kHStage + c * 128 * 128);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)        // K = 16 per instruction: 32 bytes along the row
+              tc_mma(d + c * kTcN, hd + (uint64_t)(2 * ks), wd + (uint64_t)(2 * ks), kTcIdesc, (kc | ks) != 0);
+          }
+          // the stage may be refilled once these MMAs are done
+          if (CS == 1) tc_commit(empty + 8 * slot);
+          else tc_commit_mc(empty + 8 * slot, kAll);
         }
         tc_commit(tfull + 8 * b);                  // the accumulator is complete
       }
     }
     __syncwarp();
   } else {
-    // ---- epilogue: warps 2..5 ------------------------------------------------
-    const int e = tid - 64;                        // 0 .. 127
+    // ---- epilogue: warps 2..9 ------------------------------------------------
+    const int e = tid - 64;                        // 0 .. 255
     const int q = warp & 3;                        // TMEM lane quarter this warp may read
-    const int m = q * 32 + lane;                   // the vocabulary entry (TMEM lane) this thread reads
-    const int jrow = e >> 1, half = e & 1;         // within each 64-row chunk: the row and half-tile it folds
-    DLane st[S::kChunks];
-#pragma unroll
-    for (int c = 0; c < S::kChunks; ++c) dlane_init(st[c]);
+    const int m = q * 32 + lane;                   // its TMEM lane
+    const int grp = (warp - 2) >> 2;               // the two warps of a quarter
+    const int acc = H == 256 ? grp : 0;
+    const int row = H == 256 ? grp * 128 + m : (H == 128 ? m : (m & 63));      // hidden row within the block
+    const int part = H == 256 ? 0 : (H == 128 ? grp : ((m >> 6) * 2 + grp));   // its part of the columns
+    DLane st;
+    dlane_init(st);
     for (int t = 0; t < ntiles; ++t) {
       const int b = t & 1;
       if (ok) ok = mbar_wait(tfull + 8 * b, (uint32_t)((t / 2) & 1));
+      __syncwarp();
       tc_fence_after();
-#pragma unroll
-      for (int c = 0; c < S::kChunks; ++c) {
-        float v[64];
-        tc_ld64(tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * N + 64 * c), v);
-        if (c == S::kChunks - 1) {
+      const uint32_t src = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)((b * S::kAcc + acc) * kTcN + part * S::kCols);
+      const int vq = v0 + t * kTcN + part * S::kCols;
+#pragma unroll 1
+      for (int c = 0; c < S::kCols; c += 32) {
+        float z[32];
+        __syncwarp();                              // (the fold below may have diverged)
+        tc_ld32(src + c, z);
+        if (c + 32 == S::kCols) {
           tc_fence_before();
-          mbar_arrive(tempty + 8 * b);             // this lane of the accumulator has been read
+          mbar_arrive(tempty + 8 * b);             // this thread's columns have been read
         }
-        // transpose: row j of the chunk holds hidden row 64 c + j's logits over the 128 entries
+        if (h.logits && row0 + row < h.R) {
+          float* dst = h.logits + (size_t)(row0 + row) * h.V + vq + c;
 #pragma unroll
-        for (int j = 0; j < 64; ++j) sC[j * kTcCPitch + m] = v[j];
-        epi_bar();
-        const int vq = v0 + t * kTcM + half * 64;
-        const float* zs = sC + jrow * kTcCPitch + half * 64;
-        fold32(st[c], zs, vq, v1);
-        fold32(st[c], zs + 32, vq + 32, v1);
-        const int grow = row0 + 64 * c + jrow;
-        if (h.logits && grow < h.R) {
-          float* dst = h.logits + (size_t)grow * h.V;
-          for (int k = 0; k < 64 && vq + k < v1; ++k) dst[vq + k] = zs[k];
+          for (int k = 0; k < 32; ++k)
+            if (vq + c + k < v1) dst[k] = z[k];
         }
-        epi_bar();                                 // the chunk buffer is rewritten next
+        fold32(st, z, vq + c, v1);
       }
     }
-#pragma unroll
-    for (int c = 0; c < S::kChunks; ++c) {
-      float s, t2;
-      d_final(st[c], s, t2);
-      DRed x{d_mexp(st[c]), s, t2, st[c].f2, st[c].pos};
-      DRed y;
-      y.m = __shfl_xor_sync(kFull, x.m, 1);
-      y.s = __shfl_xor_sync(kFull, x.s, 1);
-      y.t2 = __shfl_xor_sync(kFull, x.t2, 1);
-      y.top2 = __shfl_xor_sync(kFull, x.top2, 1);
-      y.idx = __shfl_xor_sync(kFull, x.idx, 1);
-      fold_d(x, y);
-      if (half == 0) {
-        Partial p;
-        p.d_m = x.m; p.d_s = x.s; p.d_t2 = x.t2; p.d_top2 = x.top2; p.d_idx = x.idx;
-        p.t_m = 0.f; p.t_s = 0.f; p.t_idx = 0; p.t_cnt = 0;
-        p.pad[0] = p.pad[1] = p.pad[2] = 0;
-        h.part[((size_t)rb * h.nct + cta) * N + 64 * c + jrow] = p;
+    float fs, ft2;
+    d_final(st, fs, ft2);
+    DRed x{d_mexp(st), fs, ft2, st.f2, st.pos};
+    if (S::kSplit > 1) {                           // the threads of a row: part 0 merges the others'
+      if (part > 0) {
+        s_red[e] = x.m;
+        s_red[kTcEpiThreads + e] = x.s;
+        s_red[2 * kTcEpiThreads + e] = x.t2;
+        s_red[3 * kTcEpiThreads + e] = x.top2;
+        s_red[4 * kTcEpiThreads + e] = __int_as_float(x.idx);
       }
+      epi_bar();
+      if (part == 0) {
+#pragma unroll
+        for (int c = 1; c < S::kSplit; ++c) {
+          // the epilogue thread of this row's part c: warp group c & 1, the other copy of 64 rows for c > 1
+          const int mo = H == 64 && (c >> 1) ? m + 64 : m;
+          const int eo = 32 * (((c & 1) << 2) + (((mo >> 5) + 2) & 3)) + lane;
+          fold_d(x, DRed{s_red[eo], s_red[kTcEpiThreads + eo], s_red[2 * kTcEpiThreads + eo],
+                         s_red[3 * kTcEpiThreads + eo], __float_as_int(s_red[4 * kTcEpiThreads + eo])});
+        }
+      }
+    }
+    if (part == 0) {
+      Partial p;
+      p.d_m = x.m; p.d_s = x.s; p.d_t2 = x.t2; p.d_top2 = x.top2; p.d_idx = x.idx;
+      p.t_m = 0.f; p.t_s = 0.f; p.t_idx = 0; p.t_cnt = 0;
+      p.pad[0] = p.pad[1] = p.pad[2] = 0;
+      h.part[((size_t)rb * h.nct + cta) * H + row] = p;
     }
   }
   if (!ok) atomicOr(h.err, 4u);
@@ -338,12 +433,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   if (warp == 0 && lane == 0) {                    // no TMA box still in flight into this CTA
     for (int g = (G > kStages ? G - kStages : 0); g < G; ++g)
       if (!mbar_wait(full + 8 * (g % kStages), (uint32_t)((g / kStages) & 1))) atomicOr(h.err, 4u);
+    if (CS > 1) {                                  // nor a peer's commit on its way to these barriers
+      for (int g = (G > kStages ? G - kStages : 0); g < G; ++g)
+        if (!mbar_wait(empty + 8 * (g % kStages), (uint32_t)((g / kStages) & 1))) atomicOr(h.err, 4u);
+    }
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
+  if (CS > 1) cluster_sync();                      // nor a peer still waiting for what this CTA multicasts
   tc_fence_after();
   if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(S::kCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(S::kTmem) : "memory");
 }
 
 // One warp per hidden row: fold the row's per-CTA partials, then the row's
@@ -388,7 +489,7 @@ int lmhead_ctas_per_block(int sms, int R, int V) {
   int nct = sms / (nrb > 0 ? nrb : 1);
   const int n8 = (V + 7) / 8;
   if (nct > n8) nct = n8;
-  return nct < 1 ? 1 : nct;
+  return nct < 4 ? 4 : nct;                        // (at least one cluster)
 }
 
 namespace {
@@ -425,30 +526,94 @@ bool encode_rows(CUtensorMap* m, const void* base, int d, int rows, int box_rows
 }
 }  // namespace
 
-template <int N>
-cudaError_t launch_tc(const LmHeadArgs& h, cudaStream_t s) {
+template <int H, int CS>
+cudaError_t tc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, unsigned grid) {
   static unsigned long long done = 0ull;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  CUtensorMap tmap_h, tmap_w;
-  if (!encode_rows(&tmap_h, h.hidden, h.d, h.R, N) || !encode_rows(&tmap_w, h.weight, h.d, h.V, kTcM))
-    return cudaErrorInvalidValue;
   const unsigned long long bit = 1ull << (dev & 63);
   if (!(__atomic_load_n(&done, __ATOMIC_ACQUIRE) & bit)) {
-    e = cudaFuncSetAttribute(lmhead_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)TcShape<N>::kSmem);
+    e = cudaFuncSetAttribute(lmhead_tc_kernel<H, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)TcShape<H>::kSmem);
     if (e != cudaSuccess) return e;
     __atomic_fetch_or(&done, bit, __ATOMIC_ACQ_REL);
   }
-  const int nrb = (h.R + N - 1) / N;
-  lmhead_tc_kernel<N><<<nrb * h.nct, kTcThreads, TcShape<N>::kSmem, s>>>(h, tmap_h, tmap_w);
-  return cudaGetLastError();
+  cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = TcShape<H>::kSmem;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = CS;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaSuccess;
 }
 
-cudaError_t launch_lmhead(const LmHeadArgs& h, const StreamArgs& a, cudaStream_t s) {
+// CTAs in clusters of CS that can be resident on the current device (cached
+// for the first 64; 0: none).
+template <int H, int CS>
+int tc_resident() {
+  static std::atomic<int> known[64];               // 0: not asked yet, else the answer + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  int v = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (v == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    int n = 0;
+    if (tc_config<H, CS>(cfg, attr, CS) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, lmhead_tc_kernel<H, CS>, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();                    // a refused query leaves no error behind for the caller
+      n = 0;
+    }
+    v = 1 + n * CS;
+    if (dev < 64) known[dev].store(v, std::memory_order_relaxed);
+  }
+  return v - 1;
+}
+
+// h.nct: on entry the most CTAs per block, on return what was launched.
+template <int H, int CS>
+cudaError_t launch_tc(LmHeadArgs& h, cudaStream_t s) {
+  const int nrb = (h.R + H - 1) / H;
+  if (CS > 1) {
+    const int res = tc_resident<H, CS>() / nrb;
+    int n = h.nct < res ? h.nct : res;
+    n -= n % CS;
+    h.nct = n < CS ? CS : n;                       // (a run may be empty)
+  }
+  const int n8 = (h.V + 7) / 8, q = n8 / h.nct;
+  const int tail0 = q > 0 ? (8 * q - 1) % kTcN + 1 : 8, tail1 = (8 * q + 7) % kTcN + 1;
+  const int step = 8 * CS;                         // a CTA's part of the hidden box: whole groups of eight rows
+  int hrows = nrb == 1 ? (h.R + step - 1) / step * step : H;
+  if (hrows > H) hrows = H;
+  CUtensorMap tmap_h, tmap_w, tmap_w0, tmap_w1;
+  if (!encode_rows(&tmap_h, h.hidden, h.d, h.R, hrows / CS) || !encode_rows(&tmap_w, h.weight, h.d, h.V, kTcN) ||
+      !encode_rows(&tmap_w0, h.weight, h.d, h.V, tail0) || !encode_rows(&tmap_w1, h.weight, h.d, h.V, tail1))
+    return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  const cudaError_t e = tc_config<H, CS>(cfg, attr, (unsigned)(nrb * h.nct));
+  if (e != cudaSuccess) return e;
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, lmhead_tc_kernel<H, CS>, h, hrows, tail0, tail1, tmap_h, tmap_w, tmap_w0, tmap_w1);
+}
+
+// Clusters of four share the hidden rows' loads up to 128 rows (R=16 d=1024
+// V=32000: 19.2 us a call against 21.0 alone; R=64 d=2048 V=128256: 89.1
+// against 92.0; R=128: 91.1 against 92.9; pairs were slower than either).  256
+// rows are bound by the MMAs' reads of shared memory (108.7 us alone, 109.3
+// with four).
+cudaError_t launch_lmhead(const LmHeadArgs& args, const StreamArgs& a, cudaStream_t s) {
+  LmHeadArgs h = args;
   if (h.nb != lmhead_block_rows(h.R)) return cudaErrorInvalidValue;
-  cudaError_t e = h.nb == 64 ? launch_tc<64>(h, s) : (h.nb == 128 ? launch_tc<128>(h, s) : launch_tc<256>(h, s));
+  cudaError_t e;
+  if (h.nb == 64) e = tc_resident<64, 4>() >= 4 ? launch_tc<64, 4>(h, s) : launch_tc<64, 1>(h, s);
+  else if (h.nb == 128) e = tc_resident<128, 4>() >= 4 ? launch_tc<128, 4>(h, s) : launch_tc<128, 1>(h, s);
+  else e = launch_tc<256, 1>(h, s);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((h.R + kMergeRowsPerCta - 1) / kMergeRowsPerCta));

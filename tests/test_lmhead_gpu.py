@@ -63,6 +63,21 @@ def test_exact_inputs_bit_exact(cmsd, R, d, V):
         assert np.max(np.abs(g[k] - o[k])) <= TOL, k
 
 
+# Several tiles per run with every kind of last tile (8 .. 128 rows, runs of two
+# lengths), rows that fill a block's boxes in part, an empty run in a cluster
+@pytest.mark.parametrize("R,V", [(9, 144 * 128 + 8), (33, 18440), (64, 144 * 8 + 1), (100, 36873), (129, 152 * 136),
+                                 (256, 19457), (200, 152 * 8 - 3), (16, 20), (513, 4099)])
+def test_runs_and_last_tiles(cmsd, R, V):
+    w = W.make_lmhead(R=R, d=128, V=V, seed=R + V, exact=True)
+    p, P = _params(cmsd)
+    g = _run(cmsd, w, p)
+    o = O.lm_head_confidence(w.hidden, w.weight, P, rows=range(0, R, 7))
+    assert np.array_equal(g["logits"].astype(np.float64), o["logits"])
+    assert np.array_equal(g["argmax"], np.argmax(o["logits"], axis=1))
+    for k in ("H", "margin", "lse", "conf"):
+        assert np.max(np.abs(g[k][::7] - o[k][::7])) <= TOL, k
+
+
 @pytest.mark.parametrize("R,d,V", [(64, 512, 20000), (16, 1024, 32000)])
 def test_realistic_inputs_within_rounding_bounds(cmsd, R, d, V):
     w = W.make_lmhead(R=R, d=d, V=V, seed=11)
