@@ -249,7 +249,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rb = blockIdx.x / h.nct, cta = blockIdx.x - rb * h.nct;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   int v0, v1;
   cta_run(h.V, h.nct, cta, v0, v1);
   const int own = v1 > v0 ? (v1 - v0 + kTcN - 1) / kTcN : 0;   // tiles of this CTA's run
@@ -301,6 +300,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   }
   tc_fence_before();
   __syncthreads();
+  // everything above overlaps the end of what precedes this grid on the stream
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (CS > 1) cluster_sync();                      // the peers' barriers exist before the first multicast
   tc_fence_after();
   const uint32_t tbase = *s_taddr;
@@ -450,6 +452,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
 // One warp per hidden row: fold the row's per-CTA partials, then the row's
 // signals and confidence (the logits pass's row arithmetic).
 __global__ void __launch_bounds__(32 * kMergeRowsPerCta) lmhead_merge_kernel(const LmHeadArgs h, const StreamArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the next call's grid waits for this one's end)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * kMergeRowsPerCta + (threadIdx.x >> 5);
@@ -527,7 +530,7 @@ bool encode_rows(CUtensorMap* m, const void* base, int d, int rows, int box_rows
 }  // namespace
 
 template <int H, int CS>
-cudaError_t tc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, unsigned grid) {
+cudaError_t tc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], unsigned grid) {
   static unsigned long long done = 0ull;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -543,12 +546,14 @@ cudaError_t tc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, unsign
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kTcThreads);
   cfg.dynamicSmemBytes = TcShape<H>::kSmem;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = CS;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CS;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   return cudaSuccess;
 }
 
@@ -562,9 +567,9 @@ int tc_resident() {
   int v = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
   if (v == 0) {
     cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
+    cudaLaunchAttribute attr[2];
     int n = 0;
-    if (tc_config<H, CS>(cfg, attr, CS) != cudaSuccess ||
+    if (tc_config<H, CS>(cfg, attr, CS) != cudaSuccess || (cfg.numAttrs = 1) == 0 ||   // (the cluster size)
         cudaOccupancyMaxActiveClusters(&n, lmhead_tc_kernel<H, CS>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();                    // a refused query leaves no error behind for the caller
       n = 0;
@@ -595,7 +600,7 @@ cudaError_t launch_tc(LmHeadArgs& h, cudaStream_t s) {
       !encode_rows(&tmap_w0, h.weight, h.d, h.V, tail0) || !encode_rows(&tmap_w1, h.weight, h.d, h.V, tail1))
     return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
+  cudaLaunchAttribute attr[2];
   const cudaError_t e = tc_config<H, CS>(cfg, attr, (unsigned)(nrb * h.nct));
   if (e != cudaSuccess) return e;
   cfg.stream = s;

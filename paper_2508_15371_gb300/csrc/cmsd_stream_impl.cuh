@@ -2044,6 +2044,7 @@ __global__ void __launch_bounds__(kDrawThreads, 4) draw_kernel(const StreamArgs 
   const int cr = (int)cl.block_rank();
   const int ncl = (int)(gridDim.x / (unsigned)nc);
   const Workspace& W = a.ws;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the next call's grid waits for this one's end)
   cluster_arrive();
   bool first = true;
   for (int b = (int)(blockIdx.x / (unsigned)nc); b < a.B; b += ncl) {
@@ -2172,6 +2173,7 @@ __global__ void __launch_bounds__(kCluThreads, 2) resample_bound_kernel(const St
   const uint32_t cw_grp = iter_word(a.iteration, kPurposeGroup);
   const uint32_t cw_ent = iter_word(a.iteration, kPurposeResidual);
   const int ncl = (int)gridDim.x / kCluCtas;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the next call's grid waits for this one's end)
   // No griddepcontrol.wait here: a sequence's draw starts as soon as its
   // epilogue has released the record word (every read below follows that
   // acquire), while the streaming kernel may still be finishing other
@@ -2368,8 +2370,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
   const Workspace& W = a.ws;
   const bool ragged = a.k_row != nullptr;
   int* s_pref = reinterpret_cast<int*>(smem);
-  // the resample kernel (launched as a programmatic dependent) may be
-  // scheduled now; it waits for this grid's completion before reading anything
+  // This grid is itself a programmatic dependent of what precedes it on the
+  // stream (another call's draw, say): its CTAs may be placed early, and read
+  // nothing before that has completed.  Only then may the second pass be
+  // scheduled, which polls this call's records.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (PH2) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // -- present rows: exclusive prefix of k_row (ragged windows) -------------
@@ -2460,6 +2465,11 @@ cudaError_t launch_one(const StreamArgs& a, int grid, size_t smem, cudaStream_t 
   cfg.blockDim = dim3(kStreamThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, stream_kernel<T, MODE, SAMPLED, PH2>, a);
 }
 
