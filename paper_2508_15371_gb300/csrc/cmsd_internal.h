@@ -120,12 +120,12 @@ struct StreamSplit {
     V = V_;
     VEC = vec;
     N = (int64_t)R * V;
-    int64_t want = N / min_len;
+    int64_t want = div_nn(N, min_len);
     if (want < 1) want = 1;
     const int Wmax = (int)(want < nwarps ? want : nwarps);
     int p = nwarps / R;                              // pieces per row that fit
-    const int64_t pm = (int64_t)V / min_len;
-    const int pmax = pm > 0 ? (int)pm : 1;
+    const int pm = (int)div_nn(V, min_len);
+    const int pmax = pm > 0 ? pm : 1;
     if (p > pmax) p = pmax;
     if (p >= 1 && (int64_t)p * R * 4 >= (int64_t)Wmax * 3) {   // uses at least 3/4 of the warps
       wpr = p;
