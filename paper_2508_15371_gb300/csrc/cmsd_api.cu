@@ -234,8 +234,8 @@ void fill_sizes(StreamArgs& a, int B, int K, int V) {
 }
 
 // CTAs per cluster that choose_seq weighs.
-constexpr int kSeqSizes[] = {1, 2, 4, 5, 8, 16};
-constexpr int kSeqNumSizes = 6;
+constexpr int kSeqSizes[] = {1, 2, 3, 4, 5, 6, 8, 16};
+constexpr int kSeqNumSizes = 8;
 
 // Clusters of seq_kernel that can be resident on device dev, which is current
 // (cached; n: index into kSeqSizes).
@@ -262,8 +262,9 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 //     through its CTAs (a CTA of 256 threads: 27 KB a microsecond under the
 //     PAPER rule, 21 with the target's exponentials or the drafter alone, 30
 //     for the target alone; one of 512 twice that), times the waves when not
-//     every cluster is resident (3.5 more each), and no less than the bytes at
-//     6900 MB/s.
+//     every cluster is resident (3.5 more each, 10 with clusters of several
+//     CTAs: B=192 K=12 V=32001 verify took 37 us in two waves of three,
+//     31.6 streamed), and no less than the bytes at 6900 MB/s.
 // Ragged windows are unknown here: half full on average, and the longest
 // decides the one-launch pass, since a sequence keeps to its cluster.
 bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int* nc, int* threads) {
@@ -290,10 +291,11 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       if (fixed + part >= best) continue;
       const int res = seq_resident(dev, dtype, k, th);
       if (res < 1) continue;
-      // (clusters of 4 and more were not all placed at once near the limit)
-      const int fit = n >= 4 ? (res * 9 + 9) / 10 : res;
+      // (clusters of 3 and more were not all placed at once near the limit; of
+      // ragged windows some end early)
+      const int fit = n >= 3 && !a.k_row ? (res * 9 + 9) / 10 : res;
       const int waves = (a.B + fit - 1) / fit;
-      const double t = fixed + (th == 512 ? 0.7 : 0.0) + 3.5 * (waves - 1) +
+      const double t = fixed + (th == 512 ? 0.7 : 0.0) + (n == 1 ? 3.5 : 10.0) * (waves - 1) +
                        (waves * part > stream ? waves * part : stream);
       if (t < best) {
         best = t;
