@@ -9,17 +9,16 @@
 // an L2 round trip of about a microsecond.  Here a sequence's rows are cut
 // over the warps of one cluster and every hand-over is a store into a peer's
 // shared memory and a cluster barrier:
-//   stream   each warp reduces its slice (the streaming kernel's arithmetic,
-//            four vectors per tensor and lane in flight ahead of the four
-//            being reduced) and stores its partial into the CTA that merges
-//            the row (row i: CTA i mod nc);
-//   rows     barrier; one warp per row merges its partials, takes the row's
-//            decision and stores it into every CTA;
-//   sequence barrier; every CTA finds the first rejection, CTA 0 writes the
-//            sequence's outputs;
+//   stream   each warp reduces its pieces (the streaming kernel's arithmetic)
+//            and stores their partials into every CTA;
+//   rows     barrier; one warp per row, in every CTA alike, merges its partials
+//            and takes the row's decision; every CTA finds the first rejection,
+//            CTA 0 writes the outputs;
 //   draw     under the sampled rule, or for the bonus row, the cluster draws
 //            the token itself: the race by group bounds (cluster_draw).
 //            Its rows were streamed moments ago and come from L2.
+// What can be formed before the preceding grid ends (a full window's first
+// piece) is, above griddepcontrol.wait.
 #pragma once
 #include "cmsd_stream_impl.cuh"
 
@@ -40,10 +39,29 @@ constexpr int kSeqMaxK = kPackedMaxK;    // positions per window
 // The cut of a window of kb rows over the cluster's warps, by kb.
 struct SeqSplit {
   int nc;                                // CTAs per cluster
-  int rcp;                               // 65536 / nc + 1: i / nc = i rcp >> 16 for i <= kSeqMaxK
+  int part_bytes;                        // shared memory of the partials
   int len[kSeqMaxK + 1];                 // entries per piece
   short pieces[kSeqMaxK + 1];            // pieces per row
 };
+
+// Piece u of the window: piece k of row i.
+template <typename T>
+struct SeqPiece {
+  int i, k;
+  const T* dp;
+  const T* tp;
+  Seg sg;
+};
+template <typename T, int MODE>
+__device__ __forceinline__ SeqPiece<T> seq_piece(const StreamArgs& a, const SeqSplit& sp, int b, int u, int p, int len) {
+  SeqPiece<T> x;
+  x.i = (int)((unsigned)u / (unsigned)p);
+  x.k = u - x.i * p;
+  x.dp = (const T*)a.draft + ((size_t)b * a.K + x.i) * (size_t)a.V;
+  x.tp = MODE != kModeConf ? (const T*)a.target + ((size_t)b * a.Kt + x.i) * (size_t)a.V : nullptr;
+  x.sg = seg_geom<T>(MODE != kModeVerify ? x.dp : x.tp, x.k * len, a.V, len);
+  return x;
+}
 
 // A row's decision as every CTA of the cluster keeps it.
 struct __align__(16) SeqRow {
@@ -61,26 +79,30 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
   extern __shared__ __align__(128) unsigned char seq_smem[];
   __shared__ SeqRow s_row[kSeqMaxK];
   cg::cluster_group cl = cg::this_cluster();
+  const int nc = sp.nc;
+  const int cr = (int)cl.block_rank(), b = (int)(blockIdx.x / (unsigned)nc);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nw = nc * NW;
+  Partial* s_part = reinterpret_cast<Partial*>(seq_smem);
+  // the warp's first piece: pieces are dealt over the CTAs in turn
+  int kb = a.K, p = sp.pieces[kb], u = warp * nc + cr;
+  SeqPiece<T> pc = {};
+  if (!a.k_row) pc = seq_piece<T, MODE>(a, sp, b, u, p, sp.len[kb]);
   // A programmatic dependent of whatever precedes it on the stream: its CTAs
   // may be placed early, and wait here for that grid's completion.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   cluster_arrive();                      // (a peer's shared memory is written only after the matching wait)
-  const int nc = sp.nc;
-  const int cr = (int)cl.block_rank(), b = (int)(blockIdx.x / (unsigned)nc);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int w = warp * nc + cr;          // pieces are dealt over the CTAs in turn
-  const int nw = nc * NW;
-  Partial* s_part = reinterpret_cast<Partial*>(seq_smem);
-  int kb = a.K;
   if (a.k_row) {
     const int raw = __ldg(a.k_row + b);
     kb = raw < 0 ? 0 : (raw > a.K ? a.K : raw);
     if (raw != kb && cr == 0 && threadIdx.x == 0) atomicOr(a.ws.err, 2u);
+    p = sp.pieces[kb];
+    if (kb > 0) pc = seq_piece<T, MODE>(a, sp, b, u, p, sp.len[kb]);
   }
   const int beta = a.beta_rank > 0 ? a.beta_rank : 0;
   // The window's drafted tokens, position i in lane i, and what the row merges
-  // of this warp need, row cr + nc (warp + NW l) in lane l: requested
+  // of this warp need, row warp + NW l in lane l: requested
   // here, used only once the slice's first logits are on their way.
   int tok = -1, tok_in = 0;
   if (HAS_T && lane < kb) tok = __ldg(a.tokens + (size_t)b * a.K + lane);
@@ -94,7 +116,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
         tok_in = 0;
       }
     }
-    const int im = cr + nc * (warp + NW * lane);
+    const int im = warp + NW * lane;
     const int tk = __shfl_sync(kFull, tok_in, im & 31);
     if (im < kb) {
       m_c = Elem<T>::load((const T*)a.target + ((size_t)b * a.Kt + im) * (size_t)a.V + tk);
@@ -106,13 +128,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     }
   };
   bool first = true;                     // the warp has not reduced a segment yet
-  const int p = sp.pieces[kb], len = sp.len[kb];
-  for (int u = w; u < kb * p; u += nw) {
-    const int i = (int)((unsigned)u / (unsigned)p), k = u - i * p;
-    const int ic = (i * sp.rcp) >> 16;   // i / nc
-    const T* dp = (const T*)a.draft + ((size_t)b * a.K + i) * (size_t)a.V;
-    const T* tp = HAS_T ? (const T*)a.target + ((size_t)b * a.Kt + i) * (size_t)a.V : nullptr;
-    const Seg sg = seg_geom<T>(HAS_D ? dp : tp, k * len, a.V, len);
+  while (u < kb * p) {
+    const int i = pc.i, k = pc.k;
+    const T* dp = pc.dp;
+    const T* tp = pc.tp;
+    const Seg sg = pc.sg;
     Pipe<T, HAS_D && HAS_T ? CMSD_SEQ_UNROLL : CMSD_SEQ_UNROLL1> pp;
     pipe_start<T, MODE>(pp, dp, tp, sg.va, sg.vb, lane);
     SegState ss;
@@ -139,25 +159,28 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     seg_reduce<T, MODE, SAMPLED>(ss, sg, !SAMPLED || a.argmax != nullptr, dp, tp, dr, tr);
     if (first) cluster_wait();         // every CTA of the cluster has started
     first = false;
-    if (lane == 0) {
+    if (lane < nc) {                     // the partial into every CTA
       Partial q;
       q.d_m = dr.m; q.d_s = dr.s; q.d_t2 = dr.t2; q.d_top2 = dr.top2; q.d_idx = dr.idx;
       q.t_m = tr.m; q.t_s = tr.s; q.t_idx = tr.idx; q.t_cnt = tr.cnt;
       q.pad[0] = q.pad[1] = q.pad[2] = 0;
-      *cl.map_shared_rank(s_part + ic * p + k, i - ic * nc) = q;
+      *cl.map_shared_rank(s_part + i * p + k, lane) = q;
     }
+    u += nw;
+    if (u < kb * p) pc = seq_piece<T, MODE>(a, sp, b, u, p, sp.len[kb]);
   }
   if (first) {
     row_inputs();
     cluster_wait();
   }
-  cluster_sync();                        // every slice's partial is in its row's CTA
-  // -- rows: merge, decide, tell every CTA ---------------------------------------
-  for (int l = 0, i = cr + nc * warp; i < kb; i += nw, ++l) {
+  cluster_sync();                        // every CTA has every piece's partial
+  // -- rows: every CTA merges and decides all of them (a second exchange and
+  // barrier took longer), CTA 0 writes their outputs -----------------------------
+  for (int l = 0, i = warp; i < kb; i += NW, ++l) {
     DRed dm = dred_empty();
     TRed tm = tred_empty();
     for (int k = lane; k < p; k += 32) {
-      const float4* src = reinterpret_cast<const float4*>(s_part + ((i * sp.rcp) >> 16) * p + k);
+      const float4* src = reinterpret_cast<const float4*>(s_part + i * p + k);
       const float4 x0 = src[0], x1 = src[1], x2 = src[2];
       if (HAS_D) fold_d(dm, DRed{x0.x, x0.y, x0.z, x0.w, __float_as_int(x1.x)});
       if (HAS_T) fold_t(tm, TRed{x1.y, x1.z, __float_as_int(x1.w), __float_as_int(x2.x)});
@@ -166,17 +189,17 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     const TRed tr = HAS_T ? reduce_t(tm) : tred_empty();
     const RowOut o = row_results<MODE, SAMPLED>(a, b * a.K + i, b, i, dr, tr, __shfl_sync(kFull, m_c, l),
                                                 __shfl_sync(kFull, m_zd, l), __shfl_sync(kFull, m_lse, l),
-                                                __shfl_sync(kFull, m_conf, l), lane);
-    if (lane < nc) {
+                                                __shfl_sync(kFull, m_conf, l), lane, cr == 0);
+    if (lane == 0) {
       SeqRow q;
       q.stat = make_float4(o.ds.x, o.ds.y, o.ts.x, o.ts.y);
       q.cfx = o.cfx;
       q.acc = o.acc ? 1 : 0;
       q.pad = 0;
-      *cl.map_shared_rank(s_row + i, lane) = q;
+      s_row[i] = q;
     }
   }
-  cluster_sync();                        // every CTA has every row's decision
+  __syncthreads();
   // -- the sequence ---------------------------------------------------------------
   const bool have = lane < kb;
   const bool acc = have && s_row[lane & (kSeqMaxK - 1)].acc != 0;
@@ -197,9 +220,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
   if (SECOND) {
     const int kind = seq_kind<MODE, SAMPLED>(a, n, kb);      // the same in every thread of the cluster
     if (kind == kSeqNone) return;
-    // the partials have been merged: the draw's state takes their place
-    DrawShared<T, NT>& sh = *reinterpret_cast<DrawShared<T, NT>*>(seq_smem);
-    float* s_u = reinterpret_cast<float*>(seq_smem + sizeof(DrawShared<T, NT>));
+    // the draw's state follows the partials, which a peer may still be merging
+    unsigned char* draw = seq_smem + sp.part_bytes;
+    DrawShared<T, NT>& sh = *reinterpret_cast<DrawShared<T, NT>*>(draw);
+    float* s_u = reinterpret_cast<float*>(draw + sizeof(DrawShared<T, NT>));
     const T* tp = (const T*)a.target + ((size_t)b * a.Kt + n) * (size_t)a.V;
     if (!SAMPLED) {
       cluster_argmax<T, NT>(a, cl, nc, cr, b, n, tp, sh);
@@ -241,22 +265,20 @@ void seq_split_window(SeqSplit& sp, int kb, int V, int nw) {
   }
 }
 
-// The partials of the rows a CTA merges; the draw's state and its share's
-// uniforms and bounds take their place.
+// The window's partials, then the draw's state and its share's uniforms and
+// bounds.
 template <typename T, int NT>
-size_t seq_smem_bytes(const SeqSplit& sp, int K, int V, bool second, bool sampled) {
-  const int nc = sp.nc;
+size_t seq_smem_bytes(SeqSplit& sp, int k0, int K, int V, bool second, bool sampled) {
   int slots = 0;
-  for (int k = 1; k <= K; ++k) {
-    const int n = ((k + nc - 1) / nc) * sp.pieces[k];
+  for (int k = k0; k <= K; ++k) {
+    const int n = k * sp.pieces[k];
     slots = n > slots ? n : slots;
   }
-  const size_t p = (size_t)slots * sizeof(Partial);
-  const size_t d = second ? sizeof(DrawShared<T, NT>) + (sampled ? draw_smem_bytes(V, nc) : 0) : 0;
-  return p > d ? p : d;
+  sp.part_bytes = (int)((slots * sizeof(Partial) + 127) / 128 * 128);
+  return (size_t)sp.part_bytes + (second ? sizeof(DrawShared<T, NT>) + (sampled ? draw_smem_bytes(V, sp.nc) : 0) : 0);
 }
 // (two CTAs of 256 threads, or one of 512, fit an SM with this much each)
-constexpr size_t kSeqSmemMax = 96 * 1024;
+constexpr size_t kSeqSmemMax = 112 * 1024;
 
 template <typename T, int NT, int MODE, bool SAMPLED, bool SECOND>
 cudaError_t seq_attrs() {
@@ -311,11 +333,11 @@ cudaError_t launch_seq_one(const StreamArgs& a, int nc, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   SeqSplit sp = {};
   sp.nc = nc;
-  sp.rcp = 65536 / nc + 1;
-  for (int k = a.k_row ? 1 : a.K; k <= a.K; ++k) seq_split_window<T>(sp, k, a.V, nc * (NT / 32));
+  const int k0 = a.k_row ? 1 : a.K;
+  for (int k = k0; k <= a.K; ++k) seq_split_window<T>(sp, k, a.V, nc * (NT / 32));
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  seq_config(cfg, attr, a.B, nc, NT, seq_smem_bytes<T, NT>(sp, a.K, a.V, SECOND, SAMPLED));
+  seq_config(cfg, attr, a.B, nc, NT, seq_smem_bytes<T, NT>(sp, k0, a.K, a.V, SECOND, SAMPLED));
   cfg.stream = s;
   return cudaLaunchKernelEx(&cfg, seq_kernel<T, NT, MODE, SAMPLED, SECOND>, a, sp);
 }
@@ -337,7 +359,8 @@ cudaError_t launch_seq_t(int mode, bool sampled, bool second, const StreamArgs& 
 // cluster's size.
 template <typename T>
 bool seq_draw_fits_t(int V) {
-  return sizeof(DrawShared<T, 512>) + draw_smem_bytes(V, 1) <= kSeqSmemMax;
+  const size_t parts = 4 * kSeqMaxCtas * 16 * sizeof(Partial);   // four pieces per warp, CTAs of 512 threads
+  return parts + sizeof(DrawShared<T, 512>) + draw_smem_bytes(V, 1) <= kSeqSmemMax;
 }
 
 }  // namespace cmsd

@@ -681,10 +681,11 @@ struct RowOut {
 // Called by the whole warp (statistics identical in every lane): the row's
 // exponentials and reciprocals are spread one per lane, so each costs one
 // instruction sequence instead of a chain on one lane.  Lane 0 writes the
-// outputs.  lse_in, conf_in: the caller's signals (verify mode).
+// outputs (when `write`).  lse_in, conf_in: the caller's signals (verify mode).
 template <int MODE, bool SAMPLED>
 __device__ __forceinline__ RowOut row_results(const StreamArgs& a, int r, int b, int i, const DRed& d, const TRed& t,
-                                              float c_tgt, float zd, float lse_in, float conf_in, int lane) {
+                                              float c_tgt, float zd, float lse_in, float conf_in, int lane,
+                                              bool write = true) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
   RowOut o;
@@ -735,7 +736,7 @@ __device__ __forceinline__ RowOut row_results(const StreamArgs& a, int r, int b,
       const long long f = __float2ll_rn(hi * kFixedScale) + __float2ll_rn(lo * kFixedScale);
       cfx = f < 0 ? 0ull : (unsigned long long)f;
     }
-    if (lane == 0) {
+    if (write && lane == 0) {
       if (a.H) a.H[r] = H;
       if (a.margin) a.margin[r] = margin;
       if (a.argmax) a.argmax[r] = d.idx;
@@ -755,7 +756,7 @@ __device__ __forceinline__ RowOut row_results(const StreamArgs& a, int r, int b,
     if (!SAMPLED) {
       // gap-bounded acceptance: log P(y1) - log P(draft) = M - z_draft <= tau
       acc = rank_ok && (t.m - c_tgt <= tau);
-      if (lane == 0 && !acc) a.out_tokens[(size_t)b * a.Ko + i] = t.idx;   // the correction, if first failure
+      if (write && lane == 0 && !acc) a.out_tokens[(size_t)b * a.Ko + i] = t.idx;   // the correction, if first failure
     } else {
       const float p = e_p * sc_t * inv_st;                      // e^(c - M) / sum e^(z - M)
       const float q = MODE == kModeVerify ? e_q : e_q * qscale;
