@@ -56,7 +56,7 @@ def peaks():
         return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("cmsd_stream_impl.cuh", "cmsd_device.cuh", "cmsd_internal.h")
+KERNEL_SOURCES = ("cmsd_stream_impl.cuh", "cmsd_seq_impl.cuh", "cmsd_device.cuh", "cmsd_internal.h")
 
 
 def measured_peaks():
@@ -91,7 +91,7 @@ def ncu_traffic(workload, rule):
         recs = recs if isinstance(recs, list) else [recs]
         for d in recs:
             if d.get("workload") == workload and d.get("rule") == rule and \
-                    d.get("kernel", "").startswith("stream_kernel") and \
+                    d.get("kernel", "").startswith(("stream_kernel", "seq_kernel")) and \
                     d.get("sources_sha256_16") == kernel_sources_sha():
                 return d.get("bytes_per_launch")
     except Exception:
@@ -778,7 +778,8 @@ def run_ours(args):
         "step_ms": step_stats,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": ncu_traffic(WORKLOAD, args.rule),
-                     "kernel": "stream_kernel (fused confidence + verify pass)",
+                     "kernel": "stream_kernel (fused confidence + verify pass)" if sampled
+                     else "seq_kernel (the pass in one launch)",
                      "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)" if peak_src == "measured"
                      else "fallback 6800 GB/s",
                      "algorithmic_bytes_per_launch": alg_bytes, "kernel_ms": k_med,

@@ -28,9 +28,13 @@
  *     device can see (a drafted token outside [0, V), k_row outside [0, K]) are
  *     clamped before any load and recorded in the workspace;
  *     cmsd_workspace_errors reads them.
- *   - Calls that draw a residual token (CMSD_RULE_SAMPLED) or use the bonus row
- *     launch a second kernel after the streaming kernel, on the same stream,
- *     which makes a second pass over one row of each sequence that needs it.
+ *   - Calls with windows of at most 16 positions and small or medium sizes run
+ *     as one kernel (a thread-block cluster per sequence); the rest as a
+ *     streaming kernel and, when they draw a residual token
+ *     (CMSD_RULE_SAMPLED) or use the bonus row, a second kernel on the same
+ *     stream, which makes a second pass over one row of each sequence that
+ *     needs it.  Results do not depend on the choice but for the rounding of
+ *     32-bit sums.
  *   - Logits must be finite or -inf (masked vocabulary entries, probability 0);
  *     |logit| < 1e29; every row needs at least one finite logit.  +inf and NaN
  *     give unspecified results.
@@ -284,8 +288,8 @@ int cmsd_philox_fill(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint3
 
 /* Kernel timing: while enabled, each cmsd_confidence / cmsd_verify /
  * cmsd_confidence_verify call records CUDA events on its stream around its
- * streaming kernel and around its resample kernel (sampled rule or bonus
- * row), for up to max_calls calls.  cmsd_profile_stop synchronises those
+ * streaming kernel (or its only kernel) and around its second kernel (sampled
+ * rule or bonus row), for up to max_calls calls.  cmsd_profile_stop synchronises those
  * events and writes, per call, the streaming-kernel time and the
  * resample-kernel time in milliseconds (0 when there was none); either array
  * may be NULL; *n_out receives the number of calls recorded.  An event

@@ -96,7 +96,7 @@ size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
   size_t err, row_done, seq_word, seq_done, rec_count, res_cta_done, res_done;
-  size_t rec, row_conf, row_acc, row_targmax, row_dstat, row_tstat, part, rpart;
+  size_t rec, row_conf, row_acc, row_dstat, row_tstat, part, rpart;
   size_t total;
 };
 
@@ -116,7 +116,6 @@ Layout make_layout(int B, int K, int wmax) {
   L.rec = o; o += up((size_t)B * sizeof(int4));
   L.row_conf = o; o += up(BK * sizeof(unsigned long long));
   L.row_acc = o; o += up(BK * sizeof(int));
-  L.row_targmax = o; o += up(BK * sizeof(int));
   L.row_dstat = o; o += up(BK * sizeof(float2));
   L.row_tstat = o; o += up(BK * sizeof(float2));
   L.part = o; o += up((BK + (size_t)wmax) * sizeof(Partial));
@@ -138,7 +137,6 @@ Workspace carve(void* ws, const Layout& L) {
   W.rec = (int4*)(p + L.rec);
   W.row_conf = (unsigned long long*)(p + L.row_conf);
   W.row_acc = (int*)(p + L.row_acc);
-  W.row_targmax = (int*)(p + L.row_targmax);
   W.row_dstat = (float2*)(p + L.row_dstat);
   W.row_tstat = (float2*)(p + L.row_tstat);
   W.part = (Partial*)(p + L.part);

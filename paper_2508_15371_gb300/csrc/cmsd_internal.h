@@ -75,7 +75,6 @@ struct Workspace {
   int4* rec;                      // [B]   queued rows: (b, position, kind, 0)
   unsigned long long* row_conf;   // [B*K] C of each position, fixed point C * 2^36
   int* row_acc;                   // [B*K] accept bit (K > 16 epilogue)
-  int* row_targmax;               // [B*K] verifier argmax
   float2* row_dstat;              // [B*K] drafter (max * log2e, sum e^(z-max))
   float2* row_tstat;              // [B*K] target  (the same)
   Partial* part;                  // [B*K + warps]

@@ -1,16 +1,20 @@
-// Streaming kernel of the CM-ASD logits pass (sm_103a).
+// Streaming kernel of the CM-ASD logits pass (sm_103a), the second pass of the
+// calls it takes, and the arithmetic that the one-launch pass
+// (cmsd_seq_impl.cuh) shares with it.
 //
 // Work split.  The present rows (sequence b, drafted position i < k_row[b])
 // are laid end to end into one stream of rows * V logits per tensor, and the
-// launched warps (a persistent grid: one 768-thread CTA per SM) each take one
+// launched warps (a persistent grid: one 512-thread CTA per SM) each take one
 // contiguous slice of that stream: whole-warp pieces of one row when there are
-// at least as many warps as rows, equal runs of 16-byte vectors otherwise.
-// Each piece of a row inside a slice is a "segment".
+// at least as many warps as rows (and that keeps three quarters of them busy),
+// equal runs of 128-byte lines otherwise.  Each piece of a row inside a slice
+// is a "segment".
 //
 // Memory pipeline.  A lane's 16-byte vectors in a segment are those with index
 // lane + 32 t; it reads CMSD_UNROLL of each tensor per stage with streaming
 // loads (ld.global.nc, no L1 allocation) into registers, and issues the loads
-// of stage s + 1 before it reduces stage s, so one stage is always in flight.
+// of stage s + 1 before it reduces stage s, so one stage is always in flight
+// (pipe_run).
 // The unaligned head and tail of a segment (under 16 bytes each) are read
 // element by element.
 //
@@ -40,14 +44,20 @@
 // Second pass.  Under the sampled rule the rejected position's token is drawn
 // from the residual max(0, p - q), and with the bonus row the verifier's extra
 // row gives a token when every draft was accepted; both need one more pass
-// over one row of the sequence after its epilogue.  The epilogue queues a
-// record for each sequence that needs one; a second kernel, launched as a
-// programmatic dependent of this one, drains the queue: under the sampled rule
-// without the bonus row, resample_bound_kernel (a cluster of CTAs per row that
-// bounds each group's residual mass by its largest target logit and races
-// only the groups the bound leaves in play); otherwise resample_kernel (the
-// queued rows' groups split evenly over its warps, every group raced).  Every
-// logit of the pass proper is read once.
+// over one row of the sequence after its epilogue, made by a second kernel
+// launched as a programmatic dependent of this one.  The epilogue releases a
+// record word at the sequence's own slot, which a cluster of CTAs polls; the
+// cluster bounds each group's mass by its largest target logit and races only
+// the groups the bound leaves in play (resample_bound_kernel, which stages its
+// share of the row, for few sequences; draw_kernel for many, and for the bonus
+// row).  Rows whose share does not fit shared memory go to resample_kernel:
+// the epilogue queues a record, and the queued rows' groups are split evenly
+// over its warps, every group raced.  Every logit of the pass proper is read
+// once.
+//
+// Bound, on a GB300: DRAM while it streams (B=64 K=8 V=128256 bf16, sampled: the
+// slices of 262.7 MB end 37 us into the launch, median, 7.1 TB/s; the last at
+// 43), then the chain of the last rows, and the draw (54 us a call).
 //
 // -inf logits (masked vocabulary) are clamped to -2^100 before the drafter
 // arithmetic so that e^(z-m) * (z-m) is 0, not NaN.
@@ -521,14 +531,14 @@ __device__ __forceinline__ int next_k(const StreamArgs& a, unsigned long long cs
   return k < a.k_min ? a.k_min : k;
 }
 
-// The word of sequence b's record that the bounded residual draw polls:
+// The word of sequence b's record that the draw by group bounds polls:
 // valid bit | kind << 1 | rejected position << 3.
 __device__ __forceinline__ unsigned* rec_word(const Workspace& W, int b) {
   return reinterpret_cast<unsigned*>(W.rec + b) + 3;
 }
 
 // Queue the sequence's second-pass record, if it needs one; or, for the
-// bounded residual draw, release it (kSeqNone included) at the sequence's own
+// draw by group bounds, release it (kSeqNone included) at the sequence's own
 // slot: one word that the draw polls, written after every other write of the
 // epilogue (the caller's warp has synchronised) and, through the row
 // counters, of the sequence's rows.

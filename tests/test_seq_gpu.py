@@ -123,3 +123,25 @@ def test_device_errors_are_reported(cmsd):
     tok[1, 2] = 0
     cmsd.confidence_verify(d, t, tok, p=p, ws=ws, k_row=torch.tensor([4, -1, 5], dtype=torch.int32, device="cuda"))
     assert cmsd.workspace_errors(ws) == 2
+
+
+@pytest.mark.parametrize("noise,bonus", [(1.0, False), (0.0, False), (1.0, True)])
+def test_rows_beyond_every_share(cmsd, noise, bonus):
+    """Rows whose share fits no CTA's shared memory take the race over every
+    group (noise 0: target equal to drafter, whose empty residual is the
+    target's argmax)."""
+    from parity_util import bonus_view, compare, gpu_fused, oracle_fused
+    from paper_2508_15371_gb300 import workloads as W
+    B, K, V = 2, 2, 3_100_000
+    rng = np.random.default_rng(3)
+    d = rng.normal(0, 1.0, (B, K + 1, V)).astype(np.float32)
+    t = d + np.float32(noise) * rng.normal(0, 1.0, d.shape).astype(np.float32) if noise else d.copy()
+    t[:, :, 77] += 9.0 if noise else 0.0
+    Kt = K + 1 if bonus else K
+    tok = rng.integers(0, V, (B, K)).astype(np.int32)
+    w = W.Workload(name="wide", B=B, K=K, V=V, dtype="bf16", draft=W.f32_to_bf16_bits(d[:, :K]),
+                   target=W.f32_to_bf16_bits(t[:, :Kt]), tokens=tok, seed=5)
+    p = cmsd.params(K, "sampled", bonus=bonus, tau_base=30.0 if bonus else -5.0)
+    g = gpu_fused(cmsd, torch, w, p, iteration=2)
+    compare(w, g, oracle_fused(w, p, iteration=2))
+    assert (g["n_accept"] == K).any() if bonus else (g["n_accept"] < K).any()
