@@ -70,6 +70,122 @@ struct __align__(16) SeqRow {
   int acc, pad;
 };
 
+// The draw of cluster_draw by racing every group of the share exactly, for
+// shares of at most Q blocks of four groups per lane set: each lane set holds
+// the vectors of its groups in registers, so the row's two loads, the keys
+// and one exchange are the whole chain (cluster_draw: maxima, bounds, probes, an
+// exchange, the groups that remain, the exchange).  Against cluster_draw, in
+// us a call: B=4 K=8 V=128256 (16 CTAs) 13.8 -> 12.5, B=16 K=4 V=32000 11.4
+// -> 10.1, with the bonus row B=8 K=8 V=128256 18.9 -> 14.9 and B=32 (Q = 2)
+// 31.8 -> 30.8.  More than eight groups per lane set cost more exponentials
+// than the bounds save; so do rows off 16-byte boundaries at Q = 2 (verify
+// B=96 K=12 V=32001 ragged: 21.0 against 22.6), which take two loads and a
+// shift per vector.
+//
+// Four groups' sums per block are reduced by exchanging halves (lane bit 0,
+// then bit 1), which leaves group k's in the lanes with sub & 3 == k, and
+// every sum is formed in the order of group_key.
+template <typename T, int NT, int Q>
+__device__ __forceinline__ void cluster_race(const StreamArgs& a, cg::cluster_group& cl, int nc, int cr, int b, int pos,
+                                             bool bonus, const T* tp, const T* dp, float2 ts, float2 ds,
+                                             DrawShared<T, NT>& sh) {
+  constexpr int VEC = Elem<T>::kVec;
+  constexpr int LPG = DrawShared<T, NT>::kLpg;
+  constexpr int SETS = DrawShared<T, NT>::kSets;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sub = lane % LPG, set = tid / LPG;
+  const int ng = (a.V + kGroup - 1) / kGroup;
+  const int ngs = draw_share(ng, nc);
+  const int gs = cr * ngs;                                   // the share: groups [gs, gs + nloc)
+  const int nloc = max(0, min(ng, gs + ngs) - gs);
+  const uint32_t k0 = seed_lo(a.seed), k1 = seed_hi(a.seed);
+  const uint32_t cw_grp = iter_word(a.iteration, kPurposeGroup);
+  const uint32_t cw_ent = iter_word(a.iteration, kPurposeResidual);
+  const bool vec_ok = ((((uintptr_t)tp) | ((uintptr_t)dp)) & 15) == 0;
+  // block q of the lane set: groups 4 (set + q SETS) .. + 3 of the share
+  uint4 qt[4 * Q], qd[4 * Q];
+#pragma unroll
+  for (int j = 0; j < 4 * Q; ++j) {
+    const int gl = 4 * (set + j / 4 * SETS) + j % 4;
+    qt[j] = gl < nloc ? load_logits<T>(tp, (gs + gl) * kGroup + sub * VEC, a.V, vec_ok) : neg_inf_vec<T>();
+    qd[j] = bonus ? make_uint4(0, 0, 0, 0) : neg_inf_vec<T>();
+    if (!bonus && gl < nloc) qd[j] = load_logits<T>(dp, (gs + gl) * kGroup + sub * VEC, a.V, vec_ok);
+  }
+  float e[Q];                            // the exponential of the lane's group of each block
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const U4 wd = philox4x32_10(U4{(uint32_t)(gs / 4 + set + q * SETS), (uint32_t)b, (uint32_t)pos, cw_grp}, k0, k1);
+    const int k = sub & 3;
+    e[q] = expo(k == 0 ? wd.x : k == 1 ? wd.y : k == 2 ? wd.z : wd.w);
+  }
+  if (tid == 0) {
+    sh.best[0] = ~0ull;
+    sh.am = 0ull;
+  }
+  RowStat st{ts.x, 1.0f / ts.y, ds.x, -1.0f / ds.y};
+  if (bonus) {                           // p relative to the row's largest logit
+    float m = -pos_inf();
+#pragma unroll
+    for (int j = 0; j < 4 * Q; ++j) m = fmaxf(m, vec_max(qt[j], (const T*)nullptr));
+    m = warp_max(m);
+    if (lane == 0) sh.wmax[warp] = m;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NT / 32; ++k) m = fmaxf(m, sh.wmax[k]);
+    if (tid < nc) *cl.map_shared_rank(&sh.ref[cr], tid) = m;
+    cluster_sync();
+    for (int c = 0; c < nc; ++c) m = fmaxf(m, sh.ref[c]);
+    st = RowStat{mlog2e(m), 1.0f, 0.f, 0.f};
+  } else {
+    __syncthreads();
+  }
+  float key = pos_inf();
+  int grp = kIntMax;
+  const bool up1 = (sub & 1) != 0, up2 = (sub & 2) != 0;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    float s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = resid_vec<T>(qt[4 * q + k], qd[4 * q + k], st);
+    const float x0 = (up1 ? s[1] : s[0]) + __shfl_xor_sync(kFull, up1 ? s[0] : s[1], 1);   // group 0 or 1
+    const float x1 = (up1 ? s[3] : s[2]) + __shfl_xor_sync(kFull, up1 ? s[2] : s[3], 1);   // group 2 or 3
+    float acc = (up2 ? x1 : x0) + __shfl_xor_sync(kFull, up2 ? x0 : x1, 2);
+    if (LPG == 8) acc += __shfl_xor_sync(kFull, acc, 4);
+    const int gl = 4 * (set + q * SETS) + (sub & 3);
+    const float kq = (gl < nloc && acc > 0.f) ? e[q] / acc : pos_inf();
+    if (kq < key) {                      // (a later block's groups are higher: ties keep the lower)
+      key = kq;
+      grp = gs + gl;
+    }
+  }
+  // the CTA's least (key, group); the warp that holds that group races its
+  // entries and pushes the result to rank 0 of the cluster
+  key_min_cta(key, grp, &sh.best[0]);
+  const int gw = grp != kIntMax ? grp - gs : 0;
+  const int hs = gw / 4 % SETS;          // the lane set that holds it
+  if (warp == hs * LPG / 32) {
+    int tok = -1;
+    if (grp != kIntMax) {
+      const int j = gw / 4 / SETS * 4 + gw % 4;
+      uint4 vt = qt[0], vd = qd[0];
+#pragma unroll
+      for (int k = 1; k < 4 * Q; ++k)
+        if (j == k) {
+          vt = qt[k];
+          vd = qd[k];
+        }
+      tok = race_group_entries<T>(vt, vd, grp, hs * LPG % 32, lane, st, (uint32_t)b, (uint32_t)pos, cw_ent, k0, k1);
+    }
+    if (lane == 0) {
+      *cl.map_shared_rank(&sh.rk[cr], 0) = key;
+      *cl.map_shared_rank(&sh.rg[cr], 0) = grp;
+      *cl.map_shared_rank(&sh.rt[cr], 0) = tok;
+    }
+  }
+  cluster_sync();                        // every CTA's result is in rank 0
+  if (cr == 0) draw_result<T, NT>(a, nc, b, pos, tp, vec_ok, sh);
+}
+
 template <typename T, int NT, int MODE, bool SAMPLED, bool SECOND>
 __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, const __grid_constant__ SeqSplit sp) {
   constexpr int NW = NT / 32;
@@ -232,7 +348,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     const bool bonus = kind == kSeqBonus;
     const float4 q = bonus ? make_float4(0.f, 1.f, 0.f, 1.f) : s_row[n].stat;
     const T* dp = bonus ? tp : (const T*)a.draft + ((size_t)b * a.K + n) * (size_t)a.V;
-    cluster_draw<T, NT, 4>(a, cl, nc, cr, b, n, bonus, tp, dp, make_float2(q.z, q.w), make_float2(q.x, q.y), s_u, sh);
+    const float2 ts = make_float2(q.z, q.w), ds = make_float2(q.x, q.y);
+    const int ngs = draw_share((a.V + kGroup - 1) / kGroup, nc);
+    const bool aligned = ((((uintptr_t)tp) | ((uintptr_t)dp)) & 15) == 0;
+    if (ngs <= 4 * DrawShared<T, NT>::kSets)
+      cluster_race<T, NT, 1>(a, cl, nc, cr, b, n, bonus, tp, dp, ts, ds, sh);
+    else if (aligned && ngs <= 8 * DrawShared<T, NT>::kSets)
+      cluster_race<T, NT, 2>(a, cl, nc, cr, b, n, bonus, tp, dp, ts, ds, sh);
+    else
+      cluster_draw<T, NT, 4>(a, cl, nc, cr, b, n, bonus, tp, dp, ts, ds, s_u, sh);
   }
 }
 

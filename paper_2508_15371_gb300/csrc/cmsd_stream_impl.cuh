@@ -1810,6 +1810,27 @@ __host__ __device__ inline size_t draw_smem_bytes(int V, int nc) {
   return (size_t)draw_share((V + kGroup - 1) / kGroup, nc) * 2 * sizeof(float);
 }
 
+// Rank 0 of the cluster: the row's token from the CTAs' (key, group, token),
+// the verifier row's argmax if no group of the row has residual mass.
+template <typename T, int NT>
+__device__ __forceinline__ void draw_result(const StreamArgs& a, int nc, int b, int pos, const T* tp, bool vec_ok,
+                                            DrawShared<T, NT>& sh) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    const float k = lane < nc ? sh.rk[lane] : pos_inf();
+    const int g = lane < nc ? sh.rg[lane] : kIntMax;
+    const uint32_t kb = __reduce_min_sync(kFull, __float_as_uint(k));      // keys are >= 0 or +inf
+    const uint32_t gb = __reduce_min_sync(kFull, __float_as_uint(k) == kb ? (uint32_t)g : 0xFFFFFFFFu);
+    const unsigned who = __ballot_sync(kFull, __float_as_uint(k) == kb && (uint32_t)g == gb);
+    const int c = __ffs(who) - 1;
+    if (lane == 0) sh.fb = (gb == (uint32_t)kIntMax || sh.rt[c] < 0) ? -1 : sh.rt[c];
+  }
+  __syncthreads();
+  int tok = sh.fb;
+  if (tok < 0) tok = row_argmax_cta<T, NT>(tp, a.V, vec_ok, &sh.am);   // empty residual: the argmax
+  if (threadIdx.x == 0) a.out_tokens[(size_t)b * a.Ko + pos] = tok;
+}
+
 // UL: vectors in flight per thread of the maxima pass.  ts, ds: the row's
 // target and drafter (max * log2e, sum).
 template <typename T, int NT, int UL>
@@ -1973,21 +1994,7 @@ __device__ void cluster_draw(const StreamArgs& a, cg::cluster_group& cl, int nc,
     }
   }
   cluster_sync();                             // every CTA's result is in rank 0
-  if (cr == 0) {
-    if (warp == 0) {
-      float k = lane < nc ? sh.rk[lane] : pos_inf();
-      const int g = lane < nc ? sh.rg[lane] : kIntMax;
-      const uint32_t kb = __reduce_min_sync(kFull, __float_as_uint(k));      // keys are >= 0 or +inf
-      const uint32_t gb = __reduce_min_sync(kFull, __float_as_uint(k) == kb ? (uint32_t)g : 0xFFFFFFFFu);
-      const unsigned who = __ballot_sync(kFull, __float_as_uint(k) == kb && (uint32_t)g == gb);
-      const int c = __ffs(who) - 1;
-      if (lane == 0) sh.fb = (gb == (uint32_t)kIntMax || sh.rt[c] < 0) ? -1 : sh.rt[c];
-    }
-    __syncthreads();
-    int tok = sh.fb;
-    if (tok < 0) tok = row_argmax_cta<T, NT>(tp, a.V, vec_ok, &sh.am);   // empty residual: the argmax
-    if (tid == 0) a.out_tokens[(size_t)b * a.Ko + pos] = tok;
-  }
+  if (cr == 0) draw_result<T, NT>(a, nc, b, pos, tp, vec_ok, sh);
 }
 
 // The extra verifier row's argmax (PAPER rule, bonus row; lowest index), each

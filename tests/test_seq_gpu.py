@@ -70,9 +70,11 @@ def _same(narrow, wide, k_row, bonus):
 
 
 # Sizes: no whole vector, one group, lines and pieces that end inside a row,
-# the cluster sizes of the rule (1 to 16 CTAs of 256 or 512 threads).
+# the cluster sizes of the rule (1 to 16 CTAs of 256 or 512 threads), draws of
+# one and of two blocks of groups per lane set (B=32) and by bounds (B=64).
 SHAPES = [(1, 1, 2), (3, 2, 33), (2, 16, 1000), (1, 4, 32000), (5, 7, 4099), (8, 8, 32128), (40, 3, 8193),
-          (70, 5, 6400), (150, 2, 4096), (700, 1, 2048), (2, 8, 128256)]
+          (70, 5, 6400), (150, 2, 4096), (700, 1, 2048), (2, 8, 128256),
+          (32, 2, 64128), (32, 2, 128256), (64, 2, 128255)]
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
