@@ -232,8 +232,9 @@ void fill_sizes(StreamArgs& a, int B, int K, int V) {
 }
 
 // CTAs per cluster that choose_seq weighs.
-constexpr int kSeqSizes[] = {1, 2, 3, 4, 5, 6, 8, 16};
-constexpr int kSeqNumSizes = 8;
+constexpr int kSeqSizes[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 16};
+constexpr int kSeqNumSizes = 12;
+constexpr int kModelWarps = 152 * 16;      // the streaming kernel's warps on a GB300
 
 // Clusters of seq_kernel that can be resident on device dev, which is current
 // (cached; n: index into kSeqSizes).
@@ -253,48 +254,75 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 //
 // Both times are estimated, in microseconds, from what was measured on a
 // GB300 over K = 1..16, V = 32000..152064, B = 1..600 (bf16; f32 alike):
-//   streaming kernel   9 + bytes / 6900 MB/s, and with a second launch 7.5
-//     more (14 for the bonus race over every group) and 0.045 (0.09) per
+//   streaming kernel   8 + bytes / 6900 MB/s, more when whole rows leave over
+//     a tenth of the warps without one (B=80 K=8 V=128256: 67.9), and with a
+//     second launch 7.5 more (12 with the bonus row) and 0.045 (0.09) per
 //     sequence beyond 64;
-//   one launch         5, a draw 4.5, and the time of a sequence's bytes
-//     through its CTAs (a CTA of 256 threads: 27 KB a microsecond under the
-//     PAPER rule, 21 with the target's exponentials or the drafter alone, 30
-//     for the target alone; one of 512 twice that), times the waves when not
-//     every cluster is resident (3.5 more each, 10 with clusters of several
-//     CTAs: B=192 K=12 V=32001 verify took 37 us in two waves of three,
-//     31.6 streamed), and no less than the bytes at 6900 MB/s.
+//   one launch         5, a draw 3.5 (4.5 by cluster_draw), and the time of a
+//     sequence's bytes through its CTAs (a CTA of 256 threads: 27 KB a
+//     microsecond under the PAPER rule, 23.5 under the sampled rule, 21 for
+//     the drafter alone, 30 for the target alone (39 under the PAPER rule when
+//     windows are ragged, a fifth less off 16-byte boundaries); one of 512
+//     twice that; a tenth more with an SM to itself, three tenths more when
+//     both tensors' windows are ragged and neighbours end early), times the
+//     waves when not every cluster is resident (3.5 more each, 10 with
+//     clusters of several CTAs), and no less than the bytes at 6900 MB/s.
 // Ragged windows are unknown here: half full on average, and the longest
-// decides the one-launch pass, since a sequence keeps to its cluster.
+// decides the one-launch pass, since a sequence keeps to its cluster; a tenth
+// more clusters than are resident find places as the shorter windows end
+// (B=48 K=12 V=32001 verify: 13.6 with 46 clusters of six resident, 15.7 with
+// clusters of five).
+//
+// Full windows need every cluster resident at once, and not all of the number
+// that the occupancy query names are: clusters of 256-thread CTAs left some
+// waiting above 93 in 100 of it (B=97 K=4 V=128256 by threes: 48.3 against
+// 35.4 streamed; B=90: 32.1), odd clusters of 512-thread CTAs, each with an SM
+// to itself, near the limit (B=28 K=8 by fives: 40.7 against 33.2; B=26:
+// 27.0), even ones not (SMs come in pairs).  Measured on both sides, K=8
+// V=128256 sampled, streamed and in one launch: B=16 26.1, 24.3 (clusters of
+// twelve); B=36 37.2, 30.8 (four of 512); B=44 42.1, 38.4 (three of 512); B=64
+// 54.2, 53.4; B=72 58.0, 54.8 (two of 512); B=48 43.6, 44.7.
 bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int* nc, int* threads) {
   if (a.K > kPackedMaxK || (second && sampled && !seq_draw_fits(dtype, a.V))) return false;
   const double kb = (double)a.K * a.V * (dtype == CMSD_F32 ? 4 : 2) * (mode == kModeFused ? 2 : 1) * 1e-3;
   const double stream = a.B * kb * (a.k_row ? 0.5 : 1.0) / 6900;
-  double flat = 9 + stream;
+  double flat = 8 + stream;
+  if (!a.k_row && a.B * a.K < kModelWarps) {             // (the rows' warps, whole rows apart from the rest)
+    const double used = (double)(kModelWarps / (a.B * a.K)) * (a.B * a.K) / kModelWarps;
+    if (used >= 0.75 && used < 0.9) flat += stream * 0.5 * (0.9 - used);
+  }
   if (second) {
-    flat += a.bonus ? 14 : 7.5;
+    flat += a.bonus ? 12 : 7.5;
     if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 0.09 : 0.045);
   }
-  const double rate = mode == kModeVerify ? 30 : (mode == kModeFused && !sampled ? 27 : 21);
-  const double fixed = 5 + (second ? 4.5 : 0);
+  const int per = dtype == CMSD_F32 ? 4 : 8;             // entries per 16-byte vector
+  double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 39) : (sampled ? 23.5 : 27));
+  if (mode == kModeVerify && a.V % per != 0) rate *= 0.8;   // rows off 16-byte boundaries
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  double best = 0.97 * flat;               // (a near tie stays with the streaming kernel)
+  double best = 0.985 * flat;              // (a near tie stays with the streaming kernel)
   *nc = 0;
   for (int th = 256; th <= 512; th *= 2) {
     for (int k = 0; k < kSeqNumSizes; ++k) {
       const int n = kSeqSizes[k];
       // at least two 16-byte vectors per lane and piece, or more CTAs gain nothing
       if (n > 1 && kb * 1e3 < (double)n * (th / 32) * 1024 * (mode == kModeFused ? 2 : 1)) break;
-      const double part = kb / n / (rate * (th / 256));
-      if (fixed + part >= best) continue;
+      const bool race = a.V <= (int64_t)8 * n * th * per;
+      const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + (second ? (sampled && !race ? 4.5 : 3.5) : 0);
+      const double full = kb / n / (rate * (th / 256));
+      if (fixed + full / 1.3 >= best) continue;
       const int res = seq_resident(dev, dtype, k, th);
       if (res < 1) continue;
-      // (clusters of 3 and more were not all placed at once near the limit; of
-      // ragged windows some end early)
-      const int fit = n >= 3 && !a.k_row ? (res * 9 + 9) / 10 : res;
+      int fit = res;
+      if (a.k_row) fit += res / 10;
+      else if (th == 512 && (n & 1)) fit = res * 96 / 100;
+      else if (th == 256 && n >= 3) fit = res * 93 / 100;
       const int waves = (a.B + fit - 1) / fit;
-      const double t = fixed + (th == 512 ? 0.7 : 0.0) + (n == 1 ? 3.5 : 10.0) * (waves - 1) +
-                       (waves * part > stream ? waves * part : stream);
+      // an SM to itself, or neighbours that end early
+      const bool early = a.k_row && mode == kModeFused && waves == 1;
+      const bool apart = a.B * n * (th / 256) <= kModelWarps / 16;
+      const double part = full / (early ? 1.3 : (apart ? 1.1 : 1.0));
+      const double t = fixed + (n == 1 ? 3.5 : 10.0) * (waves - 1) + (waves * part > stream ? waves * part : stream);
       if (t < best) {
         best = t;
         *nc = n;
