@@ -20,14 +20,25 @@ constexpr uint32_t kGenSpike = 0xC0000004u;
 // One CTA of 1024 threads per row left a second wave of a few rows on 152 SMs
 // and staged the table with one entry per load: 160 rows of 32000 took 21.6 us.
 // Two parts of 512 threads took 17.5, four of 256 16.4, and with vector loads
-// of the table 15.8.
+// of the table 15.8.  Two 16-byte stores per thread left every store of a
+// warp writing half sectors; with 32-byte stores, and the active slots first,
+// 13.5 (32 windows of 5 rows on average, 41 MB written).
 constexpr int kParts = 4;
 constexpr int kThreads = 256;
 constexpr int kTableBits = 13;   // the normal table: 2^13 float32, staged in shared memory
 
-__device__ __forceinline__ uint32_t half16(const cmsd::U4& w, int j) {
-  const uint32_t word = (j >> 1) == 0 ? w.x : (j >> 1) == 1 ? w.y : (j >> 1) == 2 ? w.z : w.w;
-  return (j & 1) ? (word >> 16) : (word & 0xFFFFu);
+// The table entry that a 16-bit half of a word names by its top bits.
+__device__ __forceinline__ float table_at(const float* table, uint32_t word, int half) {
+  constexpr uint32_t mask = ((1u << kTableBits) - 1) << 2;               // byte offsets
+  const uint32_t at = (half ? word >> (30 - kTableBits) : word >> (14 - kTableBits)) & mask;
+  return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(table) + at);
+}
+
+// 32 bytes, one whole sector, in one store (p on a 32-byte boundary).
+__device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]),
+               "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7])
+               : "memory");
 }
 
 // One cluster per (b, i) slot of the [B][Kt] verifier layout.
@@ -42,8 +53,8 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int slot = blockIdx.x / kParts, part = blockIdx.x - slot * kParts;
-  const int b = slot / Kt;
-  const int i = slot - b * Kt;
+  const int i = slot / B;                       // position-major: the idle slots come last
+  const int b = slot - i * B;
   int k = K_max;
   if (k_row) {
     k = k_row[b];
@@ -71,23 +82,34 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
   float best = -__int_as_float(0x7F800000);
   int bidx = 0x7FFFFFFF;
   const int ngrp = (V + 7) / 8;
-  // rows start on 16-byte boundaries when V is a multiple of 4: each thread
-  // then writes its 8 logits as two 16-byte stores
+  // rows start on 32-byte boundaries when V is a multiple of 8 and the tensors
+  // do: each thread then writes its 8 logits in one store; on 16-byte ones when
+  // V is a multiple of 4: two stores
   const bool vec = (V & 3) == 0;
+  const bool vec8 = (V & 7) == 0 && ((((uintptr_t)draft) | ((uintptr_t)target)) & 31) == 0;
   for (int g = part * kThreads + threadIdx.x; g < ngrp; g += kParts * kThreads) {
     const cmsd::U4 wd = cmsd::philox4x32_10(cmsd::U4{(uint32_t)g, (uint32_t)row, it, kGenDNoise}, k0, k1);
     const cmsd::U4 wt = cmsd::philox4x32_10(cmsd::U4{(uint32_t)g, (uint32_t)row, it, kGenTNoise}, k0, k1);
+    const uint32_t dw[4] = {wd.x, wd.y, wd.z, wd.w}, tw[4] = {wt.x, wt.y, wt.z, wt.w};
     float zs[8], ts[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int v = 8 * g + j;
-      float z = s_table[half16(wd, j) >> (16 - kTableBits)];
+      float z = table_at(s_table, dw[j >> 1], j & 1);
       if (v == spike) z = __fadd_rn(z, h);
       zs[j] = z;
-      ts[j] = __fadd_rn(z, __fmul_rn(0.8f, s_table[half16(wt, j) >> (16 - kTableBits)]));
-      if (v < V && z > best) { best = z; bidx = v; }
+      ts[j] = __fadd_rn(z, __fmul_rn(0.8f, table_at(s_table, tw[j >> 1], j & 1)));
     }
-    if (vec && 8 * g + 8 <= V) {
+    float m = -__int_as_float(0x7F800000);       // the group's maximum and its lowest place
+    int mj = 0;
+#pragma unroll
+    for (int j = 7; j >= 0; --j)
+      if (8 * g + j < V && zs[j] >= m) { m = zs[j]; mj = j; }
+    if (m > best) { best = m; bidx = 8 * g + mj; }
+    if (vec8) {
+      if (has_draft) store8(dz + 8 * g, zs);
+      store8(tz + 8 * g, ts);
+    } else if (vec && 8 * g + 8 <= V) {
       float4* d4 = reinterpret_cast<float4*>(dz + 8 * g);
       float4* t4 = reinterpret_cast<float4*>(tz + 8 * g);
       if (has_draft) {

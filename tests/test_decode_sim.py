@@ -36,7 +36,7 @@ def test_summarize_counts(mods):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("bonus", [0, 1])
-@pytest.mark.parametrize("V,k_row", [(1000, [5, 2, 0]), (4099, [1, 5, 3])])
+@pytest.mark.parametrize("V,k_row", [(1000, [5, 2, 0]), (1004, [3, 0, 5]), (4099, [1, 5, 3])])
 def test_device_generator_matches_host(mods, V, k_row, bonus):
     cmsd, ds, W = mods
     assert torch.cuda.is_available()
