@@ -287,7 +287,7 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
   const double kb = (double)a.K * a.V * (dtype == CMSD_F32 ? 4 : 2) * (mode == kModeFused ? 2 : 1) * 1e-3;
   const double stream = a.B * kb * (a.k_row ? 0.5 : 1.0) / 6900;
   double flat = 8 + stream;
-  if (!a.k_row && a.B * a.K < kModelWarps) {             // (the rows' warps, whole rows apart from the rest)
+  if (!a.k_row && (int64_t)a.B * a.K < kModelWarps) {             // (the rows' warps, whole rows apart from the rest)
     const double used = (double)(kModelWarps / (a.B * a.K)) * (a.B * a.K) / kModelWarps;
     if (used >= 0.75 && used < 0.9) flat += stream * 0.5 * (0.9 - used);
   }
@@ -317,10 +317,10 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       if (a.k_row) fit += res / 10;
       else if (th == 512 && (n & 1)) fit = res * 96 / 100;
       else if (th == 256 && n >= 3) fit = res * 93 / 100;
-      const int waves = (a.B + fit - 1) / fit;
+      const int waves = (a.B - 1) / fit + 1;
       // an SM to itself, or neighbours that end early
       const bool early = a.k_row && mode == kModeFused && waves == 1;
-      const bool apart = a.B * n * (th / 256) <= kModelWarps / 16;
+      const bool apart = (int64_t)a.B * n * (th / 256) <= kModelWarps / 16;
       const double part = full / (early ? 1.3 : (apart ? 1.1 : 1.0));
       const double t = fixed + (n == 1 ? 3.5 : 10.0) * (waves - 1) + (waves * part > stream ? waves * part : stream);
       if (t < best) {
