@@ -279,9 +279,9 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // 35.4 streamed; B=90: 32.1), odd clusters of 512-thread CTAs, each with an SM
 // to itself, near the limit (B=28 K=8 by fives: 40.7 against 33.2; B=26:
 // 27.0), even ones not (SMs come in pairs).  Measured on both sides, K=8
-// V=128256 sampled, streamed and in one launch: B=16 26.1, 24.3 (clusters of
-// twelve); B=36 37.2, 30.8 (four of 512); B=44 42.1, 38.4 (three of 512); B=64
-// 54.2, 53.4; B=72 58.0, 54.8 (two of 512); B=48 43.6, 44.7.
+// V=128256 sampled, streamed and in one launch: B=16 26.1, 22.6 (clusters of
+// twelve); B=32 35.6, 30.2 (of eight); B=40 39.4, 38.0 (of three with 512
+// threads); B=64 54.2, 52.8 (of four).
 bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int* nc, int* threads) {
   if (a.K > kPackedMaxK || (second && sampled && !seq_draw_fits(dtype, a.V))) return false;
   const double kb = (double)a.K * a.V * (dtype == CMSD_F32 ? 4 : 2) * (mode == kModeFused ? 2 : 1) * 1e-3;

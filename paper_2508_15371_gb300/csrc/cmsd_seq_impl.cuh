@@ -22,8 +22,8 @@
 // piece) is, above griddepcontrol.wait.
 //
 // us a call, the streaming kernel and its draw against one launch, sampled
-// bf16: B=4 K=4 V=32000 16.1, 7.7; B=32 K=8 V=128256 35.7, 30.8; B=64 54.2,
-// 53.4, where 256 CTAs stream 262.7 MB at 0.87 of the copy rate, bound by
+// bf16: B=4 K=4 V=32000 16.1, 7.7; B=32 K=8 V=128256 35.7, 30.2; B=64 54.2,
+// 52.8, where 256 CTAs stream 262.7 MB at 0.87 of the copy rate, bound by
 // issue slots, and 8 us of rows and draw follow.
 #pragma once
 #include "cmsd_stream_impl.cuh"
@@ -32,8 +32,16 @@ namespace cmsd {
 
 constexpr int kSeqMaxCtas = kDrawMaxCtas;   // CTAs per cluster (16: a non-portable size)
 constexpr int kSeqMaxK = kPackedMaxK;    // positions per window
+// Vectors per lane, tensor and stage: both tensors under the PAPER rule, under
+// the sampled rule (four spill there, and cost more registers than the deeper
+// stage gains: B=8 K=8 V=128256 14.9 against 13.4 us, B=16 24.4, 22.6, B=64
+// 53.2, 52.8; B=1 12.1, 12.5), and one tensor alone (six or four: verify
+// B=128 K=8 V=128256 41.5, 43.9 against 40.9).
 #ifndef CMSD_SEQ_UNROLL
 #define CMSD_SEQ_UNROLL 4
+#endif
+#ifndef CMSD_SEQ_UNROLL_S
+#define CMSD_SEQ_UNROLL_S 3
 #endif
 #ifndef CMSD_SEQ_UNROLL1
 #define CMSD_SEQ_UNROLL1 8
@@ -255,7 +263,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     const T* dp = pc.dp;
     const T* tp = pc.tp;
     const Seg sg = pc.sg;
-    Pipe<T, HAS_D && HAS_T ? CMSD_SEQ_UNROLL : CMSD_SEQ_UNROLL1> pp;
+    Pipe<T, HAS_D && HAS_T ? (SAMPLED ? CMSD_SEQ_UNROLL_S : CMSD_SEQ_UNROLL) : CMSD_SEQ_UNROLL1> pp;
     pipe_start<T, MODE>(pp, dp, tp, sg.va, sg.vb, lane);
     SegState ss;
     ss.c = ss.zd = 0.f;

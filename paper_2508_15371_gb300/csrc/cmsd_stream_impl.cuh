@@ -58,7 +58,7 @@
 // Bound, on a GB300: DRAM while it streams (B=64 K=8 V=128256 bf16, sampled: the
 // slices of 262.7 MB end 37 us into the launch, median, 7.1 TB/s; the last at
 // 43), then the chain of the last rows, and the draw (54.2 us a call; such a
-// call now takes one launch, 53.4).
+// call now takes one launch, 52.8).
 //
 // -inf logits (masked vocabulary) are clamped to -2^100 before the drafter
 // arithmetic so that e^(z-m) * (z-m) is 0, not NaN.
