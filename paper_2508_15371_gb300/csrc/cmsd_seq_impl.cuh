@@ -208,6 +208,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
   constexpr int VEC = Elem<T>::kVec;
   extern __shared__ __align__(128) unsigned char seq_smem[];
   __shared__ SeqRow s_row[kSeqMaxK];
+  // A tail's logits while its piece's vectors are reduced: in shared memory
+  // where the loop has no two registers to spare (PAPER, in registers: spills,
+  // and B=32 K=8 V=128256 26.4 us against 25.5), else in registers (the
+  // drafter alone, in shared memory: spills, and B=64 K=1 V=50257 5.3 us
+  // against 4.8).
+  constexpr bool kStash = MODE == kModeFused || (MODE == kModeVerify && !SAMPLED);
+  __shared__ float2 s_tail[kStash ? NW : 1][VEC - 1];
   cg::cluster_group cl = cg::this_cluster();
   const int nc = sp.nc;
   const int cr = (int)cl.block_rank(), b = (int)(blockIdx.x / (unsigned)nc);
@@ -274,16 +281,30 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     }
     dlane_init(ss.d);
     tlane_init(ss.t, ss.c, beta);
-    // the unaligned head (in the first lanes) and tail (in the last); after the
-    // pipeline instead, the sampled rule's stages compiled to slower code (36
-    // against 33.5 us at B=32 K=8 V=128256 with the bonus row)
+    // The unaligned head (in the first lanes) and tail (in the last): requested
+    // together, the head folded before the vectors and the tail after them, in
+    // the order of a lane's indices (a vector takes the maximum's place on a
+    // strict increase alone).
     const int hd = sg.va - sg.v0, tl = sg.v1 - sg.vb;
+    const int ve = lane < hd ? sg.v0 + lane : sg.v1 - 32 + lane;
+    float ze_d = 0.f, ze_t = 0.f;
     if (lane < hd || lane >= 32 - tl) {
-      const int v = lane < hd ? sg.v0 + lane : sg.v1 - 32 + lane;
-      if (HAS_D) d_scalar(ss.d, Elem<T>::load(dp + v), v);
-      if (HAS_T) t_scalar<SAMPLED>(ss.t, Elem<T>::load(tp + v), v, ss.c, beta);
+      if (HAS_D) ze_d = Elem<T>::load(dp + ve);
+      if (HAS_T) ze_t = Elem<T>::load(tp + ve);
+    }
+    if (lane < hd) {
+      if (HAS_D) d_scalar(ss.d, ze_d, ve);
+      if (HAS_T) t_scalar<SAMPLED>(ss.t, ze_t, ve, ss.c, beta);
+    } else if (kStash && lane >= 32 - tl) {
+      s_tail[warp][lane - 33 + VEC] = make_float2(ze_d, ze_t);
     }
     pipe_run<T, MODE, SAMPLED>(pp, ss, sg.va, beta, lane);
+    if (lane >= 32 - (sg.v1 - sg.vb)) {
+      const float2 z = kStash ? s_tail[warp][lane - 33 + VEC] : make_float2(ze_d, ze_t);
+      const int v = sg.v1 - 32 + lane;
+      if (HAS_D) d_scalar(ss.d, z.x, v);
+      if (HAS_T) t_scalar<SAMPLED>(ss.t, z.y, v, ss.c, beta);
+    }
     DRed dr;
     TRed tr;
     seg_reduce<T, MODE, SAMPLED>(ss, sg, !SAMPLED || a.argmax != nullptr, dp, tp, dr, tr);

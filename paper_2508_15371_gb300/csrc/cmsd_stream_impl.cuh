@@ -178,12 +178,12 @@ __device__ __forceinline__ void t_reref(TLane& t, float mx) {
   t.negrL = dup2(-nrL);
 }
 
-// --- drafter: one element at a time (segment heads/tails, in any order with
-// the lane's vectors) ----------------------------------------------------------
+// --- drafter: one element at a time (a segment's head before the lane's
+// vectors, its tail after them) ----------------------------------------------
 __device__ __forceinline__ void d_scalar(DLane& d, float z, int v) {
   d.f2 = fmaxf(d.f2, fminf(d.f1, z));
   d.f1 = fmaxf(d.f1, z);
-  if (z > d.m || (z == d.m && v < d.pos)) d.pos = v;
+  if (z > d.m) d.pos = v;
   d.m = fmaxf(d.m, z);
   const float me = d_mexp(d);
   if (me > d.ref + kRefSlack) d_reref(d, me);
@@ -242,7 +242,7 @@ __device__ __forceinline__ void d_vexp(const DLane& d, float4 q, u64& ss, u64& t
 // --- target -----------------------------------------------------------------------
 template <bool SAMPLED>
 __device__ __forceinline__ void t_scalar(TLane& t, float z, int v, float c, int beta) {
-  if (!SAMPLED && (z > t.M || (z == t.M && v < t.pos))) t.pos = v;
+  if (!SAMPLED && z > t.M) t.pos = v;
   t.M = fmaxf(t.M, z);
   if (t.cnt < beta && z > c) ++t.cnt;
   if (SAMPLED) {

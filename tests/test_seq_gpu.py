@@ -147,3 +147,79 @@ def test_rows_beyond_every_share(cmsd, noise, bonus):
     g = gpu_fused(cmsd, torch, w, p, iteration=2)
     compare(w, g, oracle_fused(w, p, iteration=2))
     assert (g["n_accept"] == K).any() if bonus else (g["n_accept"] < K).any()
+
+
+def _tie_pairs(V, es, most, seed):
+    """(lower, upper) entries for rows 0, 1, ... of a tensor of V-entry rows: two
+    that one lane of a piece reads in both of its ways, singly and in a
+    16-byte vector.
+
+    A piece starts at a whole 128-byte line from its row's start and ends at
+    one, or at V; its unaligned tail goes to the lanes 31, 30, ..., its
+    unaligned head to the lanes 0, 1, ....  The lanes of the vectors depend on
+    the starting line modulo four, so four starts stand for all.  `most`
+    candidates for each of the rows' places off 16-byte boundaries, those at
+    the row's end always among them.
+    """
+    rng = np.random.default_rng(seed)
+    vec, line = 16 // es, 128 // es
+    classes = []
+    for mis in range(vec):
+        ends, rest = [], []
+        for end in list(range(line, V, line)) + [V]:
+            for back in range(1, (end + mis) % vec + 1):
+                lane = 32 - back
+                for f in range(4):
+                    va = f * line + (-(f * line + mis)) % vec        # the piece's first whole vector
+                    j = (end - (end + mis) % vec - vec - va) // vec  # and its last one, from there
+                    j -= (j - lane) % 32
+                    for t in (j, j - 32):
+                        if t >= 0:
+                            (ends if end == V else rest).append((va + t * vec + int(rng.integers(0, vec)), end - back))
+        for start in range(0, V - 33 * vec, line):
+            for lane in range(-(start + mis) % vec):
+                va = start + (-(start + mis)) % vec
+                rest.append((start + lane, va + lane * vec + int(rng.integers(0, vec))))
+        rest = [rest[k] for k in rng.permutation(len(rest))[:max(0, most - len(ends))]]
+        classes.append(ends + rest or [(V // 2, V - 1)])
+    n = vec * max(len(c) for c in classes)
+    return [classes[r * V % vec][r // vec % len(classes[r * V % vec])] for r in range(n)]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V,most", [(129, 60), (257, 60), (4099, 800), (32001, 400)])
+def test_ties_off_vector_boundaries_take_the_lowest_index(cmsd, V, most, dtype):
+    """A maximum at two entries of a row, one read by itself and one in a
+    vector of the same lane: the argmax, and the PAPER rule's correction, is
+    the lower of the two.  Batches of several sizes, so that rows are cut into
+    pieces of several lengths."""
+    es = 4 if dtype == "f32" else 2
+    pairs = _tie_pairs(V, es, most, seed=V + es)
+    n = len(pairs)
+    # rows 0 .. n - 1 of the tensor; a batch is a run of rows that starts on a
+    # 16-byte boundary (every 8th row), so a row keeps its place off them
+    g = torch.Generator(device="cuda").manual_seed(V)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    z = (4.0 * torch.rand((n, V), generator=g, device="cuda") - 4.0).to(dt)
+    rows = torch.arange(n, device="cuda")
+    low, high = torch.tensor(pairs, device="cuda").T
+    assert (low >= 0).all() and (low < high).all() and (high < V).all()
+    z[rows, low] = 9.0
+    z[rows, high] = 9.0
+    want = low.to(torch.int32)
+    p = cmsd.params(1, "paper", beta_rank=0, tau_base=0.0, gamma=0.0)      # accepts the maximum alone
+    sizes, at = [8, 32, 64, 152, 1], 0
+    while at < n:
+        B = min(sizes[0], n - at)
+        sizes = sizes[1:] + sizes[:1]
+        x = z[at:at + B].view(B, 1, V)
+        tok = ((want[at:at + B] + 1) % V).view(B, 1)
+        tok = torch.where(x[:, 0].gather(1, tok.long()) == 9.0, (tok + 1) % V, tok)
+        a = cmsd.confidence(x)
+        f = cmsd.confidence_verify(x, x, tok, p=p)
+        v = cmsd.verify(x, x, tok, a["conf"], p=p)
+        for name, got in (("confidence", a["argmax"]), ("fused", f["argmax"]), ("fused token", f["out_tokens"]),
+                          ("verify token", v["out_tokens"])):
+            bad = (got[:, 0] != want[at:at + B]).nonzero()[:, 0]
+            assert len(bad) == 0, (name, B, [(pairs[at + int(k)], int(got[int(k), 0])) for k in bad[:4]])
+        at += (B + 7) // 8 * 8
