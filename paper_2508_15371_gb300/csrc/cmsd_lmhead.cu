@@ -26,13 +26,13 @@
 // tile.
 //
 // Bounds, on a GB300: up to 128 hidden rows DRAM (R=64 d=2048 V=128256: 525.6 MB
-// in 89 us, 5.9 TB/s); at 256 rows the MMAs, whose operands take the shared
-// memory's bandwidth (109 us, 1.23 PFLOP/s; 131 us when the epilogue transposed
-// every tile); small calls the launch, the fill of the ring and the merge
-// kernel (R=16 d=1024 V=32000: 19.2 us for 65.6 MB).
+// in 90.4 us, 5.8 TB/s); at 256 rows the MMAs, whose operands take the shared
+// memory's bandwidth (108 us, 1.25 PFLOP/s; 131 us when the epilogue transposed
+// every tile); small calls the launch, the fill of the ring, the hidden rows,
+// which every CTA reads from the same lines of L2 (R=1 d=1024 V=32000 17.3 us,
+// R=16 20.2), and the merge kernel.
 #include <cuda.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "cmsd_stream_impl.cuh"
@@ -49,17 +49,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
           "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// the same box into every CTA of the cluster named in `mask`: at the same
-// shared offset, completing the barrier at the same offset
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar,
-                                               uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
-      "[%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
       : "memory");
 }
 
@@ -198,13 +187,6 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// the same, arriving on the barrier at that offset of every CTA in `mask`
-__device__ __forceinline__ void tc_commit_mc(uint32_t bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"(mask)
-      : "memory");
-}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
@@ -229,14 +211,12 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
 // named barrier among the epilogue threads (barrier 0 is __syncthreads)
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-// CS CTAs of a cluster share the hidden rows' loads: each reads 1/CS of a
-// stage's box from L2 and multicasts it to all of them, so they walk the same
-// number of tiles in step.  hrows: rows loaded of a block (lanes beyond them
-// hold whatever was there: a lane's result depends on its own row alone).
+// hrows: rows loaded of a block (lanes beyond them hold whatever was there: a
+// lane's result depends on its own row alone).
 // tmap_w0, tmap_w1: the weight in boxes of the rows of a run's last tile (runs
 // of q and q + 1 groups of eight entries), so that no row is read twice (a
 // whole box there made the kernel read 1.06 x the weight at V=128256).
-template <int H, int CS>
+template <int H>
 __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadArgs h, const int hrows, const int tail0,
                                                                  const int tail1,
                                                                  const __grid_constant__ CUtensorMap tmap_h,
@@ -244,25 +224,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
                                                                  const __grid_constant__ CUtensorMap tmap_w0,
                                                                  const __grid_constant__ CUtensorMap tmap_w1) {
   using S = TcShape<H>;
-  constexpr uint16_t kAll = (uint16_t)((1 << CS) - 1);
   constexpr int kStages = S::kStages;
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rb = blockIdx.x / h.nct, cta = blockIdx.x - rb * h.nct;
   int v0, v1;
   cta_run(h.V, h.nct, cta, v0, v1);
-  const int own = v1 > v0 ? (v1 - v0 + kTcN - 1) / kTcN : 0;   // tiles of this CTA's run
-  const int cr = CS > 1 ? cta % CS : 0;            // rank in the cluster (nct is a multiple of CS)
-  int ntiles = own;                                // the cluster's: the longest run's
-  if (CS > 1) {
-#pragma unroll
-    for (int c = 0; c < CS; ++c) {
-      int a0, a1;
-      cta_run(h.V, h.nct, cta - cr + c, a0, a1);
-      const int n = a1 > a0 ? (a1 - a0 + kTcN - 1) / kTcN : 0;
-      ntiles = n > ntiles ? n : ntiles;
-    }
-  }
+  const int ntiles = v1 > v0 ? (v1 - v0 + kTcN - 1) / kTcN : 0;
   // the last tile's rows: runs of q + 1 groups come first
   const int n8 = (h.V + 7) / 8;
   const bool longer = cta < n8 - (n8 / h.nct) * h.nct;
@@ -284,7 +252,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   if (tid == 0) {
     for (int k = 0; k < kStages; ++k) {
       mbar_init(full + 8 * k, 1);
-      mbar_init(empty + 8 * k, CS);                // every CTA's MMAs have read what it multicast
+      mbar_init(empty + 8 * k, 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull + 8 * b, 1);
@@ -303,7 +271,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   // everything above overlaps the end of what precedes this grid on the stream
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (CS > 1) cluster_sync();                      // the peers' barriers exist before the first multicast
   tc_fence_after();
   const uint32_t tbase = *s_taddr;
   bool ok = true;
@@ -315,19 +282,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
         const int slot = g % kStages;
         if (g >= kStages && ok) ok = mbar_wait(empty + 8 * slot, (uint32_t)((g / kStages - 1) & 1));
         const int t = g / nkc, kc = g - t * nkc;
-        const uint32_t wbytes = t < own - 1 ? kTcWStage : (t == own - 1 ? tail * 128 : 0);
-        mbar_arrive_tx(full + 8 * slot, wbytes + (H == 64 ? 2 : 1) * hrows * 128);
-        if (t < own)
-          tma_load_2d(sW + slot * kTcWStage, t < own - 1 ? &tmap_w : map_last, kc * 64, v0 + t * kTcN, full + 8 * slot);
-        // the hidden rows (64 of them: twice), this CTA's part of the box
-        const uint32_t hdst = sH + slot * S::kHStage + cr * (hrows / CS) * 128;
+        const bool last = t == ntiles - 1;
+        mbar_arrive_tx(full + 8 * slot, (last ? tail * 128 : kTcWStage) + (H == 64 ? 2 : 1) * hrows * 128);
+        tma_load_2d(sW + slot * kTcWStage, last ? map_last : &tmap_w, kc * 64, v0 + t * kTcN, full + 8 * slot);
+        const uint32_t hdst = sH + slot * S::kHStage;
 #pragma unroll
-        for (int c = 0; c < (H == 64 ? 2 : 1); ++c) {
-          if (CS == 1)
-            tma_load_2d(hdst + c * 64 * 128, &tmap_h, kc * 64, row0, full + 8 * slot);
-          else
-            tma_load_2d_mc(hdst + c * 64 * 128, &tmap_h, kc * 64, row0 + cr * (hrows / CS), full + 8 * slot, kAll);
-        }
+        for (int c = 0; c < (H == 64 ? 2 : 1); ++c)       // the hidden rows (64 of them: twice)
+          tma_load_2d(hdst + c * 64 * 128, &tmap_h, kc * 64, row0, full + 8 * slot);
       }
     }
   } else if (warp == 1) {
@@ -351,8 +312,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
               tc_mma(d + c * kTcN, hd + (uint64_t)(2 * ks), wd + (uint64_t)(2 * ks), kTcIdesc, (kc | ks) != 0);
           }
           // the stage may be refilled once these MMAs are done
-          if (CS == 1) tc_commit(empty + 8 * slot);
-          else tc_commit_mc(empty + 8 * slot, kAll);
+          tc_commit(empty + 8 * slot);
         }
         tc_commit(tfull + 8 * b);                  // the accumulator is complete
       }
@@ -435,15 +395,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) lmhead_tc_kernel(const LmHeadAr
   if (warp == 0 && lane == 0) {                    // no TMA box still in flight into this CTA
     for (int g = (G > kStages ? G - kStages : 0); g < G; ++g)
       if (!mbar_wait(full + 8 * (g % kStages), (uint32_t)((g / kStages) & 1))) atomicOr(h.err, 4u);
-    if (CS > 1) {                                  // nor a peer's commit on its way to these barriers
-      for (int g = (G > kStages ? G - kStages : 0); g < G; ++g)
-        if (!mbar_wait(empty + 8 * (g % kStages), (uint32_t)((g / kStages) & 1))) atomicOr(h.err, 4u);
-    }
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (CS > 1) cluster_sync();                      // nor a peer still waiting for what this CTA multicasts
   tc_fence_after();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(S::kTmem) : "memory");
@@ -492,7 +447,7 @@ int lmhead_ctas_per_block(int sms, int R, int V) {
   int nct = sms / (nrb > 0 ? nrb : 1);
   const int n8 = (V + 7) / 8;
   if (nct > n8) nct = n8;
-  return nct < 4 ? 4 : nct;                        // (at least one cluster)
+  return nct < 1 ? 1 : nct;
 }
 
 namespace {
@@ -529,96 +484,49 @@ bool encode_rows(CUtensorMap* m, const void* base, int d, int rows, int box_rows
 }
 }  // namespace
 
-template <int H, int CS>
-cudaError_t tc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], unsigned grid) {
+template <int H>
+cudaError_t launch_tc(const LmHeadArgs& h, cudaStream_t s) {
   static unsigned long long done = 0ull;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
   if (!(__atomic_load_n(&done, __ATOMIC_ACQUIRE) & bit)) {
-    e = cudaFuncSetAttribute(lmhead_tc_kernel<H, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)TcShape<H>::kSmem);
+    e = cudaFuncSetAttribute(lmhead_tc_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcShape<H>::kSmem);
     if (e != cudaSuccess) return e;
     __atomic_fetch_or(&done, bit, __ATOMIC_ACQ_REL);
   }
-  cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kTcThreads);
-  cfg.dynamicSmemBytes = TcShape<H>::kSmem;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaSuccess;
-}
-
-// CTAs in clusters of CS that can be resident on the current device (cached
-// for the first 64; 0: none).
-template <int H, int CS>
-int tc_resident() {
-  static std::atomic<int> known[64];               // 0: not asked yet, else the answer + 1
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  int v = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
-  if (v == 0) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[2];
-    int n = 0;
-    if (tc_config<H, CS>(cfg, attr, CS) != cudaSuccess || (cfg.numAttrs = 1) == 0 ||   // (the cluster size)
-        cudaOccupancyMaxActiveClusters(&n, lmhead_tc_kernel<H, CS>, &cfg) != cudaSuccess) {
-      (void)cudaGetLastError();                    // a refused query leaves no error behind for the caller
-      n = 0;
-    }
-    v = 1 + n * CS;
-    if (dev < 64) known[dev].store(v, std::memory_order_relaxed);
-  }
-  return v - 1;
-}
-
-// h.nct: on entry the most CTAs per block, on return what was launched.
-template <int H, int CS>
-cudaError_t launch_tc(LmHeadArgs& h, cudaStream_t s) {
   const int nrb = (h.R + H - 1) / H;
-  if (CS > 1) {
-    const int res = tc_resident<H, CS>() / nrb;
-    int n = h.nct < res ? h.nct : res;
-    n -= n % CS;
-    h.nct = n < CS ? CS : n;                       // (a run may be empty)
-  }
   const int n8 = (h.V + 7) / 8, q = n8 / h.nct;
   const int tail0 = q > 0 ? (8 * q - 1) % kTcN + 1 : 8, tail1 = (8 * q + 7) % kTcN + 1;
-  const int step = 8 * CS;                         // a CTA's part of the hidden box: whole groups of eight rows
-  int hrows = nrb == 1 ? (h.R + step - 1) / step * step : H;
+  int hrows = nrb == 1 ? (h.R + 7) / 8 * 8 : H;    // whole groups of eight rows
   if (hrows > H) hrows = H;
   CUtensorMap tmap_h, tmap_w, tmap_w0, tmap_w1;
-  if (!encode_rows(&tmap_h, h.hidden, h.d, h.R, hrows / CS) || !encode_rows(&tmap_w, h.weight, h.d, h.V, kTcN) ||
+  if (!encode_rows(&tmap_h, h.hidden, h.d, h.R, hrows) || !encode_rows(&tmap_w, h.weight, h.d, h.V, kTcN) ||
       !encode_rows(&tmap_w0, h.weight, h.d, h.V, tail0) || !encode_rows(&tmap_w1, h.weight, h.d, h.V, tail1))
     return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[2];
-  const cudaError_t e = tc_config<H, CS>(cfg, attr, (unsigned)(nrb * h.nct));
-  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nrb * h.nct));
+  cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = TcShape<H>::kSmem;
   cfg.stream = s;
-  return cudaLaunchKernelEx(&cfg, lmhead_tc_kernel<H, CS>, h, hrows, tail0, tail1, tmap_h, tmap_w, tmap_w0, tmap_w1);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, lmhead_tc_kernel<H>, h, hrows, tail0, tail1, tmap_h, tmap_w, tmap_w0, tmap_w1);
 }
 
-// Clusters of four share the hidden rows' loads up to 128 rows (R=16 d=1024
-// V=32000: 19.2 us a call against 21.0 alone; R=64 d=2048 V=128256: 89.1
-// against 92.0; R=128: 91.1 against 92.9; pairs were slower than either).  256
-// rows are bound by the MMAs' reads of shared memory (108.7 us alone, 109.3
-// with four).
-cudaError_t launch_lmhead(const LmHeadArgs& args, const StreamArgs& a, cudaStream_t s) {
-  LmHeadArgs h = args;
+// Sharing the hidden rows' loads among the CTAs of a cluster would need loads
+// that write several CTAs' shared memory.  They are unsafe in a program on
+// several GPUs, which loads this same library, and are not used; they gained
+// 1 to 18 per cent (us a call with clusters of four, and without: R=16 d=1024
+// V=32000 18.3, 20.2; R=64 d=2048 V=128256 88.0, 90.4; R=128 90.1, 91.1; R=8
+// d=512 V=8000 9.4 to 10.3, 11.3).
+cudaError_t launch_lmhead(const LmHeadArgs& h, const StreamArgs& a, cudaStream_t s) {
   if (h.nb != lmhead_block_rows(h.R)) return cudaErrorInvalidValue;
-  cudaError_t e;
-  if (h.nb == 64) e = tc_resident<64, 4>() >= 4 ? launch_tc<64, 4>(h, s) : launch_tc<64, 1>(h, s);
-  else if (h.nb == 128) e = tc_resident<128, 4>() >= 4 ? launch_tc<128, 4>(h, s) : launch_tc<128, 1>(h, s);
-  else e = launch_tc<256, 1>(h, s);
+  const cudaError_t e = h.nb == 64 ? launch_tc<64>(h, s) : (h.nb == 128 ? launch_tc<128>(h, s) : launch_tc<256>(h, s));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((h.R + kMergeRowsPerCta - 1) / kMergeRowsPerCta));

@@ -35,6 +35,15 @@ def test_library_exports_every_declared_symbol(header, lib):
         assert hasattr(L, n), f"{lib} does not export {n}"
 
 
+def test_no_load_is_multicast_to_a_cluster():
+    # every rank of a multi-GPU program loads this one library, and a bulk load
+    # that writes several CTAs' shared memory is unsafe there
+    csrc = os.path.join(PKG, "csrc")
+    for f in sorted(os.listdir(csrc)):
+        code = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, f)).read())
+        assert "multicast::cluster" not in code, f
+
+
 @pytest.fixture(scope="module")
 def cmsd():
     _built("libcmsd.so")
