@@ -263,6 +263,9 @@ def lmhead_confidence(hidden, weight, p=None, logits=False, out=None, ws=None):
     V, d2 = weight.shape
     if d2 != d:
         raise CmsdError("hidden [R, d] and weight [V, d] must share d")
+    cur = torch.cuda.current_device()
+    if hidden.get_device() != cur or weight.get_device() != cur:
+        raise CmsdError("hidden and weight must be on the current device")
     p = p if p is not None else params(1)
     dev = hidden.device
     o = {n: _out(out, n, (R,), torch.float32, dev) for n in ("H", "margin", "conf", "lse")}

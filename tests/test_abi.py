@@ -156,3 +156,28 @@ def test_bonus_and_fixed_k_argument_checks(cmsd):
     rc = L.cmsd_confidence_verify(a, a, a, None, 2, 8, 4097, cmsd.BF16, ctypes.byref(odd), 0, 0,
                                   None, None, None, None, None, None, a, a, None, None, 0, None)
     assert rc == cmsd.EINVAL
+
+
+def test_lmhead_refuses_tensors_of_another_device(cmsd, monkeypatch):
+    import torch
+
+    class OnDevice:
+        """What lmhead_confidence asks of a tensor before it launches."""
+        is_cuda = True
+
+        def __init__(self, shape, index):
+            self.shape, self.device, self._index = shape, torch.device("cuda", index), index
+
+        def is_contiguous(self):
+            return True
+
+        def element_size(self):
+            return 2
+
+        def get_device(self):
+            return self._index
+
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    for dh, dw in ((1, 1), (0, 1), (1, 0)):
+        with pytest.raises(cmsd.CmsdError, match="current device"):
+            cmsd.lmhead_confidence(OnDevice((4, 64), dh), OnDevice((100, 64), dw))
