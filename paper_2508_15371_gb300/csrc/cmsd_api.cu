@@ -282,7 +282,12 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // V=128256 sampled, streamed and in one launch: B=16 26.1, 22.6 (clusters of
 // twelve); B=32 35.6, 30.2 (of eight); B=40 39.4, 38.0 (of three with 512
 // threads); B=64 54.2, 52.8 (of four).
-bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int* nc, int* threads) {
+//
+// resident(n, threads): clusters of kSeqSizes[n] such CTAs that the device
+// holds at once (a small partition may hold few or none of the large ones).
+template <typename Resident>
+bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, Resident resident, int* nc,
+                int* threads) {
   if (a.K > kPackedMaxK || (second && sampled && !seq_draw_fits(dtype, a.V))) return false;
   const double kb = (double)a.K * a.V * (dtype == CMSD_F32 ? 4 : 2) * (mode == kModeFused ? 2 : 1) * 1e-3;
   const double stream = a.B * kb * (a.k_row ? 0.5 : 1.0) / 6900;
@@ -298,8 +303,6 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
   const int per = dtype == CMSD_F32 ? 4 : 8;             // entries per 16-byte vector
   double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 39) : (sampled ? 23.5 : 27));
   if (mode == kModeVerify && a.V % per != 0) rate *= 0.8;   // rows off 16-byte boundaries
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
   double best = 0.985 * flat;              // (a near tie stays with the streaming kernel)
   *nc = 0;
   for (int th = 256; th <= 512; th *= 2) {
@@ -311,12 +314,13 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + (second ? (sampled && !race ? 4.5 : 3.5) : 0);
       const double full = kb / n / (rate * (th / 256));
       if (fixed + full / 1.3 >= best) continue;
-      const int res = seq_resident(dev, dtype, k, th);
+      const int res = resident(k, th);
       if (res < 1) continue;
       int fit = res;
       if (a.k_row) fit += res / 10;
       else if (th == 512 && (n & 1)) fit = res * 96 / 100;
       else if (th == 256 && n >= 3) fit = res * 93 / 100;
+      if (fit < 1) fit = 1;
       const int waves = (a.B - 1) / fit + 1;
       // an SM to itself, or neighbours that end early
       const bool early = a.k_row && mode == kModeFused && waves == 1;
@@ -392,8 +396,12 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   a.Kt = bonus ? a.K + 1 : a.K;
   a.Ko = bonus ? a.K + 1 : a.K;
   const bool second = mode != kModeConf && (sampled || bonus);
+  int dev = 0;
+  const cudaError_t e0 = cudaGetDevice(&dev);
+  if (e0 != cudaSuccess) return cuda_fail(e0);
   int nc = 0, threads = 0;
-  if (choose_seq(dtype, mode, sampled, second, a, &nc, &threads)) {
+  if (choose_seq(dtype, mode, sampled, second, a, [&](int n, int th) { return seq_resident(dev, dtype, n, th); }, &nc,
+                 &threads)) {
     prof_record(0, s);
     const cudaError_t e = dtype == CMSD_F32 ? launch_seq_f32(mode, sampled, second, a, nc, threads, s)
                                             : launch_seq_bf16(mode, sampled, second, a, nc, threads, s);
@@ -630,6 +638,25 @@ int cmsd_test_record_wait_timeout(const void* draft_logits, const void* target_l
   if (e != cudaSuccess) return cuda_fail(e);
   e = launch_draw(dtype, true, a, dp, s);
   return e == cudaSuccess ? CMSD_OK : cuda_fail(e);
+}
+
+int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bonus, int ragged, const int32_t* resident,
+                     int* cluster, int* threads) {
+  const int32_t some = 0;
+  const int rc = check_sizes(B, K, V, dtype, ragged ? &some : nullptr);
+  if (rc) return rc;
+  if (call < kModeConf || call > kModeFused || B < 1 || K < 1 || !resident || !cluster || !threads) return CMSD_EINVAL;
+  StreamArgs a = blank_args();
+  fill_sizes(a, B, K, V);
+  a.bonus = bonus != 0;
+  a.k_row = ragged ? &some : nullptr;
+  const bool sampled = call != kModeConf && rule == CMSD_RULE_SAMPLED;
+  int nc = 0, th = 0;
+  choose_seq(dtype, call, sampled, call != kModeConf && (sampled || bonus), a,
+             [&](int n, int t) { return (int)resident[(t == 512 ? 17 : 0) + kSeqSizes[n]]; }, &nc, &th);
+  *cluster = nc;
+  *threads = nc > 0 ? th : 0;
+  return CMSD_OK;
 }
 
 int cmsd_confidence(const void* draft_logits, int B, int K, int V, int dtype, const int32_t* k_row,

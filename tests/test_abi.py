@@ -181,3 +181,34 @@ def test_lmhead_refuses_tensors_of_another_device(cmsd, monkeypatch):
     for dh, dw in ((1, 1), (0, 1), (1, 0)):
         with pytest.raises(cmsd.CmsdError, match="current device"):
             cmsd.lmhead_confidence(OnDevice((4, 64), dh), OnDevice((100, 64), dw))
+
+
+CONF, VERIFY, FUSED = 0, 1, 2
+
+
+def _choose(cmsd, resident, call, B, K, V, dtype=1, rule=1, bonus=0, ragged=0):
+    """(CTAs per sequence, threads) of the one-launch kernel, (0, 0) for the
+    streaming kernel, on a device with these resident clusters [2, 17]."""
+    table = np.ascontiguousarray(resident, np.int32)
+    nc, th = ctypes.c_int32(-1), ctypes.c_int32(-1)
+    rc = cmsd.lib().cmsd_test_choose(call, B, K, V, dtype, rule, bonus, ragged, table.ctypes.data, ctypes.byref(nc),
+                                     ctypes.byref(th))
+    assert rc == cmsd.OK
+    return nc.value, th.value
+
+
+def test_choice_of_kernel_where_one_cluster_fits(cmsd):
+    # a small partition of a device: one cluster of each size at a time, or of
+    # the large sizes only one and of the small ones as many as there is room
+    one = np.ones((2, 17), np.int32)
+    room = np.stack([16 // np.maximum(1, np.arange(17)), 8 // np.maximum(1, np.arange(17))])
+    for resident in (one, room, np.minimum(room, 2)):
+        for call in (CONF, VERIFY, FUSED):
+            for rule in (0, 1):
+                for B, K, V in ((1, 4, 32000), (1, 16, 128256), (2, 8, 128256), (16, 8, 32001), (300, 2, 8000)):
+                    for dtype in (0, 1):
+                        for ragged in (0, 1):
+                            nc, th = _choose(cmsd, resident, call, B, K, V, dtype, rule, 0, ragged)
+                            assert (nc, th) == (0, 0) or resident[1 if th == 512 else 0][nc] >= 1
+    assert _choose(cmsd, np.zeros((2, 17)), FUSED, 1, 4, 32000) == (0, 0)
+    assert _choose(cmsd, one, FUSED, 1, 17, 32000) == (0, 0)
