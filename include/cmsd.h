@@ -149,12 +149,13 @@ int cmsd_test_record_wait_timeout(const void* draft_logits, const void* target_l
                                   int dtype, int32_t* out_tokens, void* ws, size_t ws_bytes, void* stream);
 
 /* Test support, no counterpart in the paper, needs no GPU: which kernel would
- * take a call of these sizes on a device that holds resident[(threads ==
- * 512) * 17 + n] clusters of n CTAs of 256 or 512 threads at once.  call: 0
+ * take a call of these sizes on a device of `sms` SMs that holds
+ * resident[(threads == 512) * 17 + n] clusters of n CTAs of 256 or 512 threads
+ * at once.  call: 0
  * cmsd_confidence, 1 cmsd_verify, 2 cmsd_confidence_verify; ragged: k_row is
  * given.  *cluster and *threads: the one-launch kernel's CTAs per sequence and
  * threads per CTA, or 0 for the streaming kernel. */
-int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bonus, int ragged,
+int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bonus, int ragged, int sms,
                      const int32_t* resident, int32_t* cluster, int32_t* threads);
 
 /*

@@ -61,7 +61,7 @@ _SIGS = {
     "cmsd_workspace_init": (_c_int, [_vp, _c_sz, _vp]),
     "cmsd_workspace_errors": (_c_int, [_vp, _c_sz, _vp, ctypes.POINTER(ctypes.c_uint32)]),
     "cmsd_test_record_wait_timeout": (_c_int, [_vp, _vp, _c_int, _c_int, _c_int, _c_int, _vp, _vp, _c_sz, _vp]),
-    "cmsd_test_choose": (_c_int, [_c_int] * 8 + [_vp, _vp, _vp]),
+    "cmsd_test_choose": (_c_int, [_c_int] * 9 + [_vp, _vp, _vp]),
     "cmsd_confidence": (_c_int, [_vp, _c_int, _c_int, _c_int, _c_int, _vp, _vp,
                                  _vp, _vp, _vp, _vp, _vp, _vp, _vp, _c_sz, _vp]),
     "cmsd_verify": (_c_int, [_vp, _vp, _vp, _vp, _c_int, _c_int, _c_int, _c_int, _vp,

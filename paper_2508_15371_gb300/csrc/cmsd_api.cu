@@ -234,7 +234,6 @@ void fill_sizes(StreamArgs& a, int B, int K, int V) {
 // CTAs per cluster that choose_seq weighs.
 constexpr int kSeqSizes[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 16};
 constexpr int kSeqNumSizes = 12;
-constexpr int kModelWarps = 152 * 16;      // the streaming kernel's warps on a GB300
 
 // Clusters of seq_kernel that can be resident on device dev, which is current
 // (cached; n: index into kSeqSizes).
@@ -283,17 +282,19 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // twelve); B=32 35.6, 30.2 (of eight); B=40 39.4, 38.0 (of three with 512
 // threads); B=64 54.2, 52.8 (of four).
 //
-// resident(n, threads): clusters of kSeqSizes[n] such CTAs that the device
-// holds at once (a small partition may hold few or none of the large ones).
+// sms: the device's; resident(n, threads): clusters of kSeqSizes[n] such CTAs
+// that it holds at once (a small partition may hold few or none of the large
+// ones).
 template <typename Resident>
-bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, Resident resident, int* nc,
+bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int sms, Resident resident, int* nc,
                 int* threads) {
   if (a.K > kPackedMaxK || (second && sampled && !seq_draw_fits(dtype, a.V))) return false;
   const double kb = (double)a.K * a.V * (dtype == CMSD_F32 ? 4 : 2) * (mode == kModeFused ? 2 : 1) * 1e-3;
   const double stream = a.B * kb * (a.k_row ? 0.5 : 1.0) / 6900;
   double flat = 8 + stream;
-  if (!a.k_row && (int64_t)a.B * a.K < kModelWarps) {             // (the rows' warps, whole rows apart from the rest)
-    const double used = (double)(kModelWarps / (a.B * a.K)) * (a.B * a.K) / kModelWarps;
+  const int warps = sms * kStreamWarps;                           // the streaming kernel's
+  if (!a.k_row && (int64_t)a.B * a.K < warps) {                   // (the rows' warps, whole rows apart from the rest)
+    const double used = (double)(warps / (a.B * a.K)) * (a.B * a.K) / warps;
     if (used >= 0.75 && used < 0.9) flat += stream * 0.5 * (0.9 - used);
   }
   if (second) {
@@ -324,7 +325,7 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       const int waves = (a.B - 1) / fit + 1;
       // an SM to itself, or neighbours that end early
       const bool early = a.k_row && mode == kModeFused && waves == 1;
-      const bool apart = (int64_t)a.B * n * (th / 256) <= kModelWarps / 16;
+      const bool apart = (int64_t)a.B * n * (th / 256) <= sms;
       const double part = full / (early ? 1.3 : (apart ? 1.1 : 1.0));
       const double t = fixed + (n == 1 ? 3.5 : 10.0) * (waves - 1) + (waves * part > stream ? waves * part : stream);
       if (t < best) {
@@ -396,12 +397,14 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   a.Kt = bonus ? a.K + 1 : a.K;
   a.Ko = bonus ? a.K + 1 : a.K;
   const bool second = mode != kModeConf && (sampled || bonus);
-  int dev = 0;
+  int dev = 0, sms = 0;
   const cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 != cudaSuccess) return cuda_fail(e0);
+  rc = device_sms(&sms);
+  if (rc) return rc;
   int nc = 0, threads = 0;
-  if (choose_seq(dtype, mode, sampled, second, a, [&](int n, int th) { return seq_resident(dev, dtype, n, th); }, &nc,
-                 &threads)) {
+  if (choose_seq(dtype, mode, sampled, second, a, sms, [&](int n, int th) { return seq_resident(dev, dtype, n, th); },
+                 &nc, &threads)) {
     prof_record(0, s);
     const cudaError_t e = dtype == CMSD_F32 ? launch_seq_f32(mode, sampled, second, a, nc, threads, s)
                                             : launch_seq_bf16(mode, sampled, second, a, nc, threads, s);
@@ -640,19 +643,19 @@ int cmsd_test_record_wait_timeout(const void* draft_logits, const void* target_l
   return e == cudaSuccess ? CMSD_OK : cuda_fail(e);
 }
 
-int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bonus, int ragged, const int32_t* resident,
-                     int* cluster, int* threads) {
+int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bonus, int ragged, int sms,
+                     const int32_t* resident, int32_t* cluster, int32_t* threads) {
   const int32_t some = 0;
   const int rc = check_sizes(B, K, V, dtype, ragged ? &some : nullptr);
   if (rc) return rc;
-  if (call < kModeConf || call > kModeFused || B < 1 || K < 1 || !resident || !cluster || !threads) return CMSD_EINVAL;
+  if (call < kModeConf || call > kModeFused || B < 1 || K < 1 || sms < 1 || !resident || !cluster || !threads) return CMSD_EINVAL;
   StreamArgs a = blank_args();
   fill_sizes(a, B, K, V);
   a.bonus = bonus != 0;
   a.k_row = ragged ? &some : nullptr;
   const bool sampled = call != kModeConf && rule == CMSD_RULE_SAMPLED;
   int nc = 0, th = 0;
-  choose_seq(dtype, call, sampled, call != kModeConf && (sampled || bonus), a,
+  choose_seq(dtype, call, sampled, call != kModeConf && (sampled || bonus), a, sms,
              [&](int n, int t) { return (int)resident[(t == 512 ? 17 : 0) + kSeqSizes[n]]; }, &nc, &th);
   *cluster = nc;
   *threads = nc > 0 ? th : 0;

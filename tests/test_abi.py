@@ -186,13 +186,13 @@ def test_lmhead_refuses_tensors_of_another_device(cmsd, monkeypatch):
 CONF, VERIFY, FUSED = 0, 1, 2
 
 
-def _choose(cmsd, resident, call, B, K, V, dtype=1, rule=1, bonus=0, ragged=0):
+def _choose(cmsd, resident, call, B, K, V, dtype=1, rule=1, bonus=0, ragged=0, sms=152):
     """(CTAs per sequence, threads) of the one-launch kernel, (0, 0) for the
-    streaming kernel, on a device with these resident clusters [2, 17]."""
+    streaming kernel, on a device of sms SMs with these resident clusters [2, 17]."""
     table = np.ascontiguousarray(resident, np.int32)
     nc, th = ctypes.c_int32(-1), ctypes.c_int32(-1)
-    rc = cmsd.lib().cmsd_test_choose(call, B, K, V, dtype, rule, bonus, ragged, table.ctypes.data, ctypes.byref(nc),
-                                     ctypes.byref(th))
+    rc = cmsd.lib().cmsd_test_choose(call, B, K, V, dtype, rule, bonus, ragged, sms, table.ctypes.data,
+                                     ctypes.byref(nc), ctypes.byref(th))
     assert rc == cmsd.OK
     return nc.value, th.value
 
@@ -212,3 +212,12 @@ def test_choice_of_kernel_where_one_cluster_fits(cmsd):
                             assert (nc, th) == (0, 0) or resident[1 if th == 512 else 0][nc] >= 1
     assert _choose(cmsd, np.zeros((2, 17)), FUSED, 1, 4, 32000) == (0, 0)
     assert _choose(cmsd, one, FUSED, 1, 17, 32000) == (0, 0)
+
+
+def test_choice_of_kernel_counts_the_devices_own_sms(cmsd):
+    # clusters as 16 SMs hold them: 25 CTAs of 256 threads share these SMs, and
+    # the streaming kernel is faster; on 152 SMs each would have one to itself
+    n = np.maximum(1, np.arange(17))
+    resident = np.stack([32 // n, 16 // n])
+    assert _choose(cmsd, resident, VERIFY, 5, 2, 128256, rule=0, sms=152) == (5, 256)
+    assert _choose(cmsd, resident, VERIFY, 5, 2, 128256, rule=0, sms=16) == (0, 0)
