@@ -658,8 +658,7 @@ def run_ours(args):
     # between the two kernels serialises them, so this pass is not the one
     # `value` comes from): durations of the streaming and resample kernels
     k_ms, r_ms = kernel_times(cmsd, torch, calls, args.steps)
-    # (two events with no kernel between them lie about a microsecond apart)
-    launches_per_step = 2 if statistics.median(r_ms) > 0.004 else 1
+    launches_per_step = cmsd.launch_plan(cmsd.FUSED, B, K, V, cmsd.BF16, p)[0]
     n_last = out["n_accept"].cpu().numpy()
     rejected = int((n_last < K).sum()) if sampled else 0
     ms_total = max_over_ranks(ms_total, dist, dev)

@@ -309,6 +309,15 @@ int cmsd_philox_fill(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint3
 int cmsd_profile_start(int max_calls);
 int cmsd_profile_stop(float* stream_ms, float* resample_ms, int max_out, int* n_out);
 
+/* What a call of these sizes launches on the current device, without
+ * launching it: call 0 cmsd_confidence, 1 cmsd_verify, 2
+ * cmsd_confidence_verify; ragged: k_row is given.  *launches: kernels.
+ * *cluster and *threads: the one-launch kernel's CTAs per sequence and threads
+ * per CTA, or 0 where the streaming kernel takes the call.  Any of the three
+ * may be NULL. */
+int cmsd_launch_plan(int call, int B, int K, int V, int dtype, const cmsd_params* p, int ragged,
+                     int* launches, int* cluster, int* threads);
+
 /* Launch geometry of the streaming kernels on the current device:
  * resident warps used (persistent grid) and SM count. */
 int cmsd_launch_info(int dtype, int* warps_out, int* sms_out);

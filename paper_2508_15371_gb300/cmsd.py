@@ -79,6 +79,7 @@ _SIGS = {
     "cmsd_philox_fill": (_c_int, [_c_u64, _c_u32, _c_u32, _c_u32, _c_u32, _vp, _c_sz, _vp]),
     "cmsd_profile_start": (_c_int, [_c_int]),
     "cmsd_profile_stop": (_c_int, [_vp, _vp, _c_int, ctypes.POINTER(ctypes.c_int)]),
+    "cmsd_launch_plan": (_c_int, [_c_int] * 5 + [_vp, _c_int] + [ctypes.POINTER(ctypes.c_int)] * 3),
     "cmsd_launch_info": (_c_int, [_c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     "cmsd_strerror": (ctypes.c_char_p, [_c_int]),
     "cmsd_last_cuda_error": (_c_int, []),
@@ -382,6 +383,18 @@ def profile_stop(max_calls):
     n = ctypes.c_int(0)
     _check(lib().cmsd_profile_stop(a, b, int(max_calls), ctypes.byref(n)), "cmsd_profile_stop")
     return [float(a[j]) for j in range(n.value)], [float(b[j]) for j in range(n.value)]
+
+
+CONFIDENCE, VERIFY, FUSED = 0, 1, 2
+
+
+def launch_plan(call, B, K, V, dtype, p, ragged=False):
+    """What a call (CONFIDENCE, VERIFY or FUSED) of these sizes launches on the current device:
+    (kernels, CTAs per sequence, threads per CTA), the last two 0 where the streaming kernel takes it."""
+    n, c, t = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_int(0)
+    _check(lib().cmsd_launch_plan(call, B, K, V, int(dtype), ctypes.byref(p), int(bool(ragged)), ctypes.byref(n),
+                                  ctypes.byref(c), ctypes.byref(t)), "cmsd_launch_plan")
+    return n.value, c.value, t.value
 
 
 def launch_info(dtype=BF16):

@@ -385,6 +385,21 @@ cudaError_t launch_draw(int dtype, bool sampled, const StreamArgs& a, const Draw
                            : launch_draw_bf16(sampled, a, d.clusters, d.nc, s);
 }
 
+// The current device's choice for a call: *nc CTAs of *threads threads per
+// sequence, or *nc = 0 for the streaming kernel.
+int choose(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, int* nc, int* threads) {
+  int dev = 0, sms = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_fail(e);
+  const int rc = device_sms(&sms);
+  if (rc) return rc;
+  *nc = *threads = 0;
+  if (!choose_seq(dtype, mode, sampled, second, a, sms, [&](int n, int th) { return seq_resident(dev, dtype, n, th); },
+                  nc, threads))
+    *nc = *threads = 0;
+  return CMSD_OK;
+}
+
 int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws_bytes,
            cudaStream_t s) {
   int wmax = 0;
@@ -397,14 +412,10 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   a.Kt = bonus ? a.K + 1 : a.K;
   a.Ko = bonus ? a.K + 1 : a.K;
   const bool second = mode != kModeConf && (sampled || bonus);
-  int dev = 0, sms = 0;
-  const cudaError_t e0 = cudaGetDevice(&dev);
-  if (e0 != cudaSuccess) return cuda_fail(e0);
-  rc = device_sms(&sms);
-  if (rc) return rc;
   int nc = 0, threads = 0;
-  if (choose_seq(dtype, mode, sampled, second, a, sms, [&](int n, int th) { return seq_resident(dev, dtype, n, th); },
-                 &nc, &threads)) {
+  rc = choose(dtype, mode, sampled, second, a, &nc, &threads);
+  if (rc) return rc;
+  if (nc > 0) {
     prof_record(0, s);
     const cudaError_t e = dtype == CMSD_F32 ? launch_seq_f32(mode, sampled, second, a, nc, threads, s)
                                             : launch_seq_bf16(mode, sampled, second, a, nc, threads, s);
@@ -786,6 +797,36 @@ int cmsd_profile_stop(float* stream_ms, float* resample_ms, int max_out, int* n_
   }
   if (n_out) *n_out = n;
   g_prof.n = 0;
+  return CMSD_OK;
+}
+
+int cmsd_launch_plan(int call, int B, int K, int V, int dtype, const cmsd_params* p, int ragged, int* launches,
+                     int* cluster, int* threads) {
+  const int32_t some = 0;
+  int rc = check_sizes(B, K, V, dtype, ragged ? &some : nullptr);
+  if (rc) return rc;
+  if (call < kModeConf || call > kModeFused) return CMSD_EINVAL;
+  rc = check_params(p, call != kModeConf);
+  if (rc) return rc;
+  if (call != kModeConf) {
+    rc = check_bonus_layout(p, V, dtype);
+    if (rc) return rc;
+  }
+  int nl = 0, nc = 0, th = 0;
+  if (B > 0 && K > 0) {
+    StreamArgs a = blank_args();
+    fill_sizes(a, B, K, V);
+    fill_params(a, p);
+    a.k_row = ragged ? &some : nullptr;
+    const bool sampled = call != kModeConf && p->rule == CMSD_RULE_SAMPLED;
+    const bool second = call != kModeConf && (sampled || a.bonus);
+    rc = choose(dtype, call, sampled, second, a, &nc, &th);
+    if (rc) return rc;
+    nl = nc > 0 || !second ? 1 : 2;
+  }
+  if (launches) *launches = nl;
+  if (cluster) *cluster = nc;
+  if (threads) *threads = th;
   return CMSD_OK;
 }
 

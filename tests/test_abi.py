@@ -221,3 +221,15 @@ def test_choice_of_kernel_counts_the_devices_own_sms(cmsd):
     resident = np.stack([32 // n, 16 // n])
     assert _choose(cmsd, resident, VERIFY, 5, 2, 128256, rule=0, sms=152) == (5, 256)
     assert _choose(cmsd, resident, VERIFY, 5, 2, 128256, rule=0, sms=16) == (0, 0)
+
+
+def test_launch_plan_argument_errors_and_empty_calls(cmsd):
+    p = cmsd.params(8, "sampled")
+    for call in (CONF, VERIFY, FUSED):
+        assert cmsd.launch_plan(call, 0, 8, 32000, cmsd.BF16, p) == (0, 0, 0)
+    for bad in (dict(call=3), dict(call=-1), dict(V=1), dict(K=2000), dict(p=cmsd.params(8, k_min=0)),
+                dict(V=4097, p=cmsd.params(8, bonus=1))):
+        kw = dict(call=FUSED, B=0, K=8, V=32000, dtype=cmsd.BF16, p=p)
+        kw.update(bad)
+        with pytest.raises(cmsd.CmsdError):
+            cmsd.launch_plan(**kw)

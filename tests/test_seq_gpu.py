@@ -111,6 +111,26 @@ def test_one_launch_equals_streaming(cmsd, B, K, V, rule, dtype):
         _same(a, b, kr, bonus)
 
 
+def test_launch_plan_is_what_runs(cmsd):
+    """The plan against the library's own events: a second interval is longer
+    than the microsecond or two between events around nothing only where a
+    second kernel ran."""
+    p = cmsd.params(8, "sampled")
+    assert cmsd.launch_plan(cmsd.FUSED, 4, 8, 4096, cmsd.BF16, p)[0] == 1
+    for K, rule, launches in ((8, "sampled", 1), (17, "sampled", 2), (17, "paper", 1)):
+        p = cmsd.params(K, rule)
+        n, nc, th = cmsd.launch_plan(cmsd.FUSED, 4, K, 128256, cmsd.BF16, p)
+        assert (n, nc > 0, th > 0) == (launches, K <= 16, K <= 16)
+        d, t, tok = _inputs(4, K, 128256, "bf16", False, False, seed=K)
+        cmsd.confidence_verify(d, t, tok, p=p)
+        torch.cuda.synchronize()
+        cmsd.profile_start(20)
+        for i in range(20):
+            cmsd.confidence_verify(d, t, tok, p=p, iteration=i)
+        _, second = cmsd.profile_stop(20)
+        assert (np.median(second) > 0.0035) == (launches == 2), (K, rule, np.median(second))
+
+
 def test_device_errors_are_reported(cmsd):
     """Out-of-range tokens and windows are clamped and set their bits."""
     d, t, tok = _inputs(3, 4, 4096, "bf16", False, False, 1)
