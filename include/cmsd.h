@@ -251,6 +251,20 @@ int cmsd_confidence_verify(const void* draft_logits, const void* target_logits,
                            int32_t* k_next, int32_t* n_accept, int32_t* out_tokens,
                            uint8_t* accept, void* ws, size_t ws_bytes, void* stream);
 
+/* Test support, no counterpart in the paper: cmsd_confidence_verify by the
+ * one-launch kernel with `cluster` CTAs of `threads` (256 or 512) threads per
+ * sequence, whatever its cost would be.  Returns CMSD_EDTYPE, launching
+ * nothing, where that kernel does not take the call (K > 16, a row whose draw
+ * does not fit, a cluster size that is not one of the rule's or that the
+ * current device does not hold). */
+int cmsd_test_confidence_verify_cluster(const void* draft_logits, const void* target_logits,
+                                        const int32_t* draft_tokens, const int32_t* k_row,
+                                        int B, int K, int V, int dtype, const cmsd_params* p,
+                                        uint64_t seed, uint32_t iteration, float* H, float* margin,
+                                        int32_t* argmax, float* conf, float* lse, int32_t* k_next,
+                                        int32_t* n_accept, int32_t* out_tokens, uint8_t* accept,
+                                        void* ws, size_t ws_bytes, void* stream, int cluster, int threads);
+
 /*
  * cmsd_confidence_verify without a workspace argument: the scratch is a fixed
  * array of CMSD_STATIC_SCRATCH_BYTES in the library's device image, one per

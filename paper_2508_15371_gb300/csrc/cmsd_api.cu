@@ -400,8 +400,10 @@ int choose(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, 
   return CMSD_OK;
 }
 
+// (nc > 0: the one-launch kernel with that many CTAs of `threads` threads per
+// sequence, whatever the rule says)
 int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws_bytes,
-           cudaStream_t s) {
+           cudaStream_t s, int nc = 0, int threads = 0) {
   int wmax = 0;
   int rc = wmax_warps(&wmax);
   if (rc) return rc;
@@ -412,9 +414,10 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   a.Kt = bonus ? a.K + 1 : a.K;
   a.Ko = bonus ? a.K + 1 : a.K;
   const bool second = mode != kModeConf && (sampled || bonus);
-  int nc = 0, threads = 0;
-  rc = choose(dtype, mode, sampled, second, a, &nc, &threads);
-  if (rc) return rc;
+  if (nc == 0) {
+    rc = choose(dtype, mode, sampled, second, a, &nc, &threads);
+    if (rc) return rc;
+  }
   if (nc > 0) {
     prof_record(0, s);
     const cudaError_t e = dtype == CMSD_F32 ? launch_seq_f32(mode, sampled, second, a, nc, threads, s)
@@ -671,6 +674,39 @@ int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bon
   *cluster = nc;
   *threads = nc > 0 ? th : 0;
   return CMSD_OK;
+}
+
+int cmsd_test_confidence_verify_cluster(const void* draft_logits, const void* target_logits,
+                                        const int32_t* draft_tokens, const int32_t* k_row, int B, int K, int V,
+                                        int dtype, const cmsd_params* p, uint64_t seed, uint32_t iteration, float* H,
+                                        float* margin, int32_t* argmax, float* conf, float* lse, int32_t* k_next,
+                                        int32_t* n_accept, int32_t* out_tokens, uint8_t* accept, void* ws,
+                                        size_t ws_bytes, void* stream, int cluster, int threads) {
+  const int rc = validate_fused(draft_logits, target_logits, draft_tokens, k_row, B, K, V, dtype, p,
+                                n_accept, out_tokens);
+  if (rc) return rc;
+  if (B == 0 || K == 0) return CMSD_OK;
+  const bool sampled = p->rule == CMSD_RULE_SAMPLED;
+  int size = -1, dev = 0;
+  for (int n = 0; n < kSeqNumSizes; ++n)
+    if (kSeqSizes[n] == cluster) size = n;
+  if (size < 0 || (threads != 256 && threads != 512) || K > kPackedMaxK || (sampled && !seq_draw_fits(dtype, V)))
+    return CMSD_EDTYPE;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_fail(e);
+  if (seq_resident(dev, dtype, size, threads) < 1) return CMSD_EDTYPE;
+  StreamArgs a = blank_args();
+  a.draft = draft_logits;
+  a.target = target_logits;
+  a.tokens = draft_tokens;
+  a.k_row = k_row;
+  fill_sizes(a, B, K, V);
+  fill_params(a, p);
+  a.seed = seed;
+  a.iteration = iteration;
+  a.H = H; a.margin = margin; a.argmax = argmax; a.conf = conf; a.lse = lse; a.k_next = k_next;
+  a.n_accept = n_accept; a.out_tokens = out_tokens; a.accept = accept;
+  return launch(dtype, kModeFused, sampled, a, ws, ws_bytes, (cudaStream_t)stream, cluster, threads);
 }
 
 int cmsd_confidence(const void* draft_logits, int B, int K, int V, int dtype, const int32_t* k_row,

@@ -69,9 +69,19 @@ def _same(narrow, wide, k_row, bonus):
             assert torch.equal(narrow["argmax"][b, :kb], wide["argmax"][b, :kb])
 
 
+def _in_one_launch(cmsd, d, t, tok, p, k_row, cluster, threads):
+    """The fused pass by the one-launch kernel, whatever the rule says."""
+    call = cmsd.FusedCall(d, t, tok, p, seed=9, iteration=3, k_row=k_row, signals=True)
+    rc = cmsd.lib().cmsd_test_confidence_verify_cluster(
+        *call._head, 9, 3, *call._tail, torch.cuda.current_stream().cuda_stream, cluster, threads)
+    assert rc == cmsd.OK
+    return call.out
+
+
 # Sizes: no whole vector, one group, lines and pieces that end inside a row,
-# the cluster sizes of the rule (1 to 16 CTAs of 256 or 512 threads), draws of
-# one and of two blocks of groups per lane set (B=32) and by bounds (B=64).
+# draws of one and of two blocks of groups per lane set (B=32) and by bounds
+# (B=64).  Which cluster sizes they take depends on the rule; every size is
+# asked for below.
 SHAPES = [(1, 1, 2), (3, 2, 33), (2, 16, 1000), (1, 4, 32000), (5, 7, 4099), (8, 8, 32128), (40, 3, 8193),
           (70, 5, 6400), (150, 2, 4096), (700, 1, 2048), (2, 8, 128256),
           (32, 2, 64128), (32, 2, 128256), (64, 2, 128255)]
@@ -97,6 +107,9 @@ def test_one_launch_equals_streaming(cmsd, B, K, V, rule, dtype):
             a = cmsd.confidence_verify(d, t, tok, k_row=kr, p=p, seed=9, iteration=3)
             b = cmsd.confidence_verify(d2, t2, tok2, k_row=full if kr is None else kr, p=pw, seed=9, iteration=3)
             _same(a, b, full if kr is None else kr, bonus)
+            code = cmsd.F32 if dtype == "f32" else cmsd.BF16
+            if cmsd.launch_plan(cmsd.FUSED, B, K, V, code, p, kr is not None)[1] == 0:
+                _same(_in_one_launch(cmsd, d, t, tok, p, kr, 1, 256), b, full if kr is None else kr, bonus)
         kr = k_row
         sig = cmsd.confidence(d, k_row=kr, p=p)
         sig2 = cmsd.confidence(d2, k_row=kr, p=pw)
@@ -109,6 +122,36 @@ def test_one_launch_equals_streaming(cmsd, B, K, V, rule, dtype):
         b = cmsd.verify(d2, t2, tok2, _widen(conf[:, :, None], W)[:, :, 0].contiguous(),
                         draft_lse=_widen(lse[:, :, None], W)[:, :, 0].contiguous(), k_row=kr, p=pw, seed=9, iteration=4)
         _same(a, b, kr, bonus)
+
+
+@pytest.mark.parametrize("threads", [256, 512])
+@pytest.mark.parametrize("cluster", [1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 16])
+def test_every_cluster_size_equals_streaming(cmsd, cluster, threads):
+    """The fused pass by the one-launch kernel with each cluster size, on
+    windows of odd and of aligned rows, against the streaming kernel."""
+    for B, K, V, dtype, rule, bonus in ((3, 5, 4099, "bf16", "sampled", False), (2, 16, 20008, "bf16", "paper", True),
+                                        (2, 3, 32001, "f32", "paper", False), (2, 7, 65536, "f32", "sampled", True),
+                                        (1, 4, 128256, "bf16", "sampled", True)):
+        d, t, tok = _inputs(B, K, V, dtype, bonus, masked=B == 2, seed=V + cluster)
+        p = cmsd.params(K, rule, bonus=bonus, tau_base=-0.5)
+        k_row = torch.tensor([K, max(0, K - 3), 0][:B], dtype=torch.int32, device="cuda")
+        full = torch.full((B,), K, dtype=torch.int32, device="cuda")
+        W = 17 - K
+        d2, t2, tok2 = _widen(d, W), _widen(t, W), _widen(tok[:, :, None], W)[:, :, 0].contiguous()
+        for kr in (None, k_row):
+            a = _in_one_launch(cmsd, d, t, tok, p, kr, cluster, threads)
+            wide = cmsd.confidence_verify(d2, t2, tok2, k_row=full if kr is None else kr, p=p, seed=9, iteration=3)
+            _same(a, wide, full if kr is None else kr, bonus)
+
+
+def test_cluster_sizes_that_are_refused(cmsd):
+    d, t, tok = _inputs(1, 17, 1024, "bf16", False, False, seed=1)
+    for K, cluster, threads in ((17, 1, 256), (4, 11, 256), (4, 0, 256), (4, 17, 512), (4, 2, 128)):
+        call = cmsd.FusedCall(d[:, :K].contiguous(), t[:, :K].contiguous(), tok[:, :K].contiguous(),
+                              cmsd.params(K, "sampled"))
+        rc = cmsd.lib().cmsd_test_confidence_verify_cluster(
+            *call._head, 0, 0, *call._tail, torch.cuda.current_stream().cuda_stream, cluster, threads)
+        assert rc == cmsd.EDTYPE, (K, cluster, threads)
 
 
 def test_launch_plan_is_what_runs(cmsd):
