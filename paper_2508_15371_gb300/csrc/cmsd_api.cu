@@ -260,27 +260,35 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 //   one launch         5, a draw 3.5 (4.5 by cluster_draw), and the time of a
 //     sequence's bytes through its CTAs (a CTA of 256 threads: 27 KB a
 //     microsecond under the PAPER rule, 23.5 under the sampled rule, 21 for
-//     the drafter alone, 30 for the target alone (39 under the PAPER rule when
+//     the drafter alone, 30 for the target alone (33 under the PAPER rule when
 //     windows are ragged, a fifth less off 16-byte boundaries); one of 512
-//     twice that; a tenth more with an SM to itself, three tenths more when
-//     both tensors' windows are ragged and neighbours end early), times the
-//     waves when not every cluster is resident (3.5 more each, 10 with
-//     clusters of several CTAs), and no less than the bytes at 6900 MB/s.
-// Ragged windows are unknown here: half full on average, and the longest
-// decides the one-launch pass, since a sequence keeps to its cluster; a tenth
-// more clusters than are resident find places as the shorter windows end
-// (B=48 K=12 V=32001 verify: 13.6 with 46 clusters of six resident, 15.7 with
-// clusters of five).
+//     twice that; a tenth more with an SM to itself), times the waves when not
+//     every cluster is resident (3.5 more each, 10 with clusters of several
+//     CTAs), and no less than the bytes at 6900 MB/s.
 //
-// Full windows need every cluster resident at once, and not all of the number
-// that the occupancy query names are: clusters of 256-thread CTAs left some
-// waiting above 93 in 100 of it (B=97 K=4 V=128256 by threes: 48.3 against
-// 35.4 streamed; B=90: 32.1), odd clusters of 512-thread CTAs, each with an SM
-// to itself, near the limit (B=28 K=8 by fives: 40.7 against 33.2; B=26:
-// 27.0), even ones not (SMs come in pairs).  Measured on both sides, K=8
-// V=128256 sampled, streamed and in one launch: B=16 26.1, 22.6 (clusters of
-// twelve); B=32 35.6, 30.2 (of eight); B=40 39.4, 38.0 (of three with 512
-// threads); B=64 54.2, 52.8 (of four).
+// Every cluster should be resident at once, and not all of the number that the
+// occupancy query names are: clusters of 256-thread CTAs left some waiting
+// above 93 in 100 of it (B=97 K=4 V=128256 by threes: 48.3 against 35.4
+// streamed; B=90: 32.1), odd clusters of 512-thread CTAs, each with an SM to
+// itself, near the limit (B=28 K=8 by fives: 40.7 against 33.2; B=26: 27.0),
+// even ones not (SMs come in pairs).  Measured on both sides, K=8 V=128256
+// sampled, streamed and in one launch: B=16 26.1, 22.6 (clusters of twelve);
+// B=32 35.6, 30.2 (of eight); B=40 39.4, 38.0 (of three with 512 threads);
+// B=64 54.2, 52.8 (of four).
+//
+// Ragged windows are unknown here: half full on average, and the longest
+// decides the one-launch pass, since a sequence keeps to its cluster.  They may
+// also all be full, so no more clusters count as resident than of full windows.
+// A tenth more than the query names gained where windows were short (B=48 K=12
+// V=32001 sampled verify, 46 clusters of six resident: 13.6, by fives 15.6,
+// streamed 17.9) and lost more where they were full (31.5, 26.3, 28.2; B=38
+// K=8 V=128256 sampled 49.8 by eights, 35.4 by sevens, 39.8 streamed).  Over 312
+// ragged shapes (B = 1..200, three calls, both rules, with and without the
+// bonus row), windows spread over 0..K, all half and all full, the choice takes
+// 0.86, 0.81 and 0.85 of the streaming kernel's time (geometric mean; with that
+// tenth 0.86, 0.85, 0.92).  It was nowhere slower than the streaming kernel but
+// for a few shapes with rows off 16-byte boundaries (1.09); with the tenth, and
+// with three tenths more for neighbours that end early, up to 1.37 times.
 //
 // sms: the device's; resident(n, threads): clusters of kSeqSizes[n] such CTAs
 // that it holds at once (a small partition may hold few or none of the large
@@ -302,7 +310,7 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
     if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 0.09 : 0.045);
   }
   const int per = dtype == CMSD_F32 ? 4 : 8;             // entries per 16-byte vector
-  double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 39) : (sampled ? 23.5 : 27));
+  double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 33) : (sampled ? 23.5 : 27));
   if (mode == kModeVerify && a.V % per != 0) rate *= 0.8;   // rows off 16-byte boundaries
   double best = 0.985 * flat;              // (a near tie stays with the streaming kernel)
   *nc = 0;
@@ -314,19 +322,16 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       const bool race = a.V <= (int64_t)8 * n * th * per;
       const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + (second ? (sampled && !race ? 4.5 : 3.5) : 0);
       const double full = kb / n / (rate * (th / 256));
-      if (fixed + full / 1.3 >= best) continue;
+      if (fixed + full / 1.1 >= best) continue;
       const int res = resident(k, th);
       if (res < 1) continue;
       int fit = res;
-      if (a.k_row) fit += res / 10;
-      else if (th == 512 && (n & 1)) fit = res * 96 / 100;
+      if (th == 512 && (n & 1)) fit = res * 96 / 100;
       else if (th == 256 && n >= 3) fit = res * 93 / 100;
       if (fit < 1) fit = 1;
       const int waves = (a.B - 1) / fit + 1;
-      // an SM to itself, or neighbours that end early
-      const bool early = a.k_row && mode == kModeFused && waves == 1;
-      const bool apart = (int64_t)a.B * n * (th / 256) <= sms;
-      const double part = full / (early ? 1.3 : (apart ? 1.1 : 1.0));
+      const bool apart = (int64_t)a.B * n * (th / 256) <= sms;   // an SM to itself
+      const double part = full / (apart ? 1.1 : 1.0);
       const double t = fixed + (n == 1 ? 3.5 : 10.0) * (waves - 1) + (waves * part > stream ? waves * part : stream);
       if (t < best) {
         best = t;

@@ -233,3 +233,20 @@ def test_launch_plan_argument_errors_and_empty_calls(cmsd):
         kw.update(bad)
         with pytest.raises(cmsd.CmsdError):
             cmsd.launch_plan(**kw)
+
+
+# Clusters of 1 .. 16 CTAs that a GB300 of 152 SMs holds at once, of 256 and of 512 threads.
+GB300 = np.array([[0, 304, 152, 97, 74, 58, 46, 38, 36, 30, 28, 0, 23, 0, 0, 0, 14],
+                  [0, 152, 76, 46, 36, 28, 23, 15, 15, 15, 13, 0, 8, 0, 0, 0, 7]])
+
+
+@pytest.mark.parametrize("call,K,V,rule,bonus", [(VERIFY, 12, 32001, 1, 0), (VERIFY, 12, 32001, 0, 0),
+                                                 (VERIFY, 8, 128256, 1, 0), (FUSED, 8, 128256, 1, 0),
+                                                 (FUSED, 8, 32128, 0, 0), (FUSED, 4, 32001, 1, 0),
+                                                 (FUSED, 8, 64128, 1, 1), (CONF, 8, 32001, 0, 0)])
+def test_ragged_windows_get_a_place_each(cmsd, call, K, V, rule, bonus):
+    # windows given by k_row may all be full: a cluster without a place would
+    # then run after the others, in twice the time
+    for B in range(1, 201):
+        nc, th = _choose(cmsd, GB300, call, B, K, V, 1, rule, bonus, ragged=1)
+        assert nc < 2 or B <= GB300[1 if th == 512 else 0][nc], (B, nc, th)
