@@ -255,9 +255,13 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // GB300 over K = 1..16, V = 32000..152064, B = 1..600 (bf16; f32 alike):
 //   streaming kernel   8 + bytes / 6900 MB/s, more when whole rows leave over
 //     a tenth of the warps without one (B=80 K=8 V=128256: 67.9), and with a
-//     second launch 7.5 more (12 with the bonus row) and 0.045 (0.09) per
-//     sequence beyond 64;
-//   one launch         5, a draw 3.5 (4.5 by cluster_draw), and the time of a
+//     second launch 7.5 more (12 with the bonus row), 0.045 (0.09) per
+//     sequence beyond 64, and 2.2 per 100000 entries where it draws from rows
+//     off 16-byte boundaries (B=30 K=8 ragged verify: V=128256 19.7, V=128255
+//     22.5);
+//   one launch         5, a draw 3.5 (4.5 by cluster_draw, which takes over at
+//     half the share off 16-byte boundaries: B=10 K=1 V=152063 verify 11.1 by
+//     16 CTAs of 256 threads, 9.4 raced by ten of 512), and the time of a
 //     sequence's bytes through its CTAs (a CTA of 256 threads: 27 KB a
 //     microsecond under the PAPER rule, 23.5 under the sampled rule, 21 for
 //     the drafter alone, 30 for the target alone (33 under the PAPER rule when
@@ -282,13 +286,13 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // A tenth more than the query names gained where windows were short (B=48 K=12
 // V=32001 sampled verify, 46 clusters of six resident: 13.6, by fives 15.6,
 // streamed 17.9) and lost more where they were full (31.5, 26.3, 28.2; B=38
-// K=8 V=128256 sampled 49.8 by eights, 35.4 by sevens, 39.8 streamed).  Over 312
+// K=8 V=128256 sampled 49.8 by eights, 35.4 by sevens, 39.8 streamed).  Over 442
 // ragged shapes (B = 1..200, three calls, both rules, with and without the
 // bonus row), windows spread over 0..K, all half and all full, the choice takes
-// 0.86, 0.81 and 0.85 of the streaming kernel's time (geometric mean; with that
-// tenth 0.86, 0.85, 0.92).  It was nowhere slower than the streaming kernel but
-// for a few shapes with rows off 16-byte boundaries (1.09); with the tenth, and
-// with three tenths more for neighbours that end early, up to 1.37 times.
+// 0.87, 0.81 and 0.85 of the streaming kernel's time (geometric mean; with that
+// tenth 0.86, 0.85, 0.92).  It was slower than the streaming kernel at
+// one of them (1.09, verify B=130 K=12 V=32001); with the tenth, and with three
+// tenths more for neighbours that end early, at one in eight, up to 1.37 times.
 //
 // sms: the device's; resident(n, threads): clusters of kSeqSizes[n] such CTAs
 // that it holds at once (a small partition may hold few or none of the large
@@ -305,13 +309,15 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
     const double used = (double)(warps / (a.B * a.K)) * (a.B * a.K) / warps;
     if (used >= 0.75 && used < 0.9) flat += stream * 0.5 * (0.9 - used);
   }
+  const int per = dtype == CMSD_F32 ? 4 : 8;             // entries per 16-byte vector
+  const bool odd = a.V % per != 0;                       // rows off 16-byte boundaries
   if (second) {
     flat += a.bonus ? 12 : 7.5;
     if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 0.09 : 0.045);
+    if (sampled && odd) flat += 2.2e-5 * a.V;
   }
-  const int per = dtype == CMSD_F32 ? 4 : 8;             // entries per 16-byte vector
   double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 33) : (sampled ? 23.5 : 27));
-  if (mode == kModeVerify && a.V % per != 0) rate *= 0.8;   // rows off 16-byte boundaries
+  if (mode == kModeVerify && odd) rate *= 0.8;
   double best = 0.985 * flat;              // (a near tie stays with the streaming kernel)
   *nc = 0;
   for (int th = 256; th <= 512; th *= 2) {
@@ -319,7 +325,8 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       const int n = kSeqSizes[k];
       // at least two 16-byte vectors per lane and piece, or more CTAs gain nothing
       if (n > 1 && kb * 1e3 < (double)n * (th / 32) * 1024 * (mode == kModeFused ? 2 : 1)) break;
-      const bool race = a.V <= (int64_t)8 * n * th * per;
+      // (cluster_race: two blocks of groups per lane set, one off 16-byte boundaries)
+      const bool race = a.V <= (int64_t)(odd ? 4 : 8) * n * th * per;
       const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + (second ? (sampled && !race ? 4.5 : 3.5) : 0);
       const double full = kb / n / (rate * (th / 256));
       if (fixed + full / 1.1 >= best) continue;

@@ -250,3 +250,11 @@ def test_ragged_windows_get_a_place_each(cmsd, call, K, V, rule, bonus):
     for B in range(1, 201):
         nc, th = _choose(cmsd, GB300, call, B, K, V, 1, rule, bonus, ragged=1)
         assert nc < 2 or B <= GB300[1 if th == 512 else 0][nc], (B, nc, th)
+
+
+def test_choice_of_kernel_off_vector_boundaries(cmsd):
+    # cluster_race takes half the share off 16-byte boundaries that it takes on
+    # them: 16 CTAs of 256 threads race a row of 152064 entries, not one of 152063
+    assert 152064 > 4 * 16 * 256 * 8
+    assert _choose(cmsd, GB300, VERIFY, 10, 1, 152064) == (16, 256)
+    assert _choose(cmsd, GB300, VERIFY, 10, 1, 152063) == (10, 512)
