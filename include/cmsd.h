@@ -251,6 +251,13 @@ int cmsd_confidence_verify(const void* draft_logits, const void* target_logits,
                            int32_t* k_next, int32_t* n_accept, int32_t* out_tokens,
                            uint8_t* accept, void* ws, size_t ws_bytes, void* stream);
 
+/* Test support, no counterpart in the paper, needs no GPU: which second kernel
+ * a streamed call of B sequences takes on a device that holds resident[0]
+ * clusters of the staged draw and resident[1], resident[2] clusters of four
+ * and of two CTAs of the draw from global memory at once.  *ctas: 0 the staged
+ * draw, 4 or 2 the other, -1 the race over every group. */
+int cmsd_test_draw(int B, int V, int dtype, int rule, int bonus, const int32_t* resident, int32_t* ctas);
+
 /* Test support, no counterpart in the paper: cmsd_confidence_verify by the
  * one-launch kernel with `cluster` CTAs of `threads` (256 or 512) threads per
  * sequence, whatever its cost would be.  Returns CMSD_EDTYPE, launching

@@ -69,6 +69,7 @@ _SIGS = {
     "cmsd_confidence_verify": (_c_int, [_vp, _vp, _vp, _vp, _c_int, _c_int, _c_int, _c_int, _vp,
                                         _c_u64, _c_u32, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                         _vp, _c_sz, _vp]),
+    "cmsd_test_draw": (_c_int, [_c_int] * 5 + [_vp, _vp]),
     "cmsd_test_confidence_verify_cluster": (_c_int, [_vp, _vp, _vp, _vp, _c_int, _c_int, _c_int, _c_int, _vp,
                                                      _c_u64, _c_u32, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                                      _vp, _c_sz, _vp, _c_int, _c_int]),

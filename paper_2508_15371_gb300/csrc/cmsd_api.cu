@@ -370,24 +370,58 @@ int draw_resident(int dtype, int V, int nc) {
 
 // Which kernel makes the second pass of a streamed call, or false where a
 // row's share does not fit (resample_kernel draws): the staged residual draw
-// while every sequence's cluster can be resident and there is no bonus row;
-// else draw_kernel with four CTAs per sequence up to 152 sequences (B=128 K=8
-// V=128256 with the bonus row: 94.9 us a call against 98.8 with two), two
-// beyond (B=256 K=16 V=152064: 380 us against 383).
+// (a call without the bonus row), or draw_kernel with four CTAs per sequence,
+// or with two.  Staging pays where few groups are left out by the bound (a
+// target close to its drafter: each group left is read again), and costs turns
+// beyond the resident clusters, fewer than draw_kernel's; both grow with a
+// row's bytes (`row`; half as much again off 16-byte boundaries, where a vector
+// takes two loads).  us a call at K=1, staged, four, two, for targets at drafter
+// + N(0,1) and, in brackets, + N(0,1)/2 with the drafter's argmax drafted:
+//   B=100 V=32000 bf16 17.5, 16.7, 17.2 (13.5, 12.7, 12.4);
+//   B=100 V=128256 bf16 25.0, 26.1, 29.1 (23.5, 25.2, 27.6);
+//   B=180 V=128256 bf16 33.6, 33.3, 35.4 (30.5, 32.2, 34.1);
+//   B=300 V=128256 bf16 49.2, 44.4, 43.7 (41.4, 42.6, 44.1);
+//   B=180 V=128255 bf16 38.0, 39.4, 46.4 (33.9, 36.7, 43.3);
+//   B=300 V=128255 bf16 61.6, 51.9, 56.6 (45.4, 48.7, 54.9);
+//   B=600 V=128255 bf16 109.8, 101.7, 86.5 (77.8, 74.0, 80.4);
+//   B=40 V=128255 f32 (36 staged clusters resident) 27.5, 35.3, 48.9.
+// Over 1070 such calls (V = 8001 .. 152064, K = 1 .. 24, four recipes) the
+// choice takes 1.006 times the best of the three (always staged 1.068, by the
+// number of sequences alone 1.033), and at worst 1.17 times the staged draw
+// (B=600 K=1 V=152063 f32).  The bonus row's race costs more per turn (four, two:
+// B=130 V=128256 bf16 30.4, 34.3, B=152 39.3, 36.5); its argmax under the PAPER
+// rule is one round of loads (B=450 V=128256 50.5, 55.1; V=32000 23.9, 23.4).
+// resident(nc): clusters of draw_kernel (nc > 0) or of the staged draw (0)
+// that the device holds at once.
 struct DrawPlan {
   int clusters, nc;                        // nc == 0: the staged residual draw
 };
-bool draw_plan(int dtype, bool sampled, bool bonus, int B, int V, DrawPlan* d) {
-  d->nc = 4;
-  if (sampled && !bonus && B <= draw_resident(dtype, V, 0)) d->nc = 0;
-  else if (B > 152) d->nc = 2;
-  int res = draw_resident(dtype, V, d->nc);
-  if (res < 1 && d->nc == 2) {
-    d->nc = 4;                             // (half a row's groups did not fit)
-    res = draw_resident(dtype, V, 4);
+template <typename Resident>
+bool draw_plan(int dtype, bool sampled, bool bonus, int B, int V, Resident resident, DrawPlan* d) {
+  const int es = dtype == CMSD_F32 ? 4 : 2;
+  const bool odd = (int64_t)V * es % 16 != 0;
+  const int64_t row = (int64_t)V * es * (odd ? 3 : 2) / 2;
+  const bool wide = row >= 290000, mid = row >= 140000;
+  const int64_t staged = sampled && !bonus ? resident(0) : 0;
+  int res = (int)staged;
+  d->nc = 0;
+  if (B > staged * (wide ? (odd ? 15 : 10) : (mid ? 7 : 5)) / 5) {
+    d->nc = 4;
+    res = resident(4);
+    int64_t most = res;                    // sequences with four CTAs each
+    if (!sampled) most = mid ? B : res;
+    else if (!bonus) most = (int64_t)res * (wide ? (odd ? 62 : 42) : (mid ? 40 : 21)) / 20;
+    const int two = B > most ? resident(2) : 0;      // (0: half a row's groups do not fit)
+    if (two > 0) {
+      d->nc = 2;
+      res = two;
+    }
   }
   d->clusters = B < 2 * res ? B : 2 * res;
   return res > 0;
+}
+bool draw_plan(int dtype, bool sampled, bool bonus, int B, int V, DrawPlan* d) {
+  return draw_plan(dtype, sampled, bonus, B, V, [&](int nc) { return draw_resident(dtype, V, nc); }, d);
 }
 
 cudaError_t launch_draw(int dtype, bool sampled, const StreamArgs& a, const DrawPlan& d, cudaStream_t s) {
@@ -685,6 +719,17 @@ int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bon
              [&](int n, int t) { return (int)resident[(t == 512 ? 17 : 0) + kSeqSizes[n]]; }, &nc, &th);
   *cluster = nc;
   *threads = nc > 0 ? th : 0;
+  return CMSD_OK;
+}
+
+int cmsd_test_draw(int B, int V, int dtype, int rule, int bonus, const int32_t* resident, int32_t* ctas) {
+  const int rc = check_sizes(B, 1, V, dtype, nullptr);
+  if (rc) return rc;
+  if (B < 1 || !resident || !ctas || (rule != CMSD_RULE_SAMPLED && !bonus)) return CMSD_EINVAL;
+  DrawPlan d;
+  const bool fits = draw_plan(dtype, rule == CMSD_RULE_SAMPLED, bonus != 0, B, V,
+                              [&](int nc) { return (int)resident[nc == 0 ? 0 : (nc == 4 ? 1 : 2)]; }, &d);
+  *ctas = fits ? d.nc : -1;
   return CMSD_OK;
 }
 

@@ -258,3 +258,27 @@ def test_choice_of_kernel_off_vector_boundaries(cmsd):
     assert 152064 > 4 * 16 * 256 * 8
     assert _choose(cmsd, GB300, VERIFY, 10, 1, 152064) == (16, 256)
     assert _choose(cmsd, GB300, VERIFY, 10, 1, 152063) == (10, 512)
+
+
+def _draw(cmsd, B, V, dtype, rule, bonus, resident):
+    table = np.ascontiguousarray(resident, np.int32)
+    n = ctypes.c_int32(-9)
+    assert cmsd.lib().cmsd_test_draw(B, V, dtype, rule, bonus, table.ctypes.data, ctypes.byref(n)) == cmsd.OK
+    return n.value
+
+
+def test_choice_of_the_second_kernel(cmsd):
+    # the sides measured on a GB300: (B, V, dtype, rule, bonus) -> CTAs per sequence, 0 the staged draw
+    bf16, f32 = [74, 148, 304], [36, 148, 304]
+    for args, resident, want in [
+            ((40, 128256, 1, 1, 0), bf16, 0), ((100, 128256, 1, 1, 0), bf16, 0), ((100, 32000, 1, 1, 0), bf16, 4),
+            ((40, 128255, 0, 1, 0), f32, 0), ((80, 128256, 0, 1, 0), f32, 4), ((180, 128255, 0, 1, 0), f32, 4),
+            ((180, 128255, 1, 1, 0), bf16, 0), ((180, 128256, 1, 1, 0), bf16, 4), ((300, 128255, 1, 1, 0), bf16, 4),
+            ((300, 128256, 1, 1, 0), bf16, 2), ((180, 32000, 1, 1, 0), bf16, 2), ((600, 152063, 1, 1, 0), bf16, 2),
+            ((130, 128256, 1, 1, 1), bf16, 4), ((152, 128256, 1, 1, 1), bf16, 2), ((450, 128256, 1, 0, 1), bf16, 4),
+            ((450, 32000, 1, 0, 1), bf16, 2)]:
+        assert _draw(cmsd, *args, resident) == want, args
+    # rows whose shares do not fit: no staged draw, no half row per CTA, no cluster at all
+    assert _draw(cmsd, 8, 1_000_000, 1, 1, 0, [0, 148, 304]) == 4
+    assert _draw(cmsd, 600, 1_500_000, 1, 1, 0, [0, 148, 0]) == 4
+    assert _draw(cmsd, 600, 3_100_000, 1, 1, 0, [0, 0, 0]) == -1
