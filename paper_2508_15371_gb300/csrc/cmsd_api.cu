@@ -253,22 +253,25 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 //
 // Both times are estimated, in microseconds, from what was measured on a
 // GB300 over K = 1..16, V = 32000..152064, B = 1..600 (bf16; f32 alike):
-//   streaming kernel   8 + bytes / 6900 MB/s, more when whole rows leave over
-//     a tenth of the warps without one (B=80 K=8 V=128256: 67.9), and with a
-//     second launch 7.5 more (12 with the bonus row), 0.045 (0.09) per
-//     sequence beyond 64, and 2.2 per 100000 entries where it draws from rows
-//     off 16-byte boundaries (B=30 K=8 ragged verify: V=128256 19.7, V=128255
-//     22.5);
-//   one launch         5, a draw 3.5 (4.5 by cluster_draw, which takes over at
-//     half the share off 16-byte boundaries: B=10 K=1 V=152063 verify 11.1 by
-//     16 CTAs of 256 threads, 9.4 raced by ten of 512), and the time of a
+//   streaming kernel   8 + bytes / 6900 MB/s, 1.5 to 3 more for ragged windows
+//     (their prefix, and rows cut on the device), more when whole rows leave
+//     over a tenth of the warps without one (B=80 K=8 V=128256: 67.9), and with
+//     a second launch 7.5 more (12 with the bonus row), 0.015 and 0.08 per MB
+//     of its row per sequence beyond 64 (twice with the bonus row), and 1.5 per
+//     100000 entries where it draws from rows off 16-byte boundaries (B=30 K=8
+//     ragged verify: V=128256 19.7, V=128255 22.5);
+//   one launch         5, a draw 3.5 (cluster_race) or 4.5 and 0.06 per KB of a
+//     CTA's share beyond 64 (cluster_draw; twice the share off 16-byte
+//     boundaries, where it takes over at half the share: B=10 K=1 V=152063
+//     verify 11.1 by 16 CTAs of 256 threads, 9.4 raced by ten of 512; one CTA a
+//     sequence, B=167 K=1 V=128255 f32 verify: 93.0, streamed 44.8), and the time of a
 //     sequence's bytes through its CTAs (a CTA of 256 threads: 27 KB a
 //     microsecond under the PAPER rule, 23.5 under the sampled rule, 21 for
 //     the drafter alone, 30 for the target alone (33 under the PAPER rule when
 //     windows are ragged, a fifth less off 16-byte boundaries); one of 512
 //     twice that; a tenth more with an SM to itself), times the waves when not
-//     every cluster is resident (3.5 more each, 10 with clusters of several
-//     CTAs), and no less than the bytes at 6900 MB/s.
+//     every cluster is resident (the draw and 3.5 more each, 10 with clusters of
+//     several CTAs), and no less than the bytes at 6900 MB/s.
 //
 // Every cluster should be resident at once, and not all of the number that the
 // occupancy query names are: clusters of 256-thread CTAs left some waiting
@@ -286,13 +289,13 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // A tenth more than the query names gained where windows were short (B=48 K=12
 // V=32001 sampled verify, 46 clusters of six resident: 13.6, by fives 15.6,
 // streamed 17.9) and lost more where they were full (31.5, 26.3, 28.2; B=38
-// K=8 V=128256 sampled 49.8 by eights, 35.4 by sevens, 39.8 streamed).  Over 442
-// ragged shapes (B = 1..200, three calls, both rules, with and without the
-// bonus row), windows spread over 0..K, all half and all full, the choice takes
-// 0.87, 0.81 and 0.85 of the streaming kernel's time (geometric mean; with that
-// tenth 0.86, 0.85, 0.92).  It was slower than the streaming kernel at
-// one of them (1.09, verify B=130 K=12 V=32001); with the tenth, and with three
-// tenths more for neighbours that end early, at one in eight, up to 1.37 times.
+// K=8 V=128256 sampled 49.8 by eights, 35.4 by sevens, 39.8 streamed).
+//
+// Over 6607 calls (K = 1 .. 16, B = 1 .. 600, V = 8000 .. 152064, ragged windows
+// spread over 0..K, half or full), each timed both ways and with up to ten
+// clusters, the choice takes 1.044 times the best of them and is slower than
+// the streaming kernel by over 3 % at 0.9 % of them, at worst 1.23 times (B=96
+// K=12 V=8000 PAPER, whose pieces come out uneven).
 //
 // sms: the device's; resident(n, threads): clusters of kSeqSizes[n] such CTAs
 // that it holds at once (a small partition may hold few or none of the large
@@ -311,11 +314,13 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
   }
   const int per = dtype == CMSD_F32 ? 4 : 8;             // entries per 16-byte vector
   const bool odd = a.V % per != 0;                       // rows off 16-byte boundaries
+  const double row = (double)a.V * (dtype == CMSD_F32 ? 4 : 2) * 1e-3;
   if (second) {
     flat += a.bonus ? 12 : 7.5;
-    if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 0.09 : 0.045);
-    if (sampled && odd) flat += 2.2e-5 * a.V;
+    if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 2 : 1) * (0.015 + 8e-5 * row * (sampled && odd ? 1.5 : 1));
+    if (sampled && odd) flat += 1.5e-5 * a.V;
   }
+  if (a.k_row) flat += mode == kModeFused ? 3 : (mode == kModeConf ? 2 : 1.5);
   double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 33) : (sampled ? 23.5 : 27));
   if (mode == kModeVerify && odd) rate *= 0.8;
   double best = 0.985 * flat;              // (a near tie stays with the streaming kernel)
@@ -327,7 +332,12 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       if (n > 1 && kb * 1e3 < (double)n * (th / 32) * 1024 * (mode == kModeFused ? 2 : 1)) break;
       // (cluster_race: two blocks of groups per lane set, one off 16-byte boundaries)
       const bool race = a.V <= (int64_t)(odd ? 4 : 8) * n * th * per;
-      const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + (second ? (sampled && !race ? 4.5 : 3.5) : 0);
+      double draw = second ? 3.5 : 0;
+      if (second && sampled && !race) {
+        const double share = row / (n * (th / 256)) * (odd ? 2 : 1);
+        draw = 4.5 + (share > 64 ? 0.06 * (share - 64) : 0.0);
+      }
+      const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + draw;
       const double full = kb / n / (rate * (th / 256));
       if (fixed + full / 1.1 >= best) continue;
       const int res = resident(k, th);
@@ -339,7 +349,8 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       const int waves = (a.B - 1) / fit + 1;
       const bool apart = (int64_t)a.B * n * (th / 256) <= sms;   // an SM to itself
       const double part = full / (apart ? 1.1 : 1.0);
-      const double t = fixed + (n == 1 ? 3.5 : 10.0) * (waves - 1) + (waves * part > stream ? waves * part : stream);
+      const double t = fixed + (draw + (n == 1 ? 3.5 : 10.0)) * (waves - 1) +
+                       (waves * part > stream ? waves * part : stream);
       if (t < best) {
         best = t;
         *nc = n;

@@ -282,3 +282,19 @@ def test_choice_of_the_second_kernel(cmsd):
     assert _draw(cmsd, 8, 1_000_000, 1, 1, 0, [0, 148, 304]) == 4
     assert _draw(cmsd, 600, 1_500_000, 1, 1, 0, [0, 148, 0]) == 4
     assert _draw(cmsd, 600, 3_100_000, 1, 1, 0, [0, 0, 0]) == -1
+
+
+def test_choice_of_kernel_counts_the_draws_share(cmsd):
+    # one CTA a sequence would take a whole long row's draw (B=167 K=1 V=128255
+    # f32 verify: 93.0 us, streamed 44.8; B=240 K=1 V=152063 fused: 72.3, 49.9)
+    for args in ((VERIFY, 167, 1, 128255, 0), (VERIFY, 155, 1, 152063, 1), (FUSED, 240, 1, 152063, 1),
+                 (FUSED, 300, 2, 128255, 0), (FUSED, 400, 2, 64127, 1)):
+        assert _choose(cmsd, GB300, *args) == (0, 0), args
+    assert _choose(cmsd, GB300, FUSED, 64, 8, 128256) == (4, 256)
+
+
+def test_choice_of_kernel_prices_ragged_streaming(cmsd):
+    # (B=310 K=1 V=8000 PAPER, windows of 0 and 1: 11.5 us streamed, 6.6 in one
+    # launch; B=155 K=2 V=32001 PAPER verify 9.7, 7.0)
+    assert _choose(cmsd, GB300, FUSED, 310, 1, 8000, 1, 0, 0, ragged=1) == (1, 256)
+    assert _choose(cmsd, GB300, VERIFY, 155, 2, 32001, 1, 0, 0, ragged=1)[0] > 0
