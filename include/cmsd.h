@@ -153,8 +153,8 @@ int cmsd_test_record_wait_timeout(const void* draft_logits, const void* target_l
  * resident[(threads == 512) * 17 + n] clusters of n CTAs of 256 or 512 threads
  * at once.  call: 0
  * cmsd_confidence, 1 cmsd_verify, 2 cmsd_confidence_verify; ragged: k_row is
- * given.  *cluster and *threads: the one-launch kernel's CTAs per sequence and
- * threads per CTA, or 0 for the streaming kernel. */
+ * given.  *cluster: the one-launch kernel's CTAs per sequence, or 0 for the
+ * streaming kernel; *threads: threads per CTA. */
 int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bonus, int ragged, int sms,
                      const int32_t* resident, int32_t* cluster, int32_t* threads);
 
@@ -333,9 +333,9 @@ int cmsd_profile_stop(float* stream_ms, float* resample_ms, int max_out, int* n_
 /* What a call of these sizes launches on the current device, without
  * launching it: call 0 cmsd_confidence, 1 cmsd_verify, 2
  * cmsd_confidence_verify; ragged: k_row is given.  *launches: kernels.
- * *cluster and *threads: the one-launch kernel's CTAs per sequence and threads
- * per CTA, or 0 where the streaming kernel takes the call.  Any of the three
- * may be NULL. */
+ * *cluster: the one-launch kernel's CTAs per sequence, or 0 where the streaming
+ * kernel takes the call; *threads: threads per CTA of that kernel.  Any of the
+ * three may be NULL. */
 int cmsd_launch_plan(int call, int B, int K, int V, int dtype, const cmsd_params* p, int ragged,
                      int* launches, int* cluster, int* threads);
 

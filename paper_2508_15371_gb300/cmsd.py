@@ -394,7 +394,7 @@ CONFIDENCE, VERIFY, FUSED = 0, 1, 2
 
 def launch_plan(call, B, K, V, dtype, p, ragged=False):
     """What a call (CONFIDENCE, VERIFY or FUSED) of these sizes launches on the current device:
-    (kernels, CTAs per sequence, threads per CTA), the last two 0 where the streaming kernel takes it."""
+    (kernels, CTAs per sequence or 0 where the streaming kernel takes it, threads per CTA)."""
     n, c, t = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_int(0)
     _check(lib().cmsd_launch_plan(call, B, K, V, int(dtype), ctypes.byref(p), int(bool(ragged)), ctypes.byref(n),
                                   ctypes.byref(c), ctypes.byref(t)), "cmsd_launch_plan")

@@ -48,19 +48,19 @@ int device_sms(int* sms) {
   return CMSD_OK;
 }
 
-int stream_grid(int dtype, int mode, bool sampled, bool second, size_t smem, int* grid) {
+int stream_grid(int dtype, int mode, bool sampled, bool second, int threads, size_t smem, int* grid) {
   int sms = 0;
   int rc = device_sms(&sms);
   if (rc) return rc;
   int dev = 0;
   cudaGetDevice(&dev);
-  const int variant = (sampled ? 1 : 0) | (second ? 2 : 0);
+  const int variant = (sampled ? 1 : 0) | (second ? 2 : 0) | threads << 2;
   const auto key = std::make_tuple(dev, dtype, mode, variant, (int)smem);
   std::lock_guard<std::mutex> lk(g_mu);
   auto it = g_occ.find(key);
   if (it == g_occ.end()) {
     int nb = 0;
-    cudaError_t e = occupancy_stream(dtype, mode, sampled, second, smem, &nb);
+    cudaError_t e = occupancy_stream(dtype, mode, sampled, second, threads, smem, &nb);
     if (e != cudaSuccess) return cuda_fail(e);
     if (nb < 1) nb = 1;
     it = g_occ.emplace(key, nb).first;
@@ -457,6 +457,32 @@ int choose(int dtype, int mode, bool sampled, bool second, const StreamArgs& a, 
   return CMSD_OK;
 }
 
+// Threads per CTA of the streaming kernel: kStreamThreads, but for short rows
+// that its warps' slices would cross the ends of (more rows than warps, or too
+// few of the warps used by whole pieces of a row).  There each row ends a
+// warp's pipeline and reduction, and more warps with shorter stages hide it:
+// 768 threads and two vectors against 512 and four, at 2880 rows (whole rows
+// again with 768) V=4000 sampled 0.82 of the time, V=16000 0.92, V=64128 0.96,
+// V=128256 1.03; at 7200 (crossed by both) V=8000 0.84, V=32000 0.90, V=50257
+// 0.96; PAPER at 816 rows V=4000 0.68 (14.7 against 21.6 us), V=32000 0.94; the
+// drafter alone at 7200 V=8000 0.92, V=32000 1.04.  Rows in whole pieces lose
+// 1 to 39 per cent by it (V=4000 at 2400 rows 1.23).  f32 rows gain at half the
+// length (V=8000 0.94, V=32000 0.98 at 2880 rows).  Ragged windows count half
+// their rows.
+int stream_threads(int dtype, int mode, bool sampled, const StreamArgs& a, int sms) {
+  const int64_t rows64 = (int64_t)a.B * a.K;
+  const int rows = (int)(a.k_row ? (rows64 + 1) / 2 : rows64);
+  const int vec = dtype == CMSD_F32 ? 4 : 8;
+  const int64_t min_len = stream_min_len(a.V);
+  if (StreamSplit(rows, a.V, vec, sms * (kStreamThreads / 32), min_len).wpr > 0) return kStreamThreads;
+  const bool whole = StreamSplit(rows, a.V, vec, sms * (kStreamThreadsShort / 32), min_len).wpr > 0;
+  int most;                                // entries of a bf16 row, in thousands
+  if (mode == kModeConf) most = whole ? 20 : 10;
+  else if (mode == kModeVerify) most = whole ? 65 : 33;
+  else most = sampled ? (whole ? 65 : 55) : (whole ? 33 : 20);
+  return (int64_t)a.V * (dtype == CMSD_F32 ? 4 : 1) <= most * 1000ll ? kStreamThreadsShort : kStreamThreads;
+}
+
 // (nc > 0: the one-launch kernel with that many CTAs of `threads` threads per
 // sequence, whatever the rule says)
 int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws_bytes,
@@ -486,7 +512,11 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
   }
   const size_t smem = stream_smem_bytes(a.B, a.k_row != nullptr);
   int grid = 0;
-  rc = stream_grid(dtype, mode, sampled, second, smem, &grid);
+  int sms = 0;
+  rc = device_sms(&sms);
+  if (rc) return rc;
+  const int st = stream_threads(dtype, mode, sampled, a, sms);
+  rc = stream_grid(dtype, mode, sampled, second, st, smem, &grid);
   if (rc) return rc;
   int g2 = 0;
   DrawPlan dp;
@@ -495,12 +525,12 @@ int launch(int dtype, int mode, bool sampled, StreamArgs& a, void* ws, size_t ws
     rc = resample_grid(dtype, sampled, &g2);
     if (rc) return rc;
   }
-  a.nwarps = grid * kStreamWarps;
+  a.nwarps = grid * (st / 32);
   if (!a.k_row) a.split = StreamSplit(a.B * a.K, a.V, dtype == CMSD_F32 ? 4 : 8, a.nwarps, stream_min_len(a.V));
   a.rec_by_seq = bound ? 1 : 0;
   prof_record(0, s);
-  cudaError_t e = dtype == CMSD_F32 ? launch_stream_f32(mode, sampled, second, a, grid, smem, s)
-                                    : launch_stream_bf16(mode, sampled, second, a, grid, smem, s);
+  cudaError_t e = dtype == CMSD_F32 ? launch_stream_f32(mode, sampled, second, a, grid, st, smem, s)
+                                    : launch_stream_bf16(mode, sampled, second, a, grid, st, smem, s);
   if (e != cudaSuccess) return cuda_fail(e);
   prof_record(1, s);
   if (second) {
@@ -729,7 +759,7 @@ int cmsd_test_choose(int call, int B, int K, int V, int dtype, int rule, int bon
   choose_seq(dtype, call, sampled, call != kModeConf && (sampled || bonus), a, sms,
              [&](int n, int t) { return (int)resident[(t == 512 ? 17 : 0) + kSeqSizes[n]]; }, &nc, &th);
   *cluster = nc;
-  *threads = nc > 0 ? th : 0;
+  *threads = nc > 0 ? th : stream_threads(dtype, call, sampled, a, sms);
   return CMSD_OK;
 }
 
@@ -927,6 +957,12 @@ int cmsd_launch_plan(int call, int B, int K, int V, int dtype, const cmsd_params
     rc = choose(dtype, call, sampled, second, a, &nc, &th);
     if (rc) return rc;
     nl = nc > 0 || !second ? 1 : 2;
+    if (nc == 0) {
+      int sms = 0;
+      rc = device_sms(&sms);
+      if (rc) return rc;
+      th = stream_threads(dtype, call, sampled, a, sms);
+    }
   }
   if (launches) *launches = nl;
   if (cluster) *cluster = nc;
@@ -939,7 +975,7 @@ int cmsd_launch_info(int dtype, int* warps_out, int* sms_out) {
   int sms = 0, grid = 0;
   int rc = device_sms(&sms);
   if (rc) return rc;
-  rc = stream_grid(dtype, kModeFused, true, true, stream_smem_bytes(0, false), &grid);
+  rc = stream_grid(dtype, kModeFused, true, true, kStreamThreads, stream_smem_bytes(0, false), &grid);
   if (rc) return rc;
   if (warps_out) *warps_out = grid * kStreamWarps;
   if (sms_out) *sms_out = sms;

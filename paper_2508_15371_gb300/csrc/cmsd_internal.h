@@ -5,16 +5,16 @@
 
 namespace cmsd {
 
-// The streaming kernel runs as few, large CTAs (one per SM by default): warps
-// of one CTA are scheduled evenly, warps of co-resident CTAs are not.  512
-// threads of 128 registers, four vectors per tensor and stage: B=256 K=16
-// V=152064 bf16 takes 382 us a sampled call against 395 us with 768 threads
-// and two (402 us with the loop that had conditions and copies in it), 480 and
-// 448 threads 388 and 397 us, two CTAs of 256 threads 389 us.
-#ifndef CMSD_STREAM_THREADS
-#define CMSD_STREAM_THREADS 512
-#endif
-constexpr int kStreamThreads = CMSD_STREAM_THREADS;
+// The streaming kernel runs as few, large CTAs (one per SM): warps of one CTA
+// are scheduled evenly, warps of co-resident CTAs are not.  512 threads of 128
+// registers, four vectors per tensor and stage: B=256 K=16 V=152064 bf16 takes
+// 382 us a sampled call against 395 us with 768 threads and two (402 us with the
+// loop that had conditions and copies in it), 480 and 448 threads 388 and 397
+// us, two CTAs of 256 threads 389 us.  Short rows that warps cross the ends of
+// take 768 threads and two vectors (stream_threads in cmsd_api.cu).
+constexpr int kStreamThreads = 512;
+constexpr int kStreamThreadsShort = 768;
+__host__ __device__ constexpr int stream_unroll(int threads) { return threads > kStreamThreads ? 2 : 4; }
 #ifndef CMSD_RES_THREADS
 #define CMSD_RES_THREADS 256
 #endif
@@ -202,9 +202,10 @@ struct StreamArgs {
 
 // Kernel launchers (one translation unit per dtype).  `second`: this call
 // queues rows for the resample kernel (sampled rule or bonus row).
-cudaError_t launch_stream_f32(int mode, bool sampled, bool second, const StreamArgs& a, int grid,
+// threads: kStreamThreads or kStreamThreadsShort.
+cudaError_t launch_stream_f32(int mode, bool sampled, bool second, const StreamArgs& a, int grid, int threads,
                               size_t smem, cudaStream_t s);
-cudaError_t launch_stream_bf16(int mode, bool sampled, bool second, const StreamArgs& a, int grid,
+cudaError_t launch_stream_bf16(int mode, bool sampled, bool second, const StreamArgs& a, int grid, int threads,
                                size_t smem, cudaStream_t s);
 // The pass in one launch, a cluster of nc CTAs of `threads` (256 or 512)
 // threads per sequence (cmsd_seq_impl.cuh).
@@ -232,7 +233,7 @@ cudaError_t launch_resample_bound_f32(const StreamArgs& a, int clusters, cudaStr
 cudaError_t launch_resample_bound_bf16(const StreamArgs& a, int clusters, cudaStream_t s);
 int resample_bound_clusters_f32(int V);
 int resample_bound_clusters_bf16(int V);
-cudaError_t occupancy_stream(int dtype, int mode, bool sampled, bool second, size_t smem,
+cudaError_t occupancy_stream(int dtype, int mode, bool sampled, bool second, int threads, size_t smem,
                              int* blocks_per_sm);
 cudaError_t occupancy_resample(int dtype, bool sampled, int* blocks_per_sm);
 cudaError_t launch_philox_fill(unsigned long long seed, uint32_t c0, uint32_t c1, uint32_t c2,

@@ -3,13 +3,13 @@
 
 namespace cmsd {
 
-cudaError_t launch_stream_bf16(int mode, bool sampled, bool second, const StreamArgs& a, int grid,
+cudaError_t launch_stream_bf16(int mode, bool sampled, bool second, const StreamArgs& a, int grid, int threads,
                                size_t smem, cudaStream_t s) {
-  return launch_stream_t<uint16_t>(mode, sampled, second, a, grid, smem, s);
+  return launch_stream_t<uint16_t>(mode, sampled, second, a, grid, threads, smem, s);
 }
 
-cudaError_t occupancy_stream_bf16(int mode, bool sampled, bool second, size_t smem, int* nb) {
-  return occupancy_stream_t<uint16_t>(mode, sampled, second, smem, nb);
+cudaError_t occupancy_stream_bf16(int mode, bool sampled, bool second, int threads, size_t smem, int* nb) {
+  return occupancy_stream_t<uint16_t>(mode, sampled, second, threads, smem, nb);
 }
 
 cudaError_t launch_resample_bf16(bool sampled, const StreamArgs& a, int grid, cudaStream_t s) {

@@ -942,9 +942,6 @@ __device__ void seg_finish(const StreamArgs& a, SegState& ss, const Seg& sg, int
 // t = 0, 1, ...; stage s holds t in [s*U, s*U + U) and is loaded (streaming,
 // no L1 allocation) while stage s-1 is reduced.  Only the last stage can be
 // partial: its missing vectors read as -inf, which adds nothing.
-#ifndef CMSD_UNROLL
-#define CMSD_UNROLL 4
-#endif
 template <typename T>
 __device__ __forceinline__ uint4 neg_inf_vec() {
   return sizeof(T) == 2 ? make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2)
@@ -1069,7 +1066,7 @@ __device__ __forceinline__ void pipe_run(Pipe<T, U>& p, SegState& ss, int va, in
 // Order of a segment's start: its first stage of logits is requested, then
 // the logits at its drafted token (whose index was requested one segment
 // earlier), so the slice's first loads are not held up behind the token.
-template <typename T, int MODE, bool SAMPLED, bool PH2>
+template <typename T, int MODE, bool SAMPLED, bool PH2, int U>
 __device__ void walk_slice(const StreamArgs& a, const int* s_pref, int64_t e_begin, int64_t e_end,
                            const StreamSplit& sp, int w, int lane) {
   constexpr bool HAS_D = MODE != kModeVerify;
@@ -1084,7 +1081,7 @@ __device__ void walk_slice(const StreamArgs& a, const int* s_pref, int64_t e_beg
     e0 += len;
     const T* dp = (const T*)a.draft + (size_t)sg.r * (size_t)a.V;
     const T* tp = HAS_T ? (const T*)a.target + ((size_t)sg.b * a.Kt + sg.i) * (size_t)a.V : nullptr;
-    Pipe<T, CMSD_UNROLL> pp;
+    Pipe<T, U> pp;
     pipe_start<T, MODE>(pp, dp, tp, sg.va, sg.vb, lane);
     float c = 0.f, zd = 0.f;
     if (HAS_T) {
@@ -2377,15 +2374,15 @@ __global__ void __launch_bounds__(kCluThreads, 2) resample_bound_kernel(const St
 // the kernel
 // ---------------------------------------------------------------------------
 
-template <typename T, int MODE, bool SAMPLED, bool PH2>
-__global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamArgs a) {
+template <typename T, int MODE, bool SAMPLED, bool PH2, int NT>
+__global__ void __launch_bounds__(NT, 1) stream_kernel(const StreamArgs a) {
   constexpr bool HAS_D = MODE != kModeVerify;
   constexpr bool HAS_T = MODE != kModeConf;
   constexpr int VEC = Elem<T>::kVec;
   extern __shared__ __align__(128) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
-  const int w = blockIdx.x * kStreamWarps + warp;
+  const int w = blockIdx.x * (NT / 32) + warp;
   const Workspace& W = a.ws;
   const bool ragged = a.k_row != nullptr;
   int* s_pref = reinterpret_cast<int*>(smem);
@@ -2399,7 +2396,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
   // -- present rows: exclusive prefix of k_row (ragged windows) -------------
   int nrows;
   if (ragged) {
-    const int per = (a.B + kStreamThreads - 1) / kStreamThreads;
+    const int per = (a.B + NT - 1) / NT;
     const int b0 = threadIdx.x * per;
     int tot = 0;
     for (int b = b0; b < b0 + per && b < a.B; ++b) tot += k_of(a, b);
@@ -2409,7 +2406,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
       const int y = __shfl_up_sync(kFull, incl, o);
       if (lane >= o) incl += y;
     }
-    __shared__ int s_wsum[kStreamWarps];
+    __shared__ int s_wsum[NT / 32];
     if (lane == 31) s_wsum[warp] = incl;
     __syncthreads();
     int wofs = 0;
@@ -2419,7 +2416,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
       s_pref[b] = run;
       run += k_of(a, b);
     }
-    if (threadIdx.x == kStreamThreads - 1) s_pref[a.B] = run;
+    if (threadIdx.x == NT - 1) s_pref[a.B] = run;
     __syncthreads();
     nrows = s_pref[a.B];
   } else {
@@ -2428,8 +2425,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
 
   // -- sequences with no present position, and k_row range errors -----------
   if (ragged) {
-    const int gt = blockIdx.x * kStreamThreads + threadIdx.x;
-    const int gn = gridDim.x * kStreamThreads;
+    const int gt = blockIdx.x * NT + threadIdx.x;
+    const int gn = gridDim.x * NT;
     for (int b = gt; b < a.B; b += gn) {
       const int raw = __ldg(a.k_row + b);
       if (raw < 0 || raw > a.K) atomicOr(W.err, 2u);
@@ -2453,7 +2450,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
     if (w < sp.W) {
       const int64_t e_begin = sp.start(w);
       const int64_t e_end = sp.start(w + 1);
-      if (e_begin < e_end) walk_slice<T, MODE, SAMPLED, PH2>(a, s_pref, e_begin, e_end, sp, w, lane);
+      if (e_begin < e_end) walk_slice<T, MODE, SAMPLED, PH2, stream_unroll(NT)>(a, s_pref, e_begin, e_end, sp, w, lane);
     }
   }
 }
@@ -2474,14 +2471,14 @@ cudaError_t smem_attr_once(K kernel, unsigned long long* done_mask) {
   return e;
 }
 
-template <typename T, int MODE, bool SAMPLED, bool PH2>
+template <typename T, int MODE, bool SAMPLED, bool PH2, int NT>
 cudaError_t launch_one(const StreamArgs& a, int grid, size_t smem, cudaStream_t s) {
   static unsigned long long done = 0ull;
-  cudaError_t e = smem_attr_once(stream_kernel<T, MODE, SAMPLED, PH2>, &done);
+  cudaError_t e = smem_attr_once(stream_kernel<T, MODE, SAMPLED, PH2, NT>, &done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(kStreamThreads);
+  cfg.blockDim = dim3(NT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -2489,16 +2486,15 @@ cudaError_t launch_one(const StreamArgs& a, int grid, size_t smem, cudaStream_t 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, stream_kernel<T, MODE, SAMPLED, PH2>, a);
+  return cudaLaunchKernelEx(&cfg, stream_kernel<T, MODE, SAMPLED, PH2, NT>, a);
 }
 
-template <typename T, int MODE, bool SAMPLED, bool PH2>
+template <typename T, int MODE, bool SAMPLED, bool PH2, int NT>
 cudaError_t occupancy_one(size_t smem, int* nb) {
   static unsigned long long done = 0ull;
-  cudaError_t e = smem_attr_once(stream_kernel<T, MODE, SAMPLED, PH2>, &done);
+  cudaError_t e = smem_attr_once(stream_kernel<T, MODE, SAMPLED, PH2, NT>, &done);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, stream_kernel<T, MODE, SAMPLED, PH2>,
-                                                       kStreamThreads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, stream_kernel<T, MODE, SAMPLED, PH2, NT>, NT, smem);
 }
 
 // Launched as a programmatic dependent of the streaming kernel just before it
@@ -2678,28 +2674,30 @@ cudaError_t occupancy_resample_t(bool sampled, int* nb) {
 // The kernel variants: confidence only; verify and fused, each under the
 // PAPER rule without a second pass, the PAPER rule with the bonus row, and
 // the sampled rule (always a second pass).
-#define CMSD_DISPATCH(FN, ...)                                                              \
-  do {                                                                                      \
-    if (mode == kModeConf) return FN<T, kModeConf, false, false>(__VA_ARGS__);              \
-    if (mode == kModeVerify) {                                                              \
-      if (sampled) return FN<T, kModeVerify, true, true>(__VA_ARGS__);                      \
-      if (second) return FN<T, kModeVerify, false, true>(__VA_ARGS__);                      \
-      return FN<T, kModeVerify, false, false>(__VA_ARGS__);                                 \
-    }                                                                                       \
-    if (sampled) return FN<T, kModeFused, true, true>(__VA_ARGS__);                         \
-    if (second) return FN<T, kModeFused, false, true>(__VA_ARGS__);                         \
-    return FN<T, kModeFused, false, false>(__VA_ARGS__);                                    \
+#define CMSD_DISPATCH(FN, NT, ...)                                                              \
+  do {                                                                                          \
+    if (mode == kModeConf) return FN<T, kModeConf, false, false, NT>(__VA_ARGS__);              \
+    if (mode == kModeVerify) {                                                                  \
+      if (sampled) return FN<T, kModeVerify, true, true, NT>(__VA_ARGS__);                      \
+      if (second) return FN<T, kModeVerify, false, true, NT>(__VA_ARGS__);                      \
+      return FN<T, kModeVerify, false, false, NT>(__VA_ARGS__);                                 \
+    }                                                                                           \
+    if (sampled) return FN<T, kModeFused, true, true, NT>(__VA_ARGS__);                         \
+    if (second) return FN<T, kModeFused, false, true, NT>(__VA_ARGS__);                         \
+    return FN<T, kModeFused, false, false, NT>(__VA_ARGS__);                                    \
   } while (0)
 
 template <typename T>
-cudaError_t launch_stream_t(int mode, bool sampled, bool second, const StreamArgs& a, int grid, size_t smem,
-                            cudaStream_t s) {
-  CMSD_DISPATCH(launch_one, a, grid, smem, s);
+cudaError_t launch_stream_t(int mode, bool sampled, bool second, const StreamArgs& a, int grid, int threads,
+                            size_t smem, cudaStream_t s) {
+  if (threads == kStreamThreadsShort) CMSD_DISPATCH(launch_one, kStreamThreadsShort, a, grid, smem, s);
+  CMSD_DISPATCH(launch_one, kStreamThreads, a, grid, smem, s);
 }
 
 template <typename T>
-cudaError_t occupancy_stream_t(int mode, bool sampled, bool second, size_t smem, int* nb) {
-  CMSD_DISPATCH(occupancy_one, smem, nb);
+cudaError_t occupancy_stream_t(int mode, bool sampled, bool second, int threads, size_t smem, int* nb) {
+  if (threads == kStreamThreadsShort) CMSD_DISPATCH(occupancy_one, kStreamThreadsShort, smem, nb);
+  CMSD_DISPATCH(occupancy_one, kStreamThreads, smem, nb);
 }
 #undef CMSD_DISPATCH
 

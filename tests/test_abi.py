@@ -194,7 +194,16 @@ def _choose(cmsd, resident, call, B, K, V, dtype=1, rule=1, bonus=0, ragged=0, s
     rc = cmsd.lib().cmsd_test_choose(call, B, K, V, dtype, rule, bonus, ragged, sms, table.ctypes.data,
                                      ctypes.byref(nc), ctypes.byref(th))
     assert rc == cmsd.OK
-    return nc.value, th.value
+    assert th.value in ((256, 512) if nc.value else (512, 768))
+    return (nc.value, th.value) if nc.value else (0, 0)
+
+
+def _stream_threads(cmsd, call, B, K, V, dtype=1, rule=1, ragged=0):
+    table = np.zeros((2, 17), np.int32)               # no cluster fits: the streaming kernel
+    nc, th = ctypes.c_int32(-1), ctypes.c_int32(-1)
+    assert cmsd.lib().cmsd_test_choose(call, B, K, V, dtype, rule, 0, ragged, 152, table.ctypes.data, ctypes.byref(nc),
+                                       ctypes.byref(th)) == cmsd.OK and nc.value == 0
+    return th.value
 
 
 def test_choice_of_kernel_where_one_cluster_fits(cmsd):
@@ -298,3 +307,17 @@ def test_choice_of_kernel_prices_ragged_streaming(cmsd):
     # launch; B=155 K=2 V=32001 PAPER verify 9.7, 7.0)
     assert _choose(cmsd, GB300, FUSED, 310, 1, 8000, 1, 0, 0, ragged=1) == (1, 256)
     assert _choose(cmsd, GB300, VERIFY, 155, 2, 32001, 1, 0, 0, ragged=1)[0] > 0
+
+
+def test_short_rows_crossed_by_slices_take_more_warps(cmsd):
+    # 2432 warps of 512 threads per SM: 2400 and 1190 rows in whole pieces, 816,
+    # 2880 and 7200 not
+    for B, K, want in ((100, 24, 512), (70, 17, 512), (48, 17, 768), (180, 16, 768), (300, 24, 768)):
+        for call, rule in ((FUSED, 0), (FUSED, 1), (CONF, 0), (VERIFY, 0), (VERIFY, 1)):
+            assert _stream_threads(cmsd, call, B, K, 8000, rule=rule) == want, (B, K, call, rule)
+        assert _stream_threads(cmsd, FUSED, B, K, 128256) == 512                    # long rows
+        assert _stream_threads(cmsd, FUSED, 2 * B, K, 8000, ragged=1) == want       # half full on average
+    assert _stream_threads(cmsd, CONF, 300, 24, 32000) == 512 and _stream_threads(cmsd, FUSED, 300, 24, 32000) == 768
+    assert _stream_threads(cmsd, FUSED, 300, 24, 8000, dtype=0) == 768
+    assert _stream_threads(cmsd, FUSED, 300, 24, 32000, dtype=0) == 512
+    assert _stream_threads(cmsd, FUSED, 1 << 20, 1024, 8000) == 768
