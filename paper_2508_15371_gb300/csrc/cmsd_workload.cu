@@ -41,10 +41,10 @@ __device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
                : "memory");
 }
 
-// One cluster per (b, i) slot of the [B][Kt] verifier layout.
+// One cluster per (b, i) slot of the [B][Kt] verifier layout, from slot0 on.
 __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_rows_kernel(const float* __restrict__ table,
                                                             const float* __restrict__ heights_it,
-                                                            uint32_t it, int B, int K_max, int Kt, int V,
+                                                            uint32_t it, int slot0, int B, int K_max, int Kt, int V,
                                                             const int32_t* __restrict__ k_row,
                                                             uint32_t k0, uint32_t k1, float* draft,
                                                             float* target, int32_t* tokens) {
@@ -52,7 +52,8 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
   // writes nothing before that has completed
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int slot = blockIdx.x / kParts, part = blockIdx.x - slot * kParts;
+  const int cluster = blockIdx.x / kParts, part = blockIdx.x - cluster * kParts;
+  const int slot = slot0 + cluster;
   const int i = slot / B;                       // position-major: the idle slots come last
   const int b = slot - i * B;
   int k = K_max;
@@ -169,8 +170,10 @@ extern "C" int cmsd_gen_decode_rows(const float* table, const float* heights_it,
   if (B < 0 || K_max < 1 || V < 2 || (Kt != K_max && Kt != K_max + 1)) return -1;
   if (B == 0) return 0;
   if (!table || !heights_it || !draft || !target || !tokens) return -1;
+  const int64_t slots = (int64_t)B * Kt;        // (as many launches as a grid of 2^31 - 1 CTAs needs: one)
+  if (slots > 0x7FFFFFFFll) return -1;
+  constexpr int kMostSlots = 0x7FFFFFFF / kParts;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(B * Kt * kParts));
   cfg.blockDim = dim3(kThreads);
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute attr[1];
@@ -178,8 +181,12 @@ extern "C" int cmsd_gen_decode_rows(const float* table, const float* heights_it,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gen_rows_kernel, table, heights_it, it, B, K_max, Kt, V, k_row, cmsd::seed_lo(seed),
-                            cmsd::seed_hi(seed), draft, target, tokens) == cudaSuccess
-             ? 0
-             : -3;
+  for (int64_t s0 = 0; s0 < slots; s0 += kMostSlots) {
+    const int64_t n = slots - s0 < kMostSlots ? slots - s0 : kMostSlots;
+    cfg.gridDim = dim3((unsigned)(n * kParts));
+    if (cudaLaunchKernelEx(&cfg, gen_rows_kernel, table, heights_it, it, (int)s0, B, K_max, Kt, V, k_row,
+                           cmsd::seed_lo(seed), cmsd::seed_hi(seed), draft, target, tokens) != cudaSuccess)
+      return -3;
+  }
+  return 0;
 }

@@ -60,6 +60,36 @@ def test_device_generator_matches_host(mods, V, k_row, bonus):
                 assert np.array_equal(t[b, i].view(np.uint32), ht[i].view(np.uint32)), (it, b, i)
 
 
+@pytest.mark.gpu
+def test_generator_takes_more_slots_than_one_grid_holds(mods):
+    """2^29 + 5 sequences of which three have a row: four CTAs a slot are more
+    than a grid of 2^31 - 1."""
+    import collections
+    cmsd, ds, W = mods
+    B, K, V = 2 ** 29 + 5, 1, 2
+    free, _ = torch.cuda.mem_get_info()
+    if free < 24 << 30:
+        pytest.skip("needs 24 GB of device memory")
+    k_row = torch.zeros(B, dtype=torch.int32, device="cuda")
+    heights = torch.zeros(B, dtype=torch.float32, device="cuda")
+    draft = torch.zeros((B, V), dtype=torch.float32, device="cuda")
+    target = torch.zeros((B, V), dtype=torch.float32, device="cuda")
+    tokens = torch.full((B,), -1, dtype=torch.int32, device="cuda")
+    table = torch.from_numpy(W.normal_table()).cuda()
+    rows = [0, 2 ** 29 - 2, B - 1]
+    k_row[rows] = 1
+    assert ds.wlib().cmsd_gen_decode_rows(table.data_ptr(), heights.data_ptr(), 3, B, K, K, V, k_row.data_ptr(), 4,
+                                          draft.data_ptr(), target.data_ptr(), tokens.data_ptr(), cmsd._stream()) == 0
+    torch.cuda.synchronize()
+    host = collections.defaultdict(float)
+    for b in rows:
+        d, t, tok = W.decode_row_host(W.normal_table(), host, 3, b, 0, K, V, 4)
+        assert np.array_equal(draft[b].cpu().numpy(), d) and np.array_equal(target[b].cpu().numpy(), t), b
+        assert int(tokens[b]) == tok, b
+    tokens[rows] = -1
+    assert int((tokens != -1).sum()) == 0
+
+
 def _compare_with_oracle(cmsd, ds, W, B, K, V, iterations, rule, seqs, graph=False, **kw):
     import oracle as O
     p = cmsd.params(K, rule, beta_rank=0 if rule == "sampled" else 3, **kw)
