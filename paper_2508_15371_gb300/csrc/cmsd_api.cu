@@ -253,13 +253,13 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 //
 // Both times are estimated, in microseconds, from what was measured on a
 // GB300 over K = 1..16, V = 32000..152064, B = 1..600 (bf16; f32 alike):
-//   streaming kernel   8 + bytes / 6900 MB/s, 1.5 to 3 more for ragged windows
+//   streaming kernel   8 + bytes / 6900 MB/s, up to 3 more for ragged windows
 //     (their prefix, and rows cut on the device), more when whole rows leave
 //     over a tenth of the warps without one (B=80 K=8 V=128256: 67.9), and with
-//     a second launch 7.5 more (12 with the bonus row), 0.015 and 0.08 per MB
-//     of its row per sequence beyond 64 (twice with the bonus row), and 1.5 per
-//     100000 entries where it draws from rows off 16-byte boundaries (B=30 K=8
-//     ragged verify: V=128256 19.7, V=128255 22.5);
+//     a second launch 7.5 more (11 with the bonus row), 0.015 and 0.08 per MB
+//     of its row per sequence beyond 64, and 1.5 per 100000 entries where it
+//     draws from rows off 16-byte boundaries (B=30 K=8 ragged verify: V=128256
+//     19.7, V=128255 22.5);
 //   one launch         5, a draw 3.5 (cluster_race) or 4.5 and 0.06 per KB of a
 //     CTA's share beyond 64 (cluster_draw; twice the share off 16-byte
 //     boundaries, where it takes over at half the share: B=10 K=1 V=152063
@@ -269,7 +269,9 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 //     microsecond under the PAPER rule, 23.5 under the sampled rule, 21 for
 //     the drafter alone, 30 for the target alone (33 under the PAPER rule when
 //     windows are ragged, a fifth less off 16-byte boundaries); one of 512
-//     twice that; a tenth more with an SM to itself), times the waves when not
+//     twice that; a tenth more with an SM to itself, a tenth (sampled: a fifth)
+//     more when both tensors' windows are ragged and neighbours end early),
+//     times the waves when not
 //     every cluster is resident (the draw and 3.5 more each, 10 with clusters of
 //     several CTAs), and no less than the bytes at 6900 MB/s.
 //
@@ -288,14 +290,14 @@ int seq_resident(int dev, int dtype, int n, int threads) {
 // also all be full, so no more clusters count as resident than of full windows.
 // A tenth more than the query names gained where windows were short (B=48 K=12
 // V=32001 sampled verify, 46 clusters of six resident: 13.6, by fives 15.6,
-// streamed 17.9) and lost more where they were full (31.5, 26.3, 28.2; B=38
+// streamed 18.1) and lost more where they were full (22.0, 17.6, 21.5; B=38
 // K=8 V=128256 sampled 49.8 by eights, 35.4 by sevens, 39.8 streamed).
 //
-// Over 6607 calls (K = 1 .. 16, B = 1 .. 600, V = 8000 .. 152064, ragged windows
-// spread over 0..K, half or full), each timed both ways and with up to ten
-// clusters, the choice takes 1.044 times the best of them and is slower than
-// the streaming kernel by over 3 % at 0.9 % of them, at worst 1.23 times (B=96
-// K=12 V=8000 PAPER, whose pieces come out uneven).
+// Over 7237 calls (K = 1 .. 16, B = 1 .. 600, V = 8000 .. 152064, ragged windows
+// of a third of K on average, spread over 0..K, half or full), each timed both
+// ways and with up to ten clusters, the choice takes 1.042 times the best of
+// them and is slower than the streaming kernel by over 3 % at 1.0 % of them, at
+// worst 1.23 times (B=96 K=12 V=8000 PAPER, whose pieces come out uneven).
 //
 // sms: the device's; resident(n, threads): clusters of kSeqSizes[n] such CTAs
 // that it holds at once (a small partition may hold few or none of the large
@@ -316,11 +318,11 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
   const bool odd = a.V % per != 0;                       // rows off 16-byte boundaries
   const double row = (double)a.V * (dtype == CMSD_F32 ? 4 : 2) * 1e-3;
   if (second) {
-    flat += a.bonus ? 12 : 7.5;
-    if (a.B > 64) flat += (a.B - 64) * (a.bonus ? 2 : 1) * (0.015 + 8e-5 * row * (sampled && odd ? 1.5 : 1));
+    flat += a.bonus ? 11 : 7.5;
+    if (a.B > 64) flat += (a.B - 64) * (0.015 + 8e-5 * row * (sampled && odd ? 1.5 : 1));
     if (sampled && odd) flat += 1.5e-5 * a.V;
   }
-  if (a.k_row) flat += mode == kModeFused ? 3 : (mode == kModeConf ? 2 : 1.5);
+  if (a.k_row) flat += mode == kModeVerify ? 2.5 : (second && sampled && a.bonus ? 0.5 : 3);
   double rate = mode == kModeConf ? 21 : (mode == kModeVerify ? (sampled || !a.k_row ? 30 : 33) : (sampled ? 23.5 : 27));
   if (mode == kModeVerify && odd) rate *= 0.8;
   double best = 0.985 * flat;              // (a near tie stays with the streaming kernel)
@@ -339,7 +341,7 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       }
       const double fixed = 5 + (th == 512 ? 0.7 : 0.0) + draw;
       const double full = kb / n / (rate * (th / 256));
-      if (fixed + full / 1.1 >= best) continue;
+      if (fixed + full / 1.32 >= best) continue;
       const int res = resident(k, th);
       if (res < 1) continue;
       int fit = res;
@@ -347,8 +349,9 @@ bool choose_seq(int dtype, int mode, bool sampled, bool second, const StreamArgs
       else if (th == 256 && n >= 3) fit = res * 93 / 100;
       if (fit < 1) fit = 1;
       const int waves = (a.B - 1) / fit + 1;
-      const bool apart = (int64_t)a.B * n * (th / 256) <= sms;   // an SM to itself
-      const double part = full / (apart ? 1.1 : 1.0);
+      double ease = (int64_t)a.B * n * (th / 256) <= sms ? 1.1 : 1.0;          // an SM to itself
+      if (a.k_row && mode == kModeFused && waves == 1) ease *= sampled ? 1.2 : 1.1;   // neighbours that end early
+      const double part = full / ease;
       const double t = fixed + (draw + (n == 1 ? 3.5 : 10.0)) * (waves - 1) +
                        (waves * part > stream ? waves * part : stream);
       if (t < best) {

@@ -307,6 +307,9 @@ def test_choice_of_kernel_prices_ragged_streaming(cmsd):
     # launch; B=155 K=2 V=32001 PAPER verify 9.7, 7.0)
     assert _choose(cmsd, GB300, FUSED, 310, 1, 8000, 1, 0, 0, ragged=1) == (1, 256)
     assert _choose(cmsd, GB300, VERIFY, 155, 2, 32001, 1, 0, 0, ragged=1)[0] > 0
+    # (B=32 K=16 V=32000 f32 sampled, windows of a third on average 19.5 us
+    # streamed, 17.0 by eights; spread over 0..K 26.8, 24.7; full 35.2, 29.1)
+    assert _choose(cmsd, GB300, FUSED, 32, 16, 32000, 0, 1, 0, ragged=1) == (8, 256)
 
 
 def test_short_rows_crossed_by_slices_take_more_warps(cmsd):
