@@ -212,8 +212,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
   // where the loop has no two registers to spare (PAPER, in registers: spills,
   // and B=32 K=8 V=128256 26.4 us against 25.5), else in registers (the
   // drafter alone, in shared memory: spills, and B=64 K=1 V=50257 5.3 us
-  // against 4.8).
-  constexpr bool kStash = MODE == kModeFused || (MODE == kModeVerify && !SAMPLED);
+  // against 4.8).  The bf16 target alone, PAPER, requests them afterwards (B=48
+  // K=8 V=64127 11.9 us; in registers 12.6, in shared memory 12.7).
+  constexpr bool kStash = MODE == kModeFused;
+  constexpr bool kLate = MODE == kModeVerify && !SAMPLED && VEC == 8;
   __shared__ float2 s_tail[kStash ? NW : 1][VEC - 1];
   cg::cluster_group cl = cg::this_cluster();
   const int nc = sp.nc;
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     const int hd = sg.va - sg.v0, tl = sg.v1 - sg.vb;
     const int ve = lane < hd ? sg.v0 + lane : sg.v1 - 32 + lane;
     float ze_d = 0.f, ze_t = 0.f;
-    if (lane < hd || lane >= 32 - tl) {
+    if (lane < hd || (!kLate && lane >= 32 - tl)) {
       if (HAS_D) ze_d = Elem<T>::load(dp + ve);
       if (HAS_T) ze_t = Elem<T>::load(tp + ve);
     }
@@ -300,8 +302,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) seq_kernel(const StreamArgs a, c
     }
     pipe_run<T, MODE, SAMPLED>(pp, ss, sg.va, beta, lane);
     if (lane >= 32 - (sg.v1 - sg.vb)) {
-      const float2 z = kStash ? s_tail[warp][lane - 33 + VEC] : make_float2(ze_d, ze_t);
       const int v = sg.v1 - 32 + lane;
+      float2 z = make_float2(ze_d, ze_t);
+      if (kStash) z = s_tail[warp][lane - 33 + VEC];
+      if (kLate) z.y = Elem<T>::load(tp + v);
       if (HAS_D) d_scalar(ss.d, z.x, v);
       if (HAS_T) t_scalar<SAMPLED>(ss.t, z.y, v, ss.c, beta);
     }
