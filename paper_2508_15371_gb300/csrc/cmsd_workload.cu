@@ -85,9 +85,10 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
   const int ngrp = (V + 7) / 8;
   // rows start on 32-byte boundaries when V is a multiple of 8 and the tensors
   // do: each thread then writes its 8 logits in one store; on 16-byte ones when
-  // V is a multiple of 4: two stores
-  const bool vec = (V & 3) == 0;
-  const bool vec8 = (V & 7) == 0 && ((((uintptr_t)draft) | ((uintptr_t)target)) & 31) == 0;
+  // V is a multiple of 4 and the tensors do: two stores
+  const uintptr_t at = ((uintptr_t)draft) | ((uintptr_t)target);
+  const bool vec = (V & 3) == 0 && (at & 15) == 0;
+  const bool vec8 = (V & 7) == 0 && (at & 31) == 0;
   for (int g = part * kThreads + threadIdx.x; g < ngrp; g += kParts * kThreads) {
     const cmsd::U4 wd = cmsd::philox4x32_10(cmsd::U4{(uint32_t)g, (uint32_t)row, it, kGenDNoise}, k0, k1);
     const cmsd::U4 wt = cmsd::philox4x32_10(cmsd::U4{(uint32_t)g, (uint32_t)row, it, kGenTNoise}, k0, k1);

@@ -61,6 +61,33 @@ def test_device_generator_matches_host(mods, V, k_row, bonus):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("V", [1000, 1004, 1001])
+@pytest.mark.parametrize("skip", [(1, 0), (0, 1), (4, 4), (2, 3)])
+def test_generator_writes_at_any_float(mods, V, skip):
+    """Tensors that start some floats past a 32-byte boundary."""
+    cmsd, ds, W = mods
+    B, K = 2, 2
+    table = W.normal_table()
+    heights = W.ar1_heights(B, 1, 4, table)
+    buf = [torch.full((n * V + 8,), 7.0, dtype=torch.float32, device="cuda") for n in (B * K, B * K)]
+    assert all(x.data_ptr() % 32 == 0 for x in buf)
+    tok = torch.zeros((B, K), dtype=torch.int32, device="cuda")
+    dev_table, dev_h = torch.from_numpy(table).cuda(), torch.from_numpy(heights).cuda()
+    assert ds.wlib().cmsd_gen_decode_rows(dev_table.data_ptr(), dev_h.data_ptr(), 0, B, K, K, V, None, 4,
+                                          buf[0].data_ptr() + 4 * skip[0], buf[1].data_ptr() + 4 * skip[1],
+                                          tok.data_ptr(), cmsd._stream()) == 0
+    d, t = [x.cpu().numpy() for x in buf]
+    for x, k in ((d, skip[0]), (t, skip[1])):
+        assert (x[:k] == 7.0).all() and (x[B * K * V + k:] == 7.0).all()
+    for b in range(B):
+        hd, ht, htok = W.decode_iteration_host(table, heights, 0, b, K, K, V, 4)
+        for i in range(K):
+            r = (b * K + i) * V
+            assert np.array_equal(d[skip[0] + r:skip[0] + r + V], hd[i]) and np.array_equal(t[skip[1] + r:skip[1] + r + V], ht[i])
+            assert int(tok[b, i]) == htok[i]
+
+
+@pytest.mark.gpu
 def test_generator_takes_more_slots_than_one_grid_holds(mods):
     """2^29 + 5 sequences of which three have a row: four CTAs a slot are more
     than a grid of 2^31 - 1."""
