@@ -42,6 +42,10 @@ __device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
 }
 
 // One cluster per (b, i) slot of the [B][Kt] verifier layout, from slot0 on.
+// SINGLE: rows that no vector store fits.  Eight stores of a thread's own eight
+// logits touch a sector each (B=32 K=16 V=31999 51.9 us); a warp's 256 go through
+// shared memory first and leave as whole lines (16.4 us).
+template <bool SINGLE>
 __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_rows_kernel(const float* __restrict__ table,
                                                             const float* __restrict__ heights_it,
                                                             uint32_t it, int slot0, int B, int K_max, int Kt, int V,
@@ -86,10 +90,11 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
   // rows start on 32-byte boundaries when V is a multiple of 8 and the tensors
   // do: each thread then writes its 8 logits in one store; on 16-byte ones when
   // V is a multiple of 4 and the tensors do: two stores
-  const uintptr_t at = ((uintptr_t)draft) | ((uintptr_t)target);
-  const bool vec = (V & 3) == 0 && (at & 15) == 0;
-  const bool vec8 = (V & 7) == 0 && (at & 31) == 0;
-  for (int g = part * kThreads + threadIdx.x; g < ngrp; g += kParts * kThreads) {
+  const bool vec8 = (V & 7) == 0 && ((((uintptr_t)draft) | ((uintptr_t)target)) & 31) == 0;
+  __shared__ __align__(16) float s_out[SINGLE ? kThreads / 32 : 1][SINGLE ? 256 : 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // (SINGLE: whole warps, a lane past the last group makes one that is not written)
+  for (int g = part * kThreads + threadIdx.x; (SINGLE ? g - lane : g) < ngrp; g += kParts * kThreads) {
     const cmsd::U4 wd = cmsd::philox4x32_10(cmsd::U4{(uint32_t)g, (uint32_t)row, it, kGenDNoise}, k0, k1);
     const cmsd::U4 wt = cmsd::philox4x32_10(cmsd::U4{(uint32_t)g, (uint32_t)row, it, kGenTNoise}, k0, k1);
     const uint32_t dw[4] = {wd.x, wd.y, wd.z, wd.w}, tw[4] = {wt.x, wt.y, wt.z, wt.w};
@@ -106,12 +111,26 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
     int mj = 0;
 #pragma unroll
     for (int j = 7; j >= 0; --j)
-      if (8 * g + j < V && zs[j] >= m) { m = zs[j]; mj = j; }
+      if (8u * (uint32_t)g + j < (uint32_t)V && zs[j] >= m) { m = zs[j]; mj = j; }
     if (m > best) { best = m; bidx = 8 * g + mj; }
-    if (vec8) {
+    if (SINGLE) {
+      auto put = [&](float* row_at, const float (&x)[8]) {
+        float4* out = reinterpret_cast<float4*>(s_out[warp] + 8 * lane);
+        __syncwarp();
+        out[0] = make_float4(x[0], x[1], x[2], x[3]);
+        out[1] = make_float4(x[4], x[5], x[6], x[7]);
+        __syncwarp();
+        const uint32_t v0 = 8u * (uint32_t)(g - lane) + (uint32_t)lane;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (v0 + 32u * j < (uint32_t)V) row_at[v0 + 32u * j] = s_out[warp][lane + 32 * j];
+      };
+      if (has_draft) put(dz, zs);
+      put(tz, ts);
+    } else if (vec8) {
       if (has_draft) store8(dz + 8 * g, zs);
       store8(tz + 8 * g, ts);
-    } else if (vec && 8 * g + 8 <= V) {
+    } else if (8 * g + 8 <= V) {
       float4* d4 = reinterpret_cast<float4*>(dz + 8 * g);
       float4* t4 = reinterpret_cast<float4*>(tz + 8 * g);
       if (has_draft) {
@@ -142,7 +161,6 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kParts, 1, 1) gen_r
   __shared__ int si[kThreads / 32];
   __shared__ float pb[kParts];               // part 0: each part's maximum
   __shared__ int pi[kParts];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) { sb[warp] = best; si[warp] = bidx; }
   __syncthreads();
   cg::cluster_group cl = cg::this_cluster();
@@ -174,6 +192,7 @@ extern "C" int cmsd_gen_decode_rows(const float* table, const float* heights_it,
   const int64_t slots = (int64_t)B * Kt;        // (as many launches as a grid of 2^31 - 1 CTAs needs: one)
   if (slots > 0x7FFFFFFFll) return -1;
   constexpr int kMostSlots = 0x7FFFFFFF / kParts;
+  const bool single = (V & 3) != 0 || ((((uintptr_t)draft) | ((uintptr_t)target)) & 15) != 0;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
   cfg.stream = (cudaStream_t)stream;
@@ -185,8 +204,9 @@ extern "C" int cmsd_gen_decode_rows(const float* table, const float* heights_it,
   for (int64_t s0 = 0; s0 < slots; s0 += kMostSlots) {
     const int64_t n = slots - s0 < kMostSlots ? slots - s0 : kMostSlots;
     cfg.gridDim = dim3((unsigned)(n * kParts));
-    if (cudaLaunchKernelEx(&cfg, gen_rows_kernel, table, heights_it, it, (int)s0, B, K_max, Kt, V, k_row,
-                           cmsd::seed_lo(seed), cmsd::seed_hi(seed), draft, target, tokens) != cudaSuccess)
+    if (cudaLaunchKernelEx(&cfg, single ? gen_rows_kernel<true> : gen_rows_kernel<false>, table, heights_it, it, (int)s0,
+                           B, K_max, Kt, V, k_row, cmsd::seed_lo(seed), cmsd::seed_hi(seed), draft, target,
+                           tokens) != cudaSuccess)
       return -3;
   }
   return 0;
