@@ -23,8 +23,9 @@
 //
 // us a call, the streaming kernel and its draw against one launch, sampled
 // bf16: B=4 K=4 V=32000 16.1, 7.7; B=32 K=8 V=128256 35.7, 30.2; B=64 54.2,
-// 52.8, where 256 CTAs stream 262.7 MB at 0.87 of the copy rate, bound by
-// issue slots, and 8 us of rows and draw follow.
+// 52.8, where 256 CTAs stream 262.7 MB at 0.87 of the copy rate (at two CTAs an
+// SM 48 of the 152 hold one alone, whose loads in flight do not fill its share;
+// issue is active 46 %), and 8 us of rows and draw follow.
 #pragma once
 #include "cmsd_stream_impl.cuh"
 
