@@ -5,16 +5,16 @@
 // Work split.  The present rows (sequence b, drafted position i < k_row[b])
 // are laid end to end into one stream of rows * V logits per tensor, and the
 // launched warps (a persistent grid: one CTA per SM, of 512 threads, or 768 for
-// short rows) each take one contiguous slice of that stream: whole-warp pieces of one row when there are
-// at least as many warps as rows (and that keeps three quarters of them busy),
-// equal runs of 128-byte lines otherwise.  Each piece of a row inside a slice
-// is a "segment".
+// short rows) each take one contiguous slice of that stream: whole-warp pieces
+// of one row when there are at least as many warps as rows (and that keeps
+// three quarters of them busy), equal runs of 128-byte lines otherwise.  Each
+// piece of a row inside a slice is a "segment".
 //
 // Memory pipeline.  A lane's 16-byte vectors in a segment are those with index
 // lane + 32 t; it reads stream_unroll (four, or two with 768 threads) of each
-// tensor per stage with streaming loads (ld.global.nc, no L1 allocation) into registers, and issues the loads
-// of stage s + 1 before it reduces stage s, so one stage is always in flight
-// (pipe_run).
+// tensor per stage with streaming loads (ld.global.nc, no L1 allocation) into
+// registers, and issues the loads of stage s + 1 before it reduces stage s, so
+// one stage is always in flight (pipe_run).
 // The unaligned head and tail of a segment (under 16 bytes each) are read
 // element by element, before and after the vectors: a lane meets its entries
 // in index order, so the first of equal maxima is the lowest.
