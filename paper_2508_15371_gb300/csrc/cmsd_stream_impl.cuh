@@ -2103,9 +2103,9 @@ __global__ void __launch_bounds__(kDrawThreads, 4) draw_kernel(const StreamArgs 
 //
 // The same draw by a cluster of kCluCtas CTAs of 512 threads, the share of the
 // target row copied to shared memory (cp.async, all of it in flight at once)
-// while the share's uniforms are drawn: the shorter chain, where every
-// sequence's cluster can be resident (B=64 K=8 V=128256: 54.6 us a step
-// against 56.3 with draw_kernel).
+// while the share's uniforms are drawn: the shorter chain while few sequences
+// wait for a cluster (draw_plan in cmsd_api.cu; B=64 K=8 V=128256: 54.6 us a
+// step against 56.3 with draw_kernel).
 constexpr int kCluCtas = 4;                  // CTAs per row (one cluster)
 constexpr int kCluThreads = 512;
 constexpr int kCluWarps = kCluThreads / 32;
